@@ -211,7 +211,9 @@ int dugks_kernel_bytes_per_cell(const dugks_sim *sim, int k, double *bytes);
    2 = 32x12 on 384 threads, 3 = 32x8 on 352 threads with the face fluxes in
    their own shared memory (two blocks per SM).  Strips, one thread block of
    288 threads marching up 32 columns in blocks of 32x8 cells (two blocks per
-   SM): 4 = strips of 8 blocks, 5 = 16 blocks, 6 = 32 blocks.  Every shape
+   SM): 4 = strips of 8 blocks, 5 = 16 blocks, 6 = 32 blocks.  Where the
+   meshes give too few 32x8 tiles to occupy the device, shape 0 cuts each into
+   tiles of 16x8, 8x8 or (FP64) 8x4 or 4x8 cells.  Every shape
    computes the same scheme: on uniform periodic meshes the results agree bit
    for bit, elsewhere to rounding.  A new fused-step sim starts with shape 5
    when its meshes give at least 3 strips of 16 blocks per resident strip slot

@@ -31,6 +31,10 @@ struct EventPair {
     int count;   // kernel launches between the two events
 };
 
+// The shapes of the C ABI, then the smaller tiles that shape 0 is cut into on
+// meshes that leave the device idle (kernel_shape).
+constexpr int kNumKernelShapes = DUGKS_NUM_TILE_SHAPES + 4;
+
 }  // namespace
 
 struct dugks_sim {
@@ -60,7 +64,8 @@ struct dugks_sim {
     bool fused = true;            // one-launch step (k_step) or the four-kernel step
     bool use_graph = true;        // replay multi-step calls from a captured two-step graph
     bool use_uni = true;          // uniform periodic instances take the specialised fused step
-    int shape = 0;                // shape of the fused step (index into kShapes; see default_shape)
+    int shape = 0;                // shape of the fused step (index into kShapes; see choose_shapes)
+    int tile0 = 0;                // the tile that shape 0 runs on (see tile_for_sizes)
     int n_sm = 1;                 // multiprocessors of the device (sizes persistent grids)
     // device memory source, fixed at creation (dugks_set_allocator)
     dugks_alloc_fn alloc_fn = nullptr;
@@ -68,9 +73,9 @@ struct dugks_sim {
     void *alloc_ctx = nullptr;
     // fused-step tile tables per shape: the tiles of uniform periodic instances
     // first (n_uni_s of them), then the rest
-    int4 *d_tiles_s[DUGKS_NUM_TILE_SHAPES] = {};
-    int n_tiles_s[DUGKS_NUM_TILE_SHAPES] = {};
-    int n_uni_s[DUGKS_NUM_TILE_SHAPES] = {};
+    int4 *d_tiles_s[kNumKernelShapes] = {};
+    int n_tiles_s[kNumKernelShapes] = {};
+    int n_uni_s[kNumKernelShapes] = {};
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph2 = nullptr;   // k_step(A -> B), k_step(B -> A)
     int *d_status = nullptr;
@@ -107,13 +112,17 @@ struct ShapeDesc {
     int bx, by, nt, sep, nb;   // nb > 0: a strip of up to nb blocks per thread block (k_strip)
     const char *name;
 };
-const ShapeDesc kShapes[DUGKS_NUM_TILE_SHAPES] = {{32, 8, 256, 0, 0, "32x8"},
+const ShapeDesc kShapes[kNumKernelShapes] = {{32, 8, 256, 0, 0, "32x8"},
                                                   {32, 4, 128, 0, 0, "32x4/128"},
                                                   {32, 12, 384, 0, 0, "32x12"},
                                                   {32, 8, 352, 1, 0, "32x8/352 sep"},
                                                   {32, 8, 288, 0, 8, "32x8 strip8/288"},
                                                   {32, 8, 288, 0, 16, "32x8 strip16/288"},
-                                                  {32, 8, 288, 0, 32, "32x8 strip32/288"}};
+                                                  {32, 8, 288, 0, 32, "32x8 strip32/288"},
+                                                  {16, 8, 0, 0, 0, "16x8"},
+                                                  {8, 8, 0, 0, 0, "8x8"},
+                                                  {8, 4, 0, 0, 0, "8x4"},
+                                                  {4, 8, 0, 0, 0, "4x8"}};
 
 const char *kNames[K_COUNT] = {"k_mu", "k_macro", "k_cell", "k_face", "k_init", "k_reduce", "k_step", "k_diag_f"};
 
@@ -337,15 +346,54 @@ int shape_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm
     return 0;
 }
 
-int default_shape(const dugks_sim *s)
+// The tile that shape 0 runs on: its 32x8 cells, or the smaller tile that the
+// meshes make faster.  A tile's thread block takes `lat` when it has an SM for
+// itself and adds `sat` to an SM that is busy with others, so n tiles take
+// about lat + (ceil(n / n_sm) - 1) sat; the least estimate wins, the larger
+// tile on a tie.  The times (us, GB300) are those of a step that fits one wave
+// (64x64 drop) and of a 512x512 drop per tile of an SM:
+//            FP64 lat / sat     FP32 lat / sat
+//   32x8       123 / 120          8.2 / 4.8
+//   16x8        77 / 65.5         7.2 / 2.75
+//   8x8         52 / 39.5         6.15 / 1.98
+//   8x4, 4x8    36 / 23           as 8x8 in FP32: left out
+// Steps measured with the 32x8 tile and with the choice: FP64 64x64 drop 123 and
+// 36 us (8x4), 128x128 drop 124 and 77 (16x8), 4x256 channel 129 and 47 (4x8:
+// its four columns fill a tile, where 32 columns hold each cell eight times);
+// FP32 64x64 drop 8.2 and 6.2 (8x8), 4x256 channel 10.3 and 7.2 (8x8), 256x256
+// drop 12.3 with the 32x8 tile, which the rule keeps (16x8: 13.4).
+int tile_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm)
 {
-    if (!s->fused) return 0;
+    struct Cost { int k; float lat, sat; };
+    static const Cost f64[] = {{0, 123.f, 120.f}, {7, 77.f, 65.5f}, {8, 52.f, 39.5f}, {9, 36.f, 23.f}, {10, 36.f, 23.f}};
+    static const Cost f32[] = {{0, 8.2f, 4.8f}, {7, 7.2f, 2.75f}, {8, 6.15f, 1.98f}};
+    const bool d = precision == DUGKS_FP64;
+    const Cost *c = d ? f64 : f32;
+    int best = 0;
+    float best_t = 0.f;
+    for (int i = 0; i < (d ? 5 : 3); i++) {
+        const ShapeDesc &S = kShapes[c[i].k];
+        long long tiles = 0;
+        for (int k = 0; k < n; k++) tiles += (long long)((nx[k] + S.bx - 1) / S.bx) * ((ny[k] + S.by - 1) / S.by);
+        const float t = c[i].lat + (float)((tiles + n_sm - 1) / n_sm - 1) * c[i].sat;
+        if (i == 0 || t < best_t) { best = c[i].k; best_t = t; }
+    }
+    return best;
+}
+
+// index into kShapes of the kernel that runs the sim's shape
+int kernel_shape(const dugks_sim *s) { return s->shape == 0 ? s->tile0 : s->shape; }
+
+void choose_shapes(dugks_sim *s)
+{
+    if (!s->fused) return;
     std::vector<int> nx, ny;
     for (const InstDev &I : s->h_inst) {
         nx.push_back(I.nx);
         ny.push_back(I.ny);
     }
-    return shape_for_sizes(nx.data(), ny.data(), s->n_inst, s->prec, s->n_sm);
+    s->shape = shape_for_sizes(nx.data(), ny.data(), s->n_inst, s->prec, s->n_sm);
+    s->tile0 = tile_for_sizes(nx.data(), ny.data(), s->n_inst, s->prec, s->n_sm);
 }
 
 // fused-step tile table of shape k: the uniform periodic instances' tiles first
@@ -380,9 +428,23 @@ int ensure_tiles(dugks_sim *s, int k)
 template <typename T>
 int prepare_fused(dugks_sim *s)
 {
-    int rc = ensure_tiles(s, s->shape);
+    const int k = kernel_shape(s);
+    int rc = ensure_tiles(s, k);
     if (rc) return rc;
-    switch (s->shape) {
+    if constexpr (sizeof(T) == 8) {
+        switch (k) {
+        case 7: return prepare_shape<T, 16, 8, 128, false>();
+        case 8: return prepare_shape<T, 8, 8, 128, false>();
+        case 9: return prepare_shape<T, 8, 4, 128, false>();
+        case 10: return prepare_shape<T, 4, 8, 128, false>();
+        }
+    } else {
+        switch (k) {
+        case 7: return prepare_shape<T, 16, 8, 256, false>();
+        case 8: return prepare_shape<T, 8, 8, 256, false>();
+        }
+    }
+    switch (k) {
     case 1: return prepare_shape<T, 32, 4, 128, false>();
     case 2: return prepare_shape<T, 32, 12, 384, false>();
     case 3: return prepare_shape<T, 32, 8, 352, true>();
@@ -410,7 +472,7 @@ StepIO<T> step_io(dugks_sim *s)
 // kernels one fused step launches: one per class of instance present
 int fused_launches(const dugks_sim *s)
 {
-    const int k = s->shape;
+    const int k = kernel_shape(s);
     return (s->n_uni_s[k] > 0) + (s->n_tiles_s[k] > s->n_uni_s[k]);
 }
 
@@ -439,13 +501,27 @@ void enqueue_shape(dugks_sim *s, int k, const StepIO<T> &io, cudaStream_t st)
 template <typename T>
 void enqueue_fused(dugks_sim *s, const StepIO<T> &io, cudaStream_t st)
 {
-    switch (s->shape) {
+    const int k = kernel_shape(s);
+    if constexpr (sizeof(T) == 8) {
+        switch (k) {
+        case 7: enqueue_shape<T, 16, 8, 128, false>(s, k, io, st); return;
+        case 8: enqueue_shape<T, 8, 8, 128, false>(s, k, io, st); return;
+        case 9: enqueue_shape<T, 8, 4, 128, false>(s, k, io, st); return;
+        case 10: enqueue_shape<T, 4, 8, 128, false>(s, k, io, st); return;
+        }
+    } else {
+        switch (k) {
+        case 7: enqueue_shape<T, 16, 8, 256, false>(s, k, io, st); return;
+        case 8: enqueue_shape<T, 8, 8, 256, false>(s, k, io, st); return;
+        }
+    }
+    switch (k) {
     case 1: enqueue_shape<T, 32, 4, 128, false>(s, 1, io, st); break;
     case 2: enqueue_shape<T, 32, 12, 384, false>(s, 2, io, st); break;
     case 3: enqueue_shape<T, 32, 8, 352, true>(s, 3, io, st); break;
     case 4:
     case 5:
-    case 6: enqueue_strip<T, 32, 8, 288>(s, s->shape, io, st); break;
+    case 6: enqueue_strip<T, 32, 8, 288>(s, k, io, st); break;
     default: enqueue_shape<T, 32, 8, 256, false>(s, 0, io, st); break;
     }
 }
@@ -713,7 +789,7 @@ void free_sim(dugks_sim *s)
     if (!s) return;
     dfree(s, s->d_inst);
     dfree(s, s->d_tiles);
-    for (int k = 0; k < DUGKS_NUM_TILE_SHAPES; k++) dfree(s, s->d_tiles_s[k]);
+    for (int4 *t : s->d_tiles_s) dfree(s, t);
     dfree(s, s->d_strips8);
     dfree(s, s->d_strip_rng);
     dfree(s, s->d_geo);
@@ -1064,7 +1140,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
     s->N = cell;
     s->n_dense = dense;
     s->n_tiles = (int)tiles.size();
-    s->shape = default_shape(s);
+    choose_shapes(s);
     const size_t esz = s->prec == DUGKS_FP64 ? sizeof(double) : sizeof(float);
     // the bar-plus planes exist only for the four-kernel step
     const size_t plane_elems = (size_t)((s->fused ? 2 : 4) * Q + kNumScalarPlanes) * (size_t)s->N;
