@@ -353,19 +353,19 @@ int shape_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm
 // tile on a tie.  The times (us, GB300) are those of a step that fits one wave
 // (64x64 drop) and of a 512x512 drop per tile of an SM:
 //            FP64 lat / sat     FP32 lat / sat
-//   32x8       123 / 120          8.2 / 4.8
-//   16x8        77 / 65.5         7.2 / 2.75
-//   8x8         52 / 39.5         6.15 / 1.98
-//   8x4, 4x8    36 / 23           as 8x8 in FP32: left out
-// Steps measured with the 32x8 tile and with the choice: FP64 64x64 drop 123 and
-// 36 us (8x4), 128x128 drop 124 and 77 (16x8), 4x256 channel 129 and 47 (4x8:
+//   32x8        82 / 80           8.2 / 4.8
+//   16x8        52 / 40           7.2 / 2.75
+//   8x8         36 / 24           6.15 / 1.98
+//   8x4, 4x8  22.5 / 15           as 8x8 in FP32: left out
+// Steps measured with the 32x8 tile and with the choice: FP64 64x64 drop 82 and
+// 22.5 us (8x4), 128x128 drop 82 and 52 (16x8), 4x256 channel 86 and 26.7 (4x8:
 // its four columns fill a tile, where 32 columns hold each cell eight times);
 // FP32 64x64 drop 8.2 and 6.2 (8x8), 4x256 channel 10.3 and 7.2 (8x8), 256x256
 // drop 12.3 with the 32x8 tile, which the rule keeps (16x8: 13.4).
 int tile_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm)
 {
     struct Cost { int k; float lat, sat; };
-    static const Cost f64[] = {{0, 123.f, 120.f}, {7, 77.f, 65.5f}, {8, 52.f, 39.5f}, {9, 36.f, 23.f}, {10, 36.f, 23.f}};
+    static const Cost f64[] = {{0, 82.f, 80.f}, {7, 52.f, 40.f}, {8, 36.f, 24.f}, {9, 22.5f, 15.f}, {10, 22.5f, 15.f}};
     static const Cost f32[] = {{0, 8.2f, 4.8f}, {7, 7.2f, 2.75f}, {8, 6.15f, 1.98f}};
     const bool d = precision == DUGKS_FP64;
     const Cost *c = d ? f64 : f32;
@@ -1131,6 +1131,25 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         };
         fill(I.pd);
         fill(I.pf);
+        I.b4 = 4.0 * I.beta;
+        I.cd64 = I.drho / 3.0;
+        I.cgl64 = I.gamma * I.lambda / 3.0;
+        I.rh64 = 1.0 / I.h;
+        const double K = I.muA * I.muB * (I.phiA - I.phiB), tg = I.tau_g;
+        // half the time tau over which the force of the point's velocity acts,
+        // the weights b and c of Eqs. (relations1), (original-function) over w
+        auto point = [&](PtC64 &C, double tau, double nb, double nc, double ga, double gb, double gc) {
+            C.kf = tau / 3.0;
+            C.kp1 = C.kf * I.drho;
+            C.kp2 = C.kf * I.gamma * I.lambda;
+            C.k6 = 6.0 * K;
+            C.nb = nb / 36.0; C.nc = nc / 36.0;
+            C.ga = ga; C.gb = gb / 36.0; C.gbe = C.gb * I.eta; C.gc = 3.0 * gc / 36.0;
+            C.gb36 = gb; C.gbe36 = gb * I.eta;
+        };
+        const double gcell = 2.0 * tg + I.dt, gface = 2.0 * tg + I.h;
+        point(I.cell64, 0.5 * I.dt, 3.0, 9.0 * K * I.h, (2.0 * tg - I.h) / gcell, 3.0 * I.h / gcell, 3.0 * tg * I.h / gcell);
+        point(I.face64, 0.5 * I.h, 1.0, 3.0 * K * I.h, 2.0 * tg / gface, I.h / gface, tg * I.h / gface);
         I.tile0 = (int)tiles.size();
         for (int ty = 0; ty < m.ny; ty += TY)
             for (int tx = 0; tx < m.nx; tx += TX) tiles.push_back(make_int4(k, tx, ty, 0));

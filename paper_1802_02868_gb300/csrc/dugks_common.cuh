@@ -143,6 +143,16 @@ __device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
 __device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
+// Constants of the FP64 step (dugks_fp64.cuh) at a cell (Eqs. u, P, relations1)
+// or at a face (Eqs. conservedVariable, original-function).  w = 1/36, the
+// diagonals' weight, is part of nb, nc, gb, gbe and gc.
+struct PtC64 {
+    double kf, kp1, kp2;      // c_s^2 tau, with drho, with gamma lambda; tau = dt/2 (cell), h/2 (face)
+    double k6, nb, nc;        // 6K and the numerators w b / X, w c of the f weights (see cell_weights, face_weights)
+    double ga, gb, gbe, gc;   // g weights: a; w b; w b eta; 3 w c
+    double gb36, gbe36;       // b, b eta
+};
+
 // Per-instance constants.
 struct InstDev {
     int nx, ny, nxp, bcx, bcy;
@@ -161,7 +171,16 @@ struct InstDev {
     PhiC cA, cB, cM;
     ParT<double> pd;
     ParT<float> pf;
+    // FP64 step: 4 beta, c_s^2 drho, c_s^2 gamma lambda, 1 / h
+    double b4, cd64, cgl64, rh64;
+    PtC64 cell64, face64;
 };
+
+// Flux-carrying directions of x faces (cx != 0) and of y faces (cy != 0).
+__host__ __device__ constexpr int xset(int k) { return k == 0 ? 1 : k == 1 ? 3 : k + 3; }   // 1,3,5,6,7,8
+__host__ __device__ constexpr int yset(int k) { return k == 0 ? 2 : k == 1 ? 4 : k + 3; }   // 2,4,5,6,7,8
+template <int A>
+__host__ __device__ constexpr int fset(int k) { return A == 0 ? xset(k) : yset(k); }
 
 template <typename T>
 __device__ __forceinline__ const ParT<T> &par(const InstDev &I);

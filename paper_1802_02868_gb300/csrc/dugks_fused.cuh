@@ -16,6 +16,7 @@
 // of being written to and re-read from HBM; the state is double-buffered
 // because tiles read the old state of their ring.
 #pragma once
+#include "dugks_fp64.cuh"
 #include "dugks_kernels.cuh"
 
 namespace dugks {
@@ -45,13 +46,17 @@ struct FusedLayout {
     // y faces one row of BX per warp.  Either way no warp reads two R1
     // entries of one shared-memory bank.
     static constexpr int XP = W1, NXI = XP * BY, Y0 = (NXI + 31) / 32 * 32, NFT = Y0 + NFY;
-    static constexpr int NR1 = 7 + 18;                       // R1 planes
+    // R1 planes: grad mu, lap mu, grad phi, grad p and the bar-plus pairs.  In
+    // FP64 the p phase leaves grad mu, lap mu, grad phi and u on R2 instead.
+    static constexpr bool F64 = sizeof(T) == 8;
+    static constexpr int NR1 = F64 ? 2 + 18 : 7 + 18, NR2 = F64 ? 1 + 7 : 1;
+    static constexpr int NGA = F64 ? 12 : 11;                // geometry coefficients
     static constexpr size_t al(size_t v) { return (v + 15) / 16 * 16; }
-    static constexpr size_t o_geo = 0;                       // 11 T arrays + 2 int arrays of NG
-    static constexpr size_t o_phi = al(o_geo + (sizeof(T) * 11 + sizeof(int) * 2) * NG);
+    static constexpr size_t o_geo = 0;                       // NGA T arrays + 2 int arrays of NG
+    static constexpr size_t o_phi = al(o_geo + (sizeof(T) * NGA + sizeof(int) * 2) * NG);
     static constexpr size_t o_mu = al(o_phi + sizeof(phi_t<T>) * A4);
     static constexpr size_t o_p = al(o_mu + sizeof(T) * A3);
-    static constexpr size_t o_r1 = al(o_p + sizeof(T) * A2);
+    static constexpr size_t o_r1 = al(o_p + sizeof(T) * NR2 * A2);
     // tilde f on R2 and tilde g on R1 (phases 1-4); the face fluxes (phase
     // 5-6) reuse the same bytes once the bar-plus phase is done, unless SEP
     // gives them their own (then the update reads its tilde values here)
@@ -75,12 +80,6 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Flux-carrying directions of x faces (cx != 0) and of y faces (cy != 0).
-__host__ __device__ constexpr int xset(int k) { return k == 0 ? 1 : k == 1 ? 3 : k + 3; }   // 1,3,5,6,7,8
-__host__ __device__ constexpr int yset(int k) { return k == 0 ? 2 : k == 1 ? 4 : k + 3; }   // 2,4,5,6,7,8
-template <int A>
-__host__ __device__ constexpr int fset(int k) { return A == 0 ? xset(k) : yset(k); }
-
 // Geometry of one region position on one axis, read from the SoA arrays.
 template <typename T>
 struct G1 {
@@ -97,29 +96,40 @@ struct G1 {
 template <typename T, int BX, int BY, bool UNI = false, bool SEP = false>
 struct Tile {
     using L = FusedLayout<T, BX, BY, SEP>;
-    T *ga;          // [11][NG] geometry coefficients, positions x -4..BX+3 then y -4..BY+3
+    T *ga;          // [NGA][NG] geometry coefficients, positions x -4..BX+3 then y -4..BY+3
     int *gg, *gf;   // [NG] global index (-1 outside), flags: 1 om=-1, 2 op=+1, 4 lo wall, 8 hi wall
     phi_t<T> *phi;  // R4
     pair_t<T> *flux;  // [6][NFT] (f, g) flux pairs by face item; unless SEP, aliases sf and sg (dead once phase 4 ends)
     T *mu;          // R3
     T *p;           // R2
-    T *gmx, *gmy, *lmu, *gfx, *gfy, *gpx, *gpy;  // R1
+    T *gmx, *gmy, *lmu, *gfx, *gfy;  // R1 (FP64: R2)
+    T *ux, *uy;     // R2, FP64 only
+    T *gpx, *gpy;   // R1
     pair_t<T> *bp;  // [9][A1]: (f, g) bar-plus pairs
     T *sf;          // tilde f on R2 [Q][A2]
     T *sg;          // tilde g on R1 [Q][A1]
     __device__ Tile(unsigned char *sm)
     {
         ga = (T *)(sm + L::o_geo);
-        gg = (int *)(ga + 11 * L::NG);
+        gg = (int *)(ga + L::NGA * L::NG);
         gf = gg + L::NG;
         phi = (phi_t<T> *)(sm + L::o_phi);
         flux = (pair_t<T> *)(sm + L::o_flux);
         mu = (T *)(sm + L::o_mu);
         p = (T *)(sm + L::o_p);
         T *r1 = (T *)(sm + L::o_r1);
-        gmx = r1; gmy = r1 + L::A1; lmu = r1 + 2 * L::A1; gfx = r1 + 3 * L::A1; gfy = r1 + 4 * L::A1;
-        gpx = r1 + 5 * L::A1; gpy = r1 + 6 * L::A1;
-        bp = (pair_t<T> *)(r1 + 7 * L::A1);
+        if constexpr (L::F64) {
+            T *r2 = p + L::A2;
+            gmx = r2; gmy = r2 + L::A2; lmu = r2 + 2 * L::A2; gfx = r2 + 3 * L::A2; gfy = r2 + 4 * L::A2;
+            ux = r2 + 5 * L::A2; uy = r2 + 6 * L::A2;
+            gpx = r1; gpy = r1 + L::A1;
+            bp = (pair_t<T> *)(r1 + 2 * L::A1);
+        } else {
+            gmx = r1; gmy = r1 + L::A1; lmu = r1 + 2 * L::A1; gfx = r1 + 3 * L::A1; gfy = r1 + 4 * L::A1;
+            gpx = r1 + 5 * L::A1; gpy = r1 + 6 * L::A1;
+            ux = uy = nullptr;
+            bp = (pair_t<T> *)(r1 + 7 * L::A1);
+        }
         sf = (T *)(sm + L::o_f);
         sg = (T *)(sm + L::o_g);
     }
@@ -169,6 +179,21 @@ struct Tile {
         }
     }
 };
+
+// The coefficients of geometry record R that the tile keeps; the FP64 step's
+// carry h in the distribution derivatives and the inverse distance, and dt over
+// the width.
+template <typename T>
+__device__ __forceinline__ void geo_coefficients(const AxisRecT<T> &R, const ParT<T> &Pr, T *v)
+{
+    v[0] = R.c1m; v[1] = R.c1p; v[2] = R.c2m; v[3] = R.c2p;
+    v[4] = R.e1m; v[5] = R.e10; v[6] = R.e1p;
+    v[7] = R.wL; v[8] = R.wR; v[9] = R.invd; v[10] = R.d;
+    if constexpr (sizeof(T) == 8) {
+        v[4] *= Pr.h; v[5] *= Pr.h; v[6] *= Pr.h; v[9] *= Pr.h;
+        v[11] = Pr.dt * fp64::rcp(R.d);
+    }
+}
 
 // Face macroscopic variables from the nine bar distributions of each kind at
 // t+h (Eq. conservedVariable with h, bar for tilde), then the originals of
@@ -430,26 +455,31 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         const int pos = isx ? r - 4 : r - L::W4 - 4;
         const int g = S.gg[r];
         if (UNI && pos != 0) continue;   // every position carries the record of position 0
-        T v[11];
+        T v[L::NGA];
         int fl = 0;
         if (g >= 0) {
             const AxisRecT<T> &R = geo[(isx ? I.gx_off : I.gy_off) + g];
-            v[0] = R.c1m; v[1] = R.c1p; v[2] = R.c2m; v[3] = R.c2p;
-            v[4] = R.e1m; v[5] = R.e10; v[6] = R.e1p;
-            v[7] = R.wL; v[8] = R.wR; v[9] = R.invd; v[10] = R.d;
+            geo_coefficients<T>(R, Pr, v);
             fl = (R.km == g ? 0 : 1) | (R.kp == g ? 0 : 2) | (R.lo_wall ? 4 : 0) | (R.hi_wall ? 8 : 0);
         } else {
 #pragma unroll
-            for (int k = 0; k < 11; k++) v[k] = T(0);
+            for (int k = 0; k < L::NGA; k++) v[k] = T(0);
         }
 #pragma unroll
-        for (int k = 0; k < 11; k++) S.ga[k * L::NG + r] = v[k];
+        for (int k = 0; k < L::NGA; k++) S.ga[k * L::NG + r] = v[k];
         S.gf[r] = fl;
     }
     cp_wait<1>();   // phi has landed
     __syncthreads();
 
     // ---- phase 2: mu on R3 (Eq. chemicalpotential), differences of the stored phi
+    if constexpr (L::F64) {
+        for (int r = tid; r < L::A3; r += NT) {
+            int x, y;
+            TL::ring_item(r, L::H3, 3, -3, x, y);
+            fp64::mu_point(I, S, x, y);
+        }
+    } else
     for (int r = tid; r < L::A3; r += NT) {
         int x, y;
         TL::ring_item(r, L::H3, 3, -3, x, y);
@@ -473,6 +503,16 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     const T hdt = T(0.5) * Pr.dt;
     const T cs2 = Cst<T>::cs2;
     // ---- phase 3: p on R2 (Eqs. u, P); needs grad mu, lap mu, grad phi and f~
+    if constexpr (L::F64) {
+        for (int r = tid; r < L::A2; r += NT) {
+            int x, y;
+            TL::ring_item(r, L::H2, 2, -2, x, y);
+            T f[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q++) f[q] = S.sf[q * L::A2 + TL::i2(x, y)];
+            fp64::p_point(I, S, x, y, f);
+        }
+    } else
     for (int r = tid; r < L::A2; r += NT) {
         int x, y;
         TL::ring_item(r, L::H2, 2, -2, x, y);
@@ -514,6 +554,31 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     // ---- phase 4: grad p, u and bar-plus of both distributions on R1 (Eq. relations1)
     const T dt = Pr.dt;
     const T ag = Pr.gca, bg = Pr.gcb, cg = Pr.gcc;
+    if constexpr (L::F64) {
+        // f and g of a cell on two threads where the block has them to spare
+        // (g from a warp boundary on): half the instructions on the longest path
+        constexpr int G0 = (L::A1 + 31) / 32 * 32;
+        constexpr bool SPLIT = G0 + L::A1 <= NT;
+        for (int r = tid; r < (SPLIT ? G0 + L::A1 : L::A1); r += NT) {
+            if (SPLIT && r >= L::A1 && r < G0) continue;
+            const bool second = SPLIT && r >= G0;
+            int x, y;
+            TL::ring_item(second ? r - G0 : r, L::H1, 1, -1, x, y);
+            const int k1 = TL::i1(x, y), k2 = TL::i2(x, y);
+            T f[Q], g[Q];
+            if (!second) {
+#pragma unroll
+                for (int q = 0; q < Q; q++) f[q] = S.sf[q * L::A2 + k2];
+            }
+            if (!SPLIT || second) {
+#pragma unroll
+                for (int q = 0; q < Q; q++) g[q] = S.sg[q * L::A1 + k1];
+            }
+            if (!SPLIT) fp64::bar_plus_point<3>(I, S, x, y, f, g);
+            else if (second) fp64::bar_plus_point<2>(I, S, x, y, f, g);
+            else fp64::bar_plus_point<1>(I, S, x, y, f, g);
+        }
+    } else
     for (int r = tid; r < L::A1; r += NT) {
         int x, y;
         TL::ring_item(r, L::H1, 1, -1, x, y);
@@ -593,11 +658,13 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         if (k < L::NXI) {
             const int xa = k % L::XP - 1;
             if (xa >= BX) continue;                       // the idle item of an x-face row
-            tile_face<T, 0, UNI>(I, S, xa, k / L::XP, F2o);
+            if constexpr (L::F64) fp64::face<0, UNI>(I, S, xa, k / L::XP, F2o);
+            else tile_face<T, 0, UNI>(I, S, xa, k / L::XP, F2o);
         } else if (k < L::Y0) {
             continue;
         } else {
-            tile_face<T, 1, UNI>(I, S, (k - L::Y0) % BX, (k - L::Y0) / BX - 1, F2o);
+            if constexpr (L::F64) fp64::face<1, UNI>(I, S, (k - L::Y0) % BX, (k - L::Y0) / BX - 1, F2o);
+            else tile_face<T, 1, UNI>(I, S, (k - L::Y0) % BX, (k - L::Y0) / BX - 1, F2o);
         }
 #pragma unroll
         for (int m = 0; m < 6; m++) S.flux[m * L::NFT + k] = F2o[m];
@@ -605,6 +672,25 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     __syncthreads();
 
     // ---- phase 6: update of the tile cell (Eqs. relations2, updatef)
+    if constexpr (L::F64) {
+        // f and g of a cell on two threads where the block has them
+        constexpr int NC = BX * BY;
+        constexpr bool SPLIT = 2 * NC <= NT && NC % 32 == 0;
+        const int cid = SPLIT ? tid % NC : tid, ux = cid % BX, uy = cid / BX;
+        if (tid >= (SPLIT ? 2 * NC : NC) || i0 + ux >= I.nx || j0 + uy >= I.ny) return;
+        const long long cc = cell(i0 + ux, j0 + uy);
+        const int kw = uy * L::XP + ux, ks = L::Y0 + uy * BX + ux;
+        auto e = [&](int m) { return S.flux[m * L::NFT + kw + 1]; };
+        auto w = [&](int m) { return S.flux[m * L::NFT + kw]; };
+        auto n = [&](int m) { return S.flux[m * L::NFT + ks + BX]; };
+        auto so = [&](int m) { return S.flux[m * L::NFT + ks]; };
+        bool ok;
+        if (!SPLIT) ok = fp64::update_cell<3>(io, S, ux, uy, cc, e, w, n, so);
+        else if (tid < NC) ok = fp64::update_cell<1>(io, S, ux, uy, cc, e, w, n, so);
+        else ok = fp64::update_cell<2>(io, S, ux, uy, cc, e, w, n, so);
+        if (!ok) atomicOr(io.status + t.x, ST_NONFINITE);
+        return;
+    }
     if (!own) return;
     // J of both kinds at once: east minus west for the x set, north minus south for the y set
     pair_t<T> J[Q];
@@ -632,36 +718,24 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         nw[q] = pfma(pr(T(4.0 / 3.0)), S.bp[q * L::A1 + r1], pfma(pr(T(-1.0 / 3.0)), old, pmul(pr(-dtv), J[q])));
     }
     bool finite = true;
-    if constexpr (sizeof(T) == sizeof(double)) {
-        T phi = 0;
+    // sum_i g~+_i = phi exactly, so phi advances by the flux balance alone
+    // (kept as a float pair); the rest distribution g~_0 is rebuilt from it
+    T jsum = 0, gsum = 0;
 #pragma unroll
-        for (int q = 0; q < Q; q++) {
-            io.f_out[q * N + c] = nw[q].x;
+    for (int q = 0; q < Q; q++) {
+        io.f_out[q * N + c] = nw[q].x;
+        finite = finite && isfinite(nw[q].x);
+        jsum += J[q].y;
+        if (q > 0) {
             io.g_out[q * N + c] = nw[q].y;
-            phi += nw[q].y;
-            finite = finite && isfinite(nw[q].x) && isfinite(nw[q].y);
+            gsum += nw[q].y;
+            finite = finite && isfinite(nw[q].y);
         }
-        io.phi_out[c] = phi;
-    } else {
-        // sum_i g~+_i = phi exactly, so phi advances by the flux balance alone
-        // (kept as a float pair); the rest distribution g~_0 is rebuilt from it
-        T jsum = 0, gsum = 0;
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            io.f_out[q * N + c] = nw[q].x;
-            finite = finite && isfinite(nw[q].x);
-            jsum += J[q].y;
-            if (q > 0) {
-                io.g_out[q * N + c] = nw[q].y;
-                gsum += nw[q].y;
-                finite = finite && isfinite(nw[q].y);
-            }
-        }
-        const phi_t<T> phi = phi_add(S.phi[TL::i4(x, y)], -(dtv * jsum));
-        io.phi_out[c] = phi;
-        io.g_out[c] = phi_subt(phi, gsum);
-        finite = finite && isfinite(phi_val(phi));
     }
+    const phi_t<T> phi = phi_add(S.phi[TL::i4(x, y)], -(dtv * jsum));
+    io.phi_out[c] = phi;
+    io.g_out[c] = phi_subt(phi, gsum);
+    finite = finite && isfinite(phi_val(phi));
     if (!finite) atomicOr(io.status + t.x, 1);
 }
 

@@ -123,20 +123,18 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
     auto set_geo = [&](int r, bool isx, int pos, int g) {
         S.gg[r] = g;
         if (UNI && pos != 0) return;
-        T v[11];
+        T v[L::NGA];
         int fl = 0;
         if (g >= 0) {
             const AxisRecT<T> &R = geo[(isx ? I.gx_off : I.gy_off) + g];
-            v[0] = R.c1m; v[1] = R.c1p; v[2] = R.c2m; v[3] = R.c2p;
-            v[4] = R.e1m; v[5] = R.e10; v[6] = R.e1p;
-            v[7] = R.wL; v[8] = R.wR; v[9] = R.invd; v[10] = R.d;
+            geo_coefficients<T>(R, Pr, v);
             fl = (R.km == g ? 0 : 1) | (R.kp == g ? 0 : 2) | (R.lo_wall ? 4 : 0) | (R.hi_wall ? 8 : 0);
         } else {
 #pragma unroll
-            for (int k = 0; k < 11; k++) v[k] = T(0);
+            for (int k = 0; k < L::NGA; k++) v[k] = T(0);
         }
 #pragma unroll
-        for (int k = 0; k < 11; k++) S.ga[k * L::NG + r] = v[k];
+        for (int k = 0; k < L::NGA; k++) S.ga[k * L::NG + r] = v[k];
         S.gf[r] = fl;
     };
 
@@ -266,6 +264,10 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
         for (int r = tid; r < (y1 - y0) * L::W3; r += NT) {
             int x, y;
             TL::ring_item(r, y1 - y0, 3, y0, x, y);
+            if constexpr (L::F64) {
+                fp64::mu_point(I, S, x, y);
+                continue;
+            }
             T mu = 0;
             if (S.ok(0, x) && S.ok(1, y)) {
                 const phi_t<T> p0 = S.phi[TL::i4(x, y)];
@@ -287,6 +289,14 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
         for (int r = tid; r < (y1 - y0) * L::W2; r += NT) {
             int x, y;
             TL::ring_item(r, y1 - y0, 2, y0, x, y);
+            if constexpr (L::F64) {
+                const T *fr = stf + (y - fr0) * SL::SP + (x + SL::SO);
+                T f[Q];
+#pragma unroll
+                for (int q = 0; q < Q; q++) f[q] = fr[q * SL::FROWS * SL::SP];
+                fp64::p_point(I, S, x, y, f);
+                continue;
+            }
             T vp = 0;
             if (S.ok(0, x) && S.ok(1, y)) {
                 const T m0 = S.mu[TL::i3(x, y)];
@@ -330,6 +340,17 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
         for (int r = tid; r < (y1 - y0) * L::W1; r += NT) {
             int x, y;
             TL::ring_item(r, y1 - y0, 1, y0, x, y);
+            if constexpr (L::F64) {
+                const T *fr = stf + (y - fr0) * SL::SP + (x + SL::SO), *gr = stg + (y - gr0) * SL::SP + (x + SL::SO);
+                T f[Q], g[Q];
+#pragma unroll
+                for (int q = 0; q < Q; q++) {
+                    f[q] = fr[q * SL::FROWS * SL::SP];
+                    g[q] = gr[q * SL::GROWS * SL::SP];
+                }
+                fp64::bar_plus_point<3>(I, S, x, y, f, g);
+                continue;
+            }
             const int k1 = TL::i1(x, y);
             if (!S.ok(0, x) || !S.ok(1, y)) {
                 S.gmx[k1] = 0; S.gmy[k1] = 0; S.lmu[k1] = 0; S.gfx[k1] = 0; S.gfy[k1] = 0; S.gpx[k1] = 0; S.gpy[k1] = 0;
@@ -410,7 +431,10 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
     constexpr int PHB = (int)(sizeof(phi_t<T>) * 8 * L::W4 / 16);
     constexpr int MUB = (int)(sizeof(T) * 6 * L::W3 / 16);
     constexpr int PB = (int)(sizeof(T) * 4 * L::W2 / 16);
-    constexpr int AB = (int)(sizeof(T) * 2 * L::W1 / 16);               // one aux plane
+    // one aux plane (on R1, its last grad p planes too; in FP64 seven on R2,
+    // then the two grad p planes on R1)
+    constexpr int AB = (int)(sizeof(T) * 2 * L::W1 / 16);
+    constexpr int N2 = L::F64 ? 7 : 0, N1 = L::F64 ? 2 : 7;
     constexpr int BB = (int)(sizeof(pair_t<T>) * 2 * L::W1 / 16);       // one bar-plus plane
     static_assert(sizeof(pair_t<T>) * BX % 16 == 0 && sizeof(phi_t<T>) * 8 * L::W4 % 16 == 0 &&
                       sizeof(T) * 6 * L::W3 % 16 == 0 && sizeof(T) * 4 * L::W2 % 16 == 0 &&
@@ -419,7 +443,7 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
                       sizeof(T) * BY * L::W1 % 16 == 0 && sizeof(pair_t<T>) * SL::NFT % 16 == 0 &&
                       sizeof(pair_t<T>) * (SL::Y0 + (BY - 1) * BX) % 16 == 0,
                   "16-byte ring rows");
-    constexpr int NPHI = PHB, NMU = NPHI + MUB, NP = NMU + PB, NAUX = NP + 7 * AB;
+    constexpr int NPHI = PHB, NMU = NPHI + MUB, NP = NMU + PB, NAUX = NP + N2 * PB + N1 * AB;
     constexpr int NALL = NAUX + Q * BB;
     auto shift_word = [&](int k) {
         float4 *d;
@@ -437,10 +461,15 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
         } else if (k < NP) {
             d = (float4 *)S.p + (k - NMU);
             src = (const float4 *)(S.p + BY * L::W2) + (k - NMU);
+        } else if (k < NP + N2 * PB) {
+            const int pl = (k - NP) / PB, w = (k - NP) % PB;
+            d = (float4 *)(S.gmx + pl * L::A2) + w;
+            src = (const float4 *)(S.gmx + pl * L::A2 + BY * L::W2) + w;
         } else if (k < NAUX) {
-            const int pl = (k - NP) / AB, w = (k - NP) % AB;
-            d = (float4 *)(S.gmx + pl * L::A1) + w;
-            src = (const float4 *)(S.gmx + pl * L::A1 + BY * L::W1) + w;
+            T *a = L::F64 ? S.gpx : S.gmx;
+            const int pl = (k - NP - N2 * PB) / AB, w = (k - NP - N2 * PB) % AB;
+            d = (float4 *)(a + pl * L::A1) + w;
+            src = (const float4 *)(a + pl * L::A1 + BY * L::W1) + w;
         } else {
             const int q = (k - NAUX) / BB, w = (k - NAUX) % BB;
             d = (float4 *)(S.bp + q * L::A1) + w;
@@ -474,9 +503,13 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
             if (k < SL::NXI) {
                 const int xa = k % SL::XP - 1;
                 if (xa >= BX) continue;                   // the idle item of an x-face row
-                tile_face<T, 0, UNI>(I, S, xa, k / SL::XP, F2o);
+                if constexpr (L::F64) fp64::face<0, UNI>(I, S, xa, k / SL::XP, F2o);
+                else tile_face<T, 0, UNI>(I, S, xa, k / SL::XP, F2o);
             } else if (k < SL::Y0) {
                 continue;
+            } else if constexpr (L::F64) {
+                const bool top = k < SL::NFT;
+                fp64::face<1, UNI>(I, S, top ? (k - SL::Y0) % BX : k - SL::NFT, top ? (k - SL::Y0) / BX : -1, F2o);
             } else if (k < SL::NFT) {
                 tile_face<T, 1, UNI>(I, S, (k - SL::Y0) % BX, (k - SL::Y0) / BX, F2o);
             } else {
@@ -494,7 +527,17 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
         __syncthreads();
         // ---- update of the block's cell (Eqs. relations2, updatef)
         const int gi = i0 + x, gj = j0 + b * BY + y;
-        if (tid < BX * BY && gi < I.nx && gj < I.ny) {
+        if constexpr (L::F64) {
+            if (tid < BX * BY && gi < I.nx && gj < I.ny) {
+                const int kw = y * SL::XP + x, kn = SL::Y0 + y * BX + x;
+                const pair_t<T> *kp = keep0 + (b & 1) * 6 * BX + x;
+                const bool ok = fp64::update_cell<3>(
+                    io, S, x, y, cell(gi, gj), [&](int m) { return flux[m * SL::NFT + kw + 1]; },
+                    [&](int m) { return flux[m * SL::NFT + kw]; }, [&](int m) { return flux[m * SL::NFT + kn]; },
+                    [&](int m) { return y == 0 ? kp[m * BX] : flux[m * SL::NFT + kn - BX]; });
+                if (!ok) atomicOr(io.status + t.x, ST_NONFINITE);
+            }
+        } else if (tid < BX * BY && gi < I.nx && gj < I.ny) {
             pair_t<T> J[Q];
 #pragma unroll
             for (int q = 0; q < Q; q++) J[q] = pr(T(0));
@@ -516,34 +559,22 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
                 nw[q] = pfma(pr(T(4.0 / 3.0)), S.bp[q * L::A1 + r1],
                              pfma(pr(T(-1.0 / 3.0)), pr(io.f_in[q * N + c], io.g_in[q * N + c]), pmul(pr(-dtv), J[q])));
             bool finite = true;
-            if constexpr (sizeof(T) == sizeof(double)) {
-                T phi = 0;
+            T jsum = 0, gsum = 0;
 #pragma unroll
-                for (int q = 0; q < Q; q++) {
-                    io.f_out[q * N + c] = nw[q].x;
+            for (int q = 0; q < Q; q++) {
+                io.f_out[q * N + c] = nw[q].x;
+                finite = finite && isfinite(nw[q].x);
+                jsum += J[q].y;
+                if (q > 0) {
                     io.g_out[q * N + c] = nw[q].y;
-                    phi += nw[q].y;
-                    finite = finite && isfinite(nw[q].x) && isfinite(nw[q].y);
+                    gsum += nw[q].y;
+                    finite = finite && isfinite(nw[q].y);
                 }
-                io.phi_out[c] = phi;
-            } else {
-                T jsum = 0, gsum = 0;
-#pragma unroll
-                for (int q = 0; q < Q; q++) {
-                    io.f_out[q * N + c] = nw[q].x;
-                    finite = finite && isfinite(nw[q].x);
-                    jsum += J[q].y;
-                    if (q > 0) {
-                        io.g_out[q * N + c] = nw[q].y;
-                        gsum += nw[q].y;
-                        finite = finite && isfinite(nw[q].y);
-                    }
-                }
-                const phi_t<T> phi = phi_add(S.phi[TL::i4(x, y)], -(dtv * jsum));
-                io.phi_out[c] = phi;
-                io.g_out[c] = phi_subt(phi, gsum);
-                finite = finite && isfinite(phi_val(phi));
             }
+            const phi_t<T> phi = phi_add(S.phi[TL::i4(x, y)], -(dtv * jsum));
+            io.phi_out[c] = phi;
+            io.g_out[c] = phi_subt(phi, gsum);
+            finite = finite && isfinite(phi_val(phi));
             if (!finite) atomicOr(io.status + t.x, ST_NONFINITE);
         }
         // the threads that the update leaves idle shift the mu, p and aux
@@ -575,7 +606,7 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
             if (!UNI) {
                 S.gf[L::W4 + r] = S.gf[L::W4 + BY + r];
 #pragma unroll
-                for (int k = 0; k < 11; k++) S.ga[k * L::NG + L::W4 + r] = S.ga[k * L::NG + L::W4 + BY + r];
+                for (int k = 0; k < L::NGA; k++) S.ga[k * L::NG + L::W4 + r] = S.ga[k * L::NG + L::W4 + BY + r];
             }
             // the same thread then writes the geometry of the next block's new row r
             set_geo(L::W4 + 8 + r, false, 4 + r, grow(b + 1, 4 + r));
