@@ -78,7 +78,13 @@ struct dugks_sim {
     int n_uni_s[kNumKernelShapes] = {};
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph2 = nullptr;   // k_step(A -> B), k_step(B -> A)
-    int *d_status = nullptr;
+    int *d_status = nullptr;      // per instance, then the error word of the many-step launches
+    // many-step launches: progress counters, ring neighbours (FLOW_NB per tile) and the value
+    // that every counter holds; built by the first call that uses it
+    unsigned *d_flow = nullptr;
+    int *d_flow_nbr = nullptr;
+    unsigned flow_base = 0;
+    bool flow_off = false;        // the cooperative launch was refused
     double2 *d_partials = nullptr;
     RedTile *d_red = nullptr;     // FP32 sims: one record per tile for the conservation sums
     float2 *d_redgeo = nullptr;   // FP32 sims: the widths {d, d_lo} of the geometry records
@@ -347,35 +353,40 @@ int shape_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm
 }
 
 // The tile that shape 0 runs on: its 32x8 cells, or the smaller tile that the
-// meshes make faster.  A tile's thread block takes `lat` when it has an SM for
-// itself and adds `sat` to an SM that is busy with others, so n tiles take
-// about lat + (ceil(n / n_sm) - 1) sat; the least estimate wins, the larger
-// tile on a tie.  The times (us, GB300) are those of a step that fits one wave
-// (64x64 drop) and of a 512x512 drop per tile of an SM:
+// meshes make faster.  A step takes about `lat` while no SM has more than one
+// tile, and `sat` more for each further tile of an SM; the least estimate wins,
+// the larger tile on a tie.  An SM's tiles share its FP64 pipe, so up to two per
+// SM the fullest SM counts in FP64; beyond that, and in FP32, where they hide each
+// other's latencies, the mean does.  us, measured in many-step launches (32x8 of a
+// 192x192, 16x8 of a 128x128, 8x8 of a 96x96 and FP64 8x4 of a 64x64 drop; sat
+// from a 512x512 drop):
 //            FP64 lat / sat     FP32 lat / sat
-//   32x8        82 / 80           8.2 / 4.8
-//   16x8        52 / 40           7.2 / 2.75
-//   8x8         36 / 24           6.15 / 1.98
-//   8x4, 4x8  22.5 / 15           as 8x8 in FP32: left out
-// Steps measured with the 32x8 tile and with the choice: FP64 64x64 drop 82 and
-// 22.5 us (8x4), 128x128 drop 82 and 52 (16x8), 4x256 channel 86 and 26.7 (4x8:
-// its four columns fill a tile, where 32 columns hold each cell eight times);
-// FP32 64x64 drop 8.2 and 6.2 (8x8), 4x256 channel 10.3 and 7.2 (8x8), 256x256
-// drop 12.3 with the 32x8 tile, which the rule keeps (16x8: 13.4).
+//   32x8        80 / 82.5         9.1 / 4.2
+//   16x8        51 / 41           7.0 / 2.6
+//   8x8       33.7 / 25           5.4 / 2.4
+//   8x4, 4x8  20.6 / 15.8         no gain over 8x8: left out
+// us per step with 32x8 tiles, 16x8, 8x8 and (FP64) 8x4: 64x64 drop FP64 80, 51,
+// 33.7, 20.6, FP32 7.3, 5.4, 4.4; 128x128 FP64 80, 51, 53, 58, FP32 8.2, 7.0, 7.5;
+// 256x256 FP64 162, 156, 168, 215, FP32 11.7, 12.1, 16.1; 512x512 FP64 556, 551,
+// 670, 851, FP32 32.8, 41, 62; 4x256 channel FP64 85, 57, 36, 25 (4x8: its four
+// columns fill a tile, where 32 columns hold each cell eight times), FP32 9.1,
+// 6.4, 5.1; four 100x100 drops FP64 111, 99, 111, 136, FP32 11.3, 10.1, 10.9.
 int tile_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm)
 {
-    struct Cost { int k; float lat, sat; };
-    static const Cost f64[] = {{0, 82.f, 80.f}, {7, 52.f, 40.f}, {8, 36.f, 24.f}, {9, 22.5f, 15.f}, {10, 22.5f, 15.f}};
-    static const Cost f32[] = {{0, 8.2f, 4.8f}, {7, 7.2f, 2.75f}, {8, 6.15f, 1.98f}};
+    struct Cost { int k; double lat, sat; };
+    static const Cost f64[] = {{0, 80, 82.5}, {7, 51, 41}, {8, 33.7, 25}, {9, 20.6, 15.8}, {10, 20.6, 15.8}};
+    static const Cost f32[] = {{0, 9.1, 4.2}, {7, 7.0, 2.6}, {8, 5.4, 2.4}};
     const bool d = precision == DUGKS_FP64;
     const Cost *c = d ? f64 : f32;
     int best = 0;
-    float best_t = 0.f;
+    double best_t = 0;
     for (int i = 0; i < (d ? 5 : 3); i++) {
         const ShapeDesc &S = kShapes[c[i].k];
         long long tiles = 0;
         for (int k = 0; k < n; k++) tiles += (long long)((nx[k] + S.bx - 1) / S.bx) * ((ny[k] + S.by - 1) / S.by);
-        const float t = c[i].lat + (float)((tiles + n_sm - 1) / n_sm - 1) * c[i].sat;
+        double per = (double)tiles / n_sm;
+        if (d && per <= 2) per = std::ceil(per);
+        const double t = c[i].lat + std::max(0.0, per - 1) * c[i].sat;
         if (i == 0 || t < best_t) { best = c[i].k; best_t = t; }
     }
     return best;
@@ -573,9 +584,161 @@ int build_graph2(dugks_sim *s)
     return cuda_status(e);
 }
 
+// Steps of one call from which a many-step launch takes them, and the most per
+// launch.  A call of fewer steps keeps its launch per step (or per two): the
+// cooperative launch costs about two of a small mesh's steps.  us per step in
+// calls of 60, launches and many-step: FP32 64x64 drop 6.2 and 4.5, four 4x256
+// channels 7.2 and 5.8, Rayleigh-Taylor 256x512 24.7 and 19.4 and 256x1024 39.0
+// and 38.3; FP64 64x64 drop 22.5 and 20.6, 4x256 channel 26.7 and 24.7, four
+// 100x100 drops 132 and 98.6, Rayleigh-Taylor 256x1024 594 and 576.  FP32
+// meshes of more tiles than FLOW_TILES per SM keep the launches: their last wave
+// is a small part of a step, and a tile that comes by the hardware's scheduler
+// needs no wait (512x512 drop, 6.7 tiles per SM: 32.8 and 32.8; 1024x1024, 27
+// tiles per SM: 130 and 147).
+constexpr long FLOW_MIN = 16, FLOW_MAX = 512;
+constexpr int FLOW_TILES = 7;
+
+// The tiles that each tile's 4-cell ring reads, itself among them, by the tile
+// columns and rows that hold the ring's cells (a narrow last column or row lets
+// the ring reach past it).
+int ensure_flow(dugks_sim *s, int k)
+{
+    if (s->d_flow) return DUGKS_OK;
+    const int bx = kShapes[k].bx, by = kShapes[k].by;
+    std::vector<int> nbr;
+    auto reach = [](int n, int b, bool periodic) {
+        const int m = (n + b - 1) / b;
+        std::vector<std::vector<char>> r(m, std::vector<char>(m, 0));
+        for (int c = 0; c < m; c++)
+            for (int g = c * b - 4; g < std::min(n, (c + 1) * b) + 4; g++) {
+                if (!periodic && (g < 0 || g >= n)) continue;
+                const int d = ((g % n) + n) % n / b;
+                r[c][d] = r[d][c] = 1;
+            }
+        std::vector<std::vector<int>> out(m);
+        for (int c = 0; c < m; c++)
+            for (int d = 0; d < m; d++) if (r[c][d]) out[c].push_back(d);
+        return out;
+    };
+    int first = 0;
+    for (const InstDev &I : s->h_inst) {   // the tile table's order: one class of instance, row by row
+        const auto rx = reach(I.nx, bx, I.bcx == 0), ry = reach(I.ny, by, I.bcy == 0);
+        for (size_t ty = 0; ty < ry.size(); ty++)
+            for (size_t tx = 0; tx < rx.size(); tx++) {
+                const size_t at = nbr.size();
+                nbr.resize(at + FLOW_NB, -1);
+                size_t c = 0;
+                for (int y : ry[ty])
+                    for (int x : rx[tx]) {
+                        if (c == FLOW_NB) return DUGKS_ERR_UNSUPPORTED;
+                        nbr[at + c++] = first + y * (int)rx.size() + x;
+                    }
+            }
+        first += (int)(rx.size() * ry.size());
+    }
+    cudaError_t e = dmalloc(s, (void **)&s->d_flow_nbr, sizeof(int) * nbr.size());
+    if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_flow, sizeof(unsigned) * first);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->d_flow_nbr, nbr.data(), sizeof(int) * nbr.size(), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_flow, 0, sizeof(unsigned) * first, s->stream);
+    if (e != cudaSuccess) {
+        dfree(s, s->d_flow_nbr);
+        dfree(s, s->d_flow);
+        s->d_flow_nbr = nullptr;
+        s->d_flow = nullptr;
+    }
+    s->flow_base = 0;
+    return cuda_status(e);
+}
+
+template <typename T, int BX, int BY, int NT>
+int launch_flow(dugks_sim *s, int k, int n)
+{
+    using L = FusedLayout<T, BX, BY, false>;
+    constexpr int MB = fused_minb<T, NT, false>();
+    static int resident[2] = {0, 0};   // blocks per SM of each class's kernel
+    const bool uni = s->n_uni_s[k] > 0;
+    const void *f = uni ? (const void *)k_step<T, BX, BY, NT, MB, true, false, true>
+                        : (const void *)k_step<T, BX, BY, NT, MB, false, false, true>;
+    if (!resident[uni]) {
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[uni], f, NT, L::bytes);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    int rc = ensure_flow(s, k);
+    if (rc) return rc;
+    const AxisRecT<T> *geo = (const AxisRecT<T> *)s->d_geoT;
+    StepIO<T> io = step_io<T>(s);
+    Flow<T> fl;
+    fl.io[0] = fl.io[1] = io;
+    fl.io[1].f_in = io.f_out; fl.io[1].g_in = io.g_out; fl.io[1].phi_in = io.phi_out;
+    fl.io[1].f_out = const_cast<T *>(io.f_in); fl.io[1].g_out = const_cast<T *>(io.g_in);
+    fl.io[1].phi_out = const_cast<phi_t<T> *>(io.phi_in);
+    fl.n_tiles = s->n_tiles_s[k];
+    fl.n_steps = n;
+    fl.base = s->flow_base;
+    fl.done = s->d_flow;
+    fl.nbr = s->d_flow_nbr;
+    fl.err = s->d_status + s->n_inst;
+    fl.limit = 1u << 22;   // a few seconds of polls
+    const int grid = std::min(fl.n_tiles, resident[uni] * s->n_sm);
+    const int4 *tiles = s->d_tiles_s[k];
+    const InstDev *insts = s->d_inst;
+    void *args[] = {&insts, &tiles, &geo, &fl};
+    cudaError_t e;
+    {
+        Timed t(s, K_STEP, n, 1);
+        e = cudaLaunchCooperativeKernel(f, dim3(grid), dim3(NT), args, L::bytes, s->stream);
+    }
+    if (e != cudaSuccess) {
+        s->launches--;
+        return cuda_status(e);
+    }
+    s->flow_base += (unsigned)n;
+    if (n & 1) swap_state<T>(s, io);
+    return DUGKS_OK;
+}
+
+// Many steps of a sim whose step is one kernel of tiles: returns the steps done,
+// 0 where the launches of step_fused have to do (a stream under capture, whose
+// replay would meet old counters; two classes of instance; a refused launch).
+template <typename T>
+long step_flow(dugks_sim *s, long n)
+{
+    const int k = kernel_shape(s);
+    if (s->flow_off || s->shape != 0 || n < FLOW_MIN || !s->use_graph || prepare_fused<T>(s) != DUGKS_OK) return 0;
+    if (s->n_uni_s[k] > 0 && s->n_uni_s[k] < s->n_tiles_s[k]) return 0;
+    if (sizeof(T) == 4 && s->n_tiles_s[k] > FLOW_TILES * s->n_sm) return 0;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return 0;
+    }
+    long done = 0;
+    while (n - done >= FLOW_MIN) {
+        const int m = (int)std::min(n - done, FLOW_MAX);
+        int rc;
+        if constexpr (sizeof(T) == 8) {
+            rc = k == 7 ? launch_flow<T, 16, 8, 128>(s, k, m) : k == 8 ? launch_flow<T, 8, 8, 128>(s, k, m)
+               : k == 9 ? launch_flow<T, 8, 4, 128>(s, k, m) : k == 10 ? launch_flow<T, 4, 8, 128>(s, k, m)
+                                                                       : launch_flow<T, 32, 8, 256>(s, k, m);
+        } else {
+            rc = k == 7 ? launch_flow<T, 16, 8, 256>(s, k, m) : k == 8 ? launch_flow<T, 8, 8, 256>(s, k, m)
+                                                                       : launch_flow<T, 32, 8, 256>(s, k, m);
+        }
+        if (rc) {
+            cudaGetLastError();
+            s->flow_off = true;
+            break;
+        }
+        done += m;
+    }
+    return done;
+}
+
 template <typename T>
 int step_fused(dugks_sim *s, long n)
 {
+    n -= step_flow<T>(s, n);
     // the graph starts from the first buffer; one plain step realigns
     const bool in_first = (void *)planes<T>(s).f == s->d_planes;
     long k = 0;
@@ -800,6 +963,8 @@ void free_sim(dugks_sim *s)
     dfree(s, s->d_alt_alloc);
     dfree(s, s->d_phi_alt_alloc);
     dfree(s, s->d_status);
+    dfree(s, s->d_flow);
+    dfree(s, s->d_flow_nbr);
     dfree(s, s->d_partials);
     dfree(s, s->d_red);
     dfree(s, s->d_redgeo);
@@ -820,6 +985,18 @@ void free_sim(dugks_sim *s)
     delete s;
 }
 
+// A new state: every instance finite and running, the counters of the many-step launches (which a
+// wait that ran out leaves uneven) and error word at zero.
+cudaError_t reset_status(dugks_sim *s)
+{
+    cudaError_t e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * (s->n_inst + 1), s->stream);
+    if (e == cudaSuccess && s->d_flow) {
+        e = cudaMemsetAsync(s->d_flow, 0, sizeof(unsigned) * s->n_tiles_s[s->tile0], s->stream);
+        s->flow_base = 0;
+    }
+    return e;
+}
+
 // After a synchronisation: a single simulation reports a non-finite state as
 // DUGKS_ERR_NONFINITE; a batch masks the affected instances and reports them
 // through dugks_batch_status only.
@@ -827,12 +1004,14 @@ int sync_status(dugks_sim *s)
 {
     cudaError_t e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
-    if (s->n_inst > 1) return DUGKS_OK;
-    std::vector<int> st(s->n_inst);
-    e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
+    if (s->n_inst > 1 && !s->d_flow) return DUGKS_OK;
+    // the status of the instance (of a single sim) and the error word
+    const int first = s->n_inst > 1 ? s->n_inst : 0, n = s->n_inst + 1 - first;
+    int st[2] = {0, 0};
+    e = cudaMemcpy(st, s->d_status + first, sizeof(int) * n, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
-    for (int v : st) if (v & ST_NONFINITE) return DUGKS_ERR_NONFINITE;
-    return DUGKS_OK;
+    if (st[n - 1]) return DUGKS_ERR_TIMEOUT;
+    return n == 2 && (st[0] & ST_NONFINITE) ? DUGKS_ERR_NONFINITE : DUGKS_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -905,7 +1084,7 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     int rc = DUGKS_OK;
     // forward from the saved init inputs, with checkpoints
     e = cudaMemcpyAsync(s->d_stage, s->d_init_in, sizeof(double) * 4 * D, cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * n, s->stream);
+    if (e == cudaSuccess) e = reset_status(s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(w.target, target_h, sizeof(double) * D, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.pk, 0, sizeof(double) * 3 * n, s->stream);
     if (e != cudaSuccess) rc = cuda_status(e);
@@ -1191,7 +1370,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
     chk(dmalloc(s, (void **)&s->d_phi_alt_alloc, sizeof(double) * (size_t)s->N));
     s->d_alt = s->d_alt_alloc;
     s->d_phi_alt = s->d_phi_alt_alloc;
-    chk(dmalloc(s, (void **)&s->d_status, sizeof(int) * n));
+    chk(dmalloc(s, (void **)&s->d_status, sizeof(int) * (n + 1)));
     chk(dmalloc(s, (void **)&s->d_partials, sizeof(double2) * tiles.size()));
     // FP32 sims: the conservation sums' tile records and compact widths
     std::vector<RedTile> red;
@@ -1235,7 +1414,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
     chk(cudaMemset(s->d_phi, 0, sizeof(double) * (size_t)s->N));
     chk(cudaMemset(s->d_alt_alloc, 0, esz * 2 * Q * (size_t)s->N));
     chk(cudaMemset(s->d_phi_alt_alloc, 0, sizeof(double) * (size_t)s->N));
-    chk(cudaMemset(s->d_status, 0, sizeof(int) * n));
+    chk(cudaMemset(s->d_status, 0, sizeof(int) * (n + 1)));
     if (e != cudaSuccess) {
         int rc = cuda_status(e);
         free_sim(s);
@@ -1282,7 +1461,7 @@ int dugks_init(dugks_sim *s, const double *phi, const double *ux, const double *
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     if (bad) return DUGKS_ERR_NONFINITE;
-    e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * s->n_inst, s->stream);
+    e = reset_status(s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(s->d_init_in, s->d_stage, sizeof(double) * 4 * D, cudaMemcpyDeviceToDevice, s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     int rc = s->prec == DUGKS_FP64 ? do_init<double>(s) : do_init<float>(s);
@@ -1380,13 +1559,13 @@ int dugks_conservation_async(dugks_sim *s, double *sums)
     if (!host_alias(sums)) return DUGKS_ERR_ARG;   // pageable memory: the copy could not be asynchronous
     cudaError_t e = cudaSuccess;
     if (!s->ev_cons) e = cudaEventCreateWithFlags(&s->ev_cons, cudaEventDisableTiming);
-    if (e == cudaSuccess && !s->h_status) e = cudaHostAlloc((void **)&s->h_status, sizeof(int) * s->n_inst, cudaHostAllocDefault);
+    if (e == cudaSuccess && !s->h_status) e = cudaHostAlloc((void **)&s->h_status, sizeof(int) * (s->n_inst + 1), cudaHostAllocDefault);
     if (e != cudaSuccess) return cuda_status(e);
     int rc = s->prec == DUGKS_FP64 ? do_reduce<double>(s) : do_reduce<float>(s);
     if (rc) return rc;
     // d_sums holds (sum phi, sum rho) per instance: the layout of sums
     e = cudaMemcpyAsync(sums, s->d_sums, sizeof(double2) * s->n_inst, cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_status, s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_status, s->d_status, sizeof(int) * (s->n_inst + 1), cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaEventRecord(s->ev_cons, s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     s->cons_pending = true;
@@ -1400,6 +1579,7 @@ int dugks_conservation_wait(dugks_sim *s)
     const cudaError_t e = cudaEventSynchronize(s->ev_cons);
     if (e != cudaSuccess) return cuda_status(e);
     s->cons_pending = false;
+    if (s->h_status[s->n_inst]) return DUGKS_ERR_TIMEOUT;
     if (s->n_inst == 1 && (s->h_status[0] & ST_NONFINITE)) return DUGKS_ERR_NONFINITE;
     return DUGKS_OK;
 }
@@ -1514,7 +1694,7 @@ int dugks_load(dugks_sim *s, const void *buf, size_t bytes)
     const double *h = (const double *)buf;
     for (size_t k = 0; k < need / sizeof(double); k++) if (!std::isfinite(h[k])) return DUGKS_ERR_NONFINITE;
     cudaError_t e = cudaMemcpyAsync(s->d_stage, buf, need, cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * s->n_inst, s->stream);
+    if (e == cudaSuccess) e = reset_status(s);
     if (e != cudaSuccess) return cuda_status(e);
     int rc = s->prec == DUGKS_FP64 ? do_unpack_state<double>(s, s->d_stage) : do_unpack_state<float>(s, s->d_stage);
     if (rc) return rc;

@@ -16,6 +16,8 @@
 // of being written to and re-read from HBM; the state is double-buffered
 // because tiles read the old state of their ring.
 #pragma once
+#include <type_traits>
+
 #include "dugks_fp64.cuh"
 #include "dugks_kernels.cuh"
 
@@ -358,26 +360,97 @@ __device__ __forceinline__ void tile_face(const InstDev &I, const TL &S, int xa,
     face_tail<T, A>(I, fb, gb, ax, true, side, area, F2o);
 }
 
+// What k_step needs to run many steps in one launch: the tiles it runs and for
+// how many steps, one progress counter per tile, and the tiles that a tile's
+// 4-cell ring reads (FLOW_NB entries per tile, -1 beyond the last).
+constexpr int FLOW_NB = 32;
+template <typename T>
+struct Flow {
+    StepIO<T> io[2];           // of the even and the odd steps: the two state buffers alternate
+    int n_tiles, n_steps;
+    unsigned base;             // every counter's value before the first step
+    unsigned *done;            // base + steps completed, per tile
+    const int *nbr;
+    int *err;                  // set when a wait ran out
+    unsigned limit;            // polls before a wait gives up
+};
+template <typename T>
+__device__ __forceinline__ const StepIO<T> &step_io_of(const StepIO<T> &io, int) { return io; }
+template <typename T>
+__device__ __forceinline__ const StepIO<T> &step_io_of(const Flow<T> &fl, int step) { return fl.io[step & 1]; }
+
 // NT threads (a multiple of 32, at least BX * BY) share the phases of a
 // BX x BY tile; the first BX * BY of them own one cell each in the update.
-template <typename T, int BX, int BY, int NT, int MINB, bool UNI, bool SEP>
+// One step: a thread block per tile.  FLOW: many steps in one cooperative launch,
+// without a barrier of the device between them: block b takes the items b, b + gridDim.x, ... of the sequence (step 0:
+// all tiles, step 1: all tiles, ...), and waits for an item only until the tiles
+// that its ring reads have finished the step before.  All blocks are resident
+// (cooperative launch) and an item waits only for earlier items, so every wait
+// ends.  The two state buffers alternate: a tile overwrites a buffer only after
+// its neighbours, which are the tiles that read it (the ring relation is
+// symmetric), have finished the step that read it.
+// What bounded the launches it replaces: a small mesh paid the gap between two
+// dependent kernels (about 2 us) and the geometry set-up every step, and a step of
+// a few waves waited for its last, partly filled one (four 100x100 drops in FP64:
+// 364 tiles of 16x8 on 304 resident blocks, 132 -> 98.6 us per step).
+template <typename T, int BX, int BY, int NT, int MINB, bool UNI, bool SEP, bool FLOW = false>
 __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                   const AxisRecT<T> *__restrict__ geo, StepIO<T> io)
+                                                   const AxisRecT<T> *__restrict__ geo,
+                                                   const __grid_constant__ std::conditional_t<FLOW, Flow<T>, StepIO<T>> arg)
 {
     static_assert(NT % 32 == 0 && NT >= BX * BY, "thread count");
     using TL = Tile<T, BX, BY, UNI, SEP>;
     using L = typename TL::L;
     extern __shared__ __align__(16) unsigned char smem[];
     TL S(smem);
-    const int4 t = tiles[blockIdx.x];
+    const int tid = threadIdx.x;
+    __shared__ int s_status;   // FLOW: one reading for the whole block (another block may set a bit meanwhile)
+    int item = blockIdx.x, step = 0, last = -1;   // FLOW: the tile, the step, the tile whose geometry S holds
+    for (;;) {
+    if constexpr (FLOW) {
+        if (item >= arg.n_tiles) {
+            item -= arg.n_tiles;
+            if (++step == arg.n_steps) return;
+            continue;
+        }
+        bool late = false;
+        if (tid < 32 && step > 0) {
+            const int n = arg.nbr[item * FLOW_NB + tid];
+            if (n >= 0) {
+                const unsigned want = arg.base + (unsigned)step;
+                for (unsigned k = 0;; k++) {
+                    unsigned v;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arg.done + n) : "memory");
+                    if ((int)(v - want) >= 0) break;
+                    if (k >= arg.limit || (k % 256 == 255 && *(volatile int *)arg.err)) {
+                        late = true;
+                        break;
+                    }
+                }
+            }
+            if (late) atomicExch(arg.err, 1);
+        }
+        if (tid == 0) s_status = *(const volatile int *)(arg.io[0].status + tiles[item].x);
+        // also: every thread is done with shared memory, and the neighbours'
+        // state (seen by the polling warp) is visible to all
+        if (__syncthreads_or(late)) return;
+    }
+    const bool fresh = !FLOW || item != last;
+    const int4 t = tiles[item];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
+    const StepIO<T> &io = step_io_of(arg, step);
     const int i0 = t.y, j0 = t.z;
-    const int tid = threadIdx.x;
+    do {   // left by the threads that have nothing more to do for the tile
     {
-        const int st = io.status[t.x];
-        if (st & ST_NONFINITE) return;   // masked: non-finite instance of a batch
-        if (st & ST_PAUSED) {            // paused: the state passes to the other buffer unchanged
+        int st;
+        if constexpr (FLOW) {
+            st = s_status;
+        } else {
+            st = io.status[t.x];
+        }
+        if (st & ST_NONFINITE) break;   // masked: non-finite instance of a batch
+        if (st & ST_PAUSED) {           // paused: the state passes to the other buffer unchanged
             const int x = tid % BX, y = tid / BX;
             if (tid < BX * BY && i0 + x < I.nx && j0 + y < I.ny) {
                 const long long c = I.cell0 + (long long)(j0 + y) * I.nxp + (i0 + x);
@@ -388,13 +461,14 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
                 }
                 io.phi_out[c] = io.phi_in[c];
             }
-            return;
+            break;
         }
     }
     const long long N = io.N;
 
     // global index of every region column and row (wrapped on periodic axes,
     // -1 outside the domain), kept in shared memory for all later phases
+    if (fresh)
     for (int r = tid; r < L::NG; r += NT) {
         const bool isx = r < L::W4;
         const int n = isx ? I.nx : I.ny;
@@ -407,7 +481,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         }
         S.gg[r] = g;
     }
-    __syncthreads();
+    if (fresh) __syncthreads();
     auto gpos = [&](bool isx, int pos) -> int { return S.gg[isx ? pos + 4 : L::W4 + pos + 4]; };
     auto cell = [&](int gi, int gj) -> long long { return I.cell0 + (long long)gj * I.nxp + gi; };
 
@@ -450,6 +524,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     cp_commit();
 
     // ---- geometry of the region columns and rows (SoA)
+    if (fresh)
     for (int r = tid; r < L::NG; r += NT) {
         const bool isx = r < L::W4;
         const int pos = isx ? r - 4 : r - L::W4 - 4;
@@ -647,11 +722,6 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     }
     __syncthreads();
 
-    const int x = tid % BX, y = tid / BX;
-    const int gi = i0 + x, gj = j0 + y;
-    const bool own = tid < BX * BY && gi < I.nx && gj < I.ny;
-    const long long c = own ? cell(gi, gj) : 0;
-
     // ---- phase 5: every face of the tile once (x faces first in the item space)
     for (int k = tid; k < L::NFT; k += NT) {
         pair_t<T> F2o[6];
@@ -677,7 +747,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         constexpr int NC = BX * BY;
         constexpr bool SPLIT = 2 * NC <= NT && NC % 32 == 0;
         const int cid = SPLIT ? tid % NC : tid, ux = cid % BX, uy = cid / BX;
-        if (tid >= (SPLIT ? 2 * NC : NC) || i0 + ux >= I.nx || j0 + uy >= I.ny) return;
+        if (tid >= (SPLIT ? 2 * NC : NC) || i0 + ux >= I.nx || j0 + uy >= I.ny) break;
         const long long cc = cell(i0 + ux, j0 + uy);
         const int kw = uy * L::XP + ux, ks = L::Y0 + uy * BX + ux;
         auto e = [&](int m) { return S.flux[m * L::NFT + kw + 1]; };
@@ -689,9 +759,12 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         else if (tid < NC) ok = fp64::update_cell<1>(io, S, ux, uy, cc, e, w, n, so);
         else ok = fp64::update_cell<2>(io, S, ux, uy, cc, e, w, n, so);
         if (!ok) atomicOr(io.status + t.x, ST_NONFINITE);
-        return;
+        break;
     }
-    if (!own) return;
+    const int x = tid % BX, y = tid / BX;
+    const int gi = i0 + x, gj = j0 + y;
+    if (tid >= BX * BY || gi >= I.nx || gj >= I.ny) break;
+    const long long c = cell(gi, gj);
     // J of both kinds at once: east minus west for the x set, north minus south for the y set
     pair_t<T> J[Q];
 #pragma unroll
@@ -737,6 +810,17 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     io.g_out[c] = phi_subt(phi, gsum);
     finite = finite && isfinite(phi_val(phi));
     if (!finite) atomicOr(io.status + t.x, 1);
+    } while (false);
+    if constexpr (!FLOW) {
+        return;
+    } else {
+        last = item;
+        __syncthreads();
+        if (tid == 0)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(arg.done + item), "r"(arg.base + (unsigned)step + 1u) : "memory");
+        item += gridDim.x;
+    }
+    }
 }
 
 }  // namespace dugks
