@@ -1,34 +1,540 @@
 // dugks_adjoint.cuh -- reverse-mode (adjoint) sweep of one DUGKS step and of
-// the initialisation, written by hand as the transpose of the forward kernels
-// of dugks_kernels.cuh (Sec. 2.2 procedure).
+// the initialisation, written by hand as the transpose of the forward step
+// (Sec. 2.2 procedure).
 //
-// Forward step n (the four-kernel form, whose intermediates the adjoint reads):
-//   k_mu    mu = psi'(phi) - kappa lap(phi)
-//   k_macro grad mu, lap mu, grad phi, F, u, p
-//   k_cell  grad p, equilibria, sources, bar-plus (Eq. relations1)
-//   k_face  reconstruction, face macros, originals, flux, update (Eq. updatef)
+// Forward step n leaves what the reverse step reads (k_step, MODE_PLANES):
+//   mu, grad mu, lap mu, grad phi, u, p, grad p and bar-plus of every cell.
 // Reverse, given the adjoint xb of the state at n+1:
-//   ka_face_t update and faces  -> adjoint of bar-plus and of the face aux fields
-//   ka_cell   bar-plus          -> adjoint of tilde, of u, p, phi, mu and gradients
-//   ka_macro  transpose grad p, then p, u, F -> adjoint of tilde f, phi, grad mu, ...
-//   ka_mu     transpose grad mu, lap mu, then mu -> adjoint of phi, lap phi
-//   ka_phi    transpose grad phi, lap phi, then phi = sum g -> adjoint of tilde g
-// The parameters kappa and lambda (the mobility) collect their adjoints per
-// instance in FP64.
+//   ka_face  one thread per face: reconstruction and face macros again, then their
+//            transpose -> what each face gives its bar values and aux fields
+//   ka_cell  gathers the gifts of a cell's faces (the transpose of the
+//            reconstruction), then bar-plus -> adjoint of tilde, of u, p, phi, mu
+//            and the gradients
+//   ka_tail  transpose grad p, then p, u, F -> adjoint of tilde f, phi, grad mu, ...;
+//            transpose grad mu, lap mu, then mu -> adjoint of phi, lap phi;
+//            transpose grad phi, lap phi, then phi = sum g -> adjoint of tilde g
+// Nothing is scattered: every value has one writer, so a gradient comes out the
+// same every time.  The parameters kappa and lambda (the mobility) collect their
+// adjoints in FP64, one slot per warp of a kernel, added up per instance at the
+// end.
+//
+// One warp takes a run of 32 cells or faces of a row (AdjSeg), so that the work of
+// a small mesh spreads over all SM sub-partitions; the point transpose is that of
+// the regrouped equilibria and sources (dugks_fp64.cuh), about a third of the
+// operations of the transpose of the separate ones.
 #pragma once
 #include "dugks_fused.cuh"
 
 namespace dugks {
 
+// Gifts of a face, one plane each: to the bar f and bar g of the six flux
+// directions (fset order), to every bar f (AS), to +-bar f along the face (AM), to
+// every bar g (AP), and to the aux fields.
+constexpr int AF = 0, AG = 6, AS = 12, AM = 13, AP = 14, AX = 15, NFP = 23;
+
+// positions i .. i + 31 of row j of an instance; -1 is the face at a low wall.  Runs
+// follow each other up a column of 32, so that the warps of a block read each
+// other's rows.
+struct AdjSeg {
+    int inst, i, j, axis;   // axis: of the faces
+};
+
 template <typename T>
 struct AdjPlanes {
     const T *xf, *xg;   // adjoint of the tracked state at step n+1 [Q][N]
     T *af, *ag;         // adjoint of the tracked state at step n   [Q][N]
-    T *bp;              // adjoint of bar-plus [2Q][N]
+    T *face[2];         // [NFP][NF] per axis: the face between a cell and its high neighbour at
+                        // the cell's index; one at a low wall at N + the other axis' record
     T *phi, *mu, *lapmu, *gmx, *gmy, *gfx, *gfy, *gpx, *gpy, *p, *ux, *uy, *lapphi;  // [N]
-    double *pk;         // [2 * n_inst]: d/dlambda, d/dkappa per instance
-    long long N;
+    double *lam_face, *lam_cell, *lam_macro, *kap, *kap0;   // slots of the parameters' adjoints, per warp
+    long long N, NF;
 };
+
+template <typename T>
+__device__ __forceinline__ T recip(T x);
+template <>
+__device__ __forceinline__ float recip<float>(float x) { return __frcp_rn(x); }
+template <>
+__device__ __forceinline__ double recip<double>(double x) { return fp64::rcp(x); }
+
+// add a warp's sum of v to its slot
+template <typename T>
+__device__ __forceinline__ void slot_add(double *slot, T v)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) *slot += (double)v;
+}
+
+// A point of the scheme (a cell in bar-plus, or a face) and its adjoint.
+template <typename T>
+struct APt {
+    T phi, ux, uy, p, mu, lmu, gmx, gmy, gfx, gfy, gpx, gpy;
+};
+
+// Transpose of bar-plus of a cell (A = -1: all directions) or of the originals of
+// a face of axis A (its flux directions) with respect to the point's variables:
+// a f + b f^eq + c F^f and ga g + ..., given their adjoints ob, yb.  Returns a
+// (a cell: b = 1 - a); fsum is sum f ob, the adjoint of a.  B: the adjoint of the
+// point, with that of rho and of the weights in phi's; of a cell's u and p, and at a
+// face, whose p and u are formed from its bars, of sum f (in p) and sum xi f (in u).
+template <typename T, int A>
+__device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const T (&ob)[Q], const T (&yb)[Q], T fsum, bool wall,
+                                       APt<T> &B, T &lam)
+{
+    constexpr bool CELL = A < 0;
+    const ParT<T> &Pr = par<T>(I);
+    const PtC<T> &C = CELL ? cellc<T>(I) : facec<T>(I);
+    const T rho = Pr.rhoB + Pr.drho * (s.phi - Pr.phiB), irho = recip(rho);
+    const T Fx = -s.phi * s.gmx + (rho - Pr.rho_ref) * Pr.gxa, Fy = -s.phi * s.gmy + (rho - Pr.rho_ref) * Pr.gya;
+    const T D = (s.phi - Pr.phiB) * Pr.hmuB + (Pr.phiA - s.phi) * Pr.hmuA, X = D * rho;
+    const T kx = CELL ? T(2) : T(1);
+    const T r = recip(C.k6 + kx * X);
+    const T a = (CELL ? C.k6 - X : C.k6) * r, b = C.nb * X * r, c = C.nc * r;
+    const T ECx = Fx + C.cd * s.gfx, ECy = Fy + C.cd * s.gfy;      // F + c_s^2 grad rho
+    const T uF = s.ux * Fx + s.uy * Fy, uE = s.ux * ECx + s.uy * ECy;
+    const T rl = rho * s.lmu, src = C.cgl * rl + uF;
+    const T rho3 = rho * T(1.0 / 3.0);
+    const T K1 = b * rho3 - c * uE;
+    const T fx = c * Fx, fy = c * Fy, ex = c * ECx, ey = c * ECy;
+    const T Gx = Fx - s.gpx, Gy = Fy - s.gpy, Pg = C.gc * s.phi * irho, gx = Pg * Gx, gy = Pg * Gy;
+    const T ug = s.ux * gx + s.uy * gy, D2 = C.gb * s.phi - ug;
+    const T s0 = T(-1.5) * (s.ux * s.ux + s.uy * s.uy);
+    // directions: z, y are the adjoints times the weight over the diagonals'
+    T K0b = 0, K1b = 0, fxb = 0, fyb = 0, exb = 0, eyb = 0, A2b = 0, D2b = 0, gxb = 0, gyb = 0, s0b = 0, uxb = 0, uyb = 0;
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        if (!CELL && ca(q, CELL ? 0 : A) == 0) continue;
+        const T w = q == 0 ? T(16) : q < 5 ? T(4) : T(1);
+        const T z = w * ob[q], y = w * yb[q];
+        const T xu = xi_dot<T>(q, s.ux, s.uy), sq = s0 + (q == 0 ? T(0) : xu * (T(4.5) * xu + T(3)));
+        const T zs = z * sq, ys = y * sq;
+        K0b += z;
+        K1b += zs;
+        A2b += y;
+        D2b += ys;
+        T sb = z * K1 + y * D2;
+        if (q > 0) {
+            if (cx(q)) { fxb += T(cx(q)) * z; exb += T(cx(q)) * zs; gxb += T(cx(q)) * (y + ys); }
+            if (cy(q)) { fyb += T(cy(q)) * z; eyb += T(cy(q)) * zs; gyb += T(cy(q)) * (y + ys); }
+            sb += z * xi_dot<T>(q, ex, ey) + y * xi_dot<T>(q, gx, gy);
+            const T xub = sb * (T(9) * xu + T(3));
+            if (cx(q)) uxb += T(cx(q)) * xub;
+            if (cy(q)) uyb += T(cy(q)) * xub;
+        }
+        s0b += sb;
+    }
+    uxb -= T(3) * s.ux * s0b;
+    uyb -= T(3) * s.uy * s0b;
+    T phib = C.gb * D2b, rhob = 0, Hb = A2b;
+    if (CELL) {
+        // H of the rest direction is phi - (1 - w_0) eta mu: the adjoint of eta mu
+        // is sum w (yb_q - yb_0), formed from the differences, for yb hardly varies
+        // with q and the sum of separately rounded weights would leave a bias
+        phib += C.gb36 * yb[0];
+        Hb = 0;
+#pragma unroll
+        for (int q = 1; q < Q; q++) Hb += (q < 5 ? T(4) : T(1)) * (yb[q] - yb[0]);
+    }
+    const T mub = C.gbe * Hb;
+    lam += C.dgbe * s.mu * Hb;
+    // g: D2 = gb phi - u.G', A2 = gbe mu - u.G', G' = P (F - grad p), P = gc phi / rho
+    const T ugb = -(A2b + D2b);
+    uxb += ugb * gx;
+    uyb += ugb * gy;
+    gxb += ugb * s.ux;
+    gyb += ugb * s.uy;
+    const T Pb = gxb * Gx + gyb * Gy;
+    T Fxb = Pg * gxb, Fyb = Pg * gyb;
+    B.gpx = -Fxb;
+    B.gpy = -Fyb;
+    phib += C.gc * irho * Pb;
+    rhob -= Pg * irho * Pb;
+    // f: K0 = b p - c (cgl rho lap mu + u.F), K1 = b rho / 3 - c u.E, c F, c E
+    T bb = s.p * K0b + rho3 * K1b;
+    T cb = -(src * K0b) - uE * K1b + Fx * fxb + Fy * fyb + ECx * exb + ECy * eyb;
+    T pb = b * K0b;
+    const T tb = -c * K0b, uEb = -c * K1b;
+    rhob += C.cgl * s.lmu * tb + b * T(1.0 / 3.0) * K1b;
+    T lmub = C.cgl * rho * tb;
+    lam += C.dcgl * rl * tb;
+    const T ExB = c * exb + uEb * s.ux, EyB = c * eyb + uEb * s.uy;
+    Fxb += c * fxb + tb * s.ux + ExB;
+    Fyb += c * fyb + tb * s.uy + EyB;
+    uxb += tb * Fx + uEb * ECx;
+    uyb += tb * Fy + uEb * ECy;
+    T gfxb = C.cd * ExB, gfyb = C.cd * EyB;
+    // weights: a, b, c over 6K + k X; b-bar and a-bar nearly cancel (f is near
+    // equilibrium), so their difference is formed first
+    const T Xb = r * r * (C.k6 * (C.nb * bb - (CELL ? T(3) : T(1)) * fsum) - kx * C.nc * cb);
+    rhob += D * Xb;
+    phib += (Pr.hmuB - Pr.hmuA) * rho * Xb;
+    if (!CELL) {
+        // p = sum f + kp1 u.grad phi - kp2 rho lap mu, u = (m + kf F) 3 / rho
+        uxb += C.kp1 * pb * s.gfx;
+        uyb += C.kp1 * pb * s.gfy;
+        gfxb += C.kp1 * pb * s.ux;
+        gfyb += C.kp1 * pb * s.uy;
+        rhob -= C.kp2 * s.lmu * pb;
+        lmub -= C.kp2 * rho * pb;
+        lam -= C.dkp2 * rl * pb;
+        if (wall) uxb = uyb = T(0);
+        rhob -= (s.ux * uxb + s.uy * uyb) * irho;
+        uxb *= T(3) * irho;   // the adjoint of the momentum sum
+        uyb *= T(3) * irho;
+        Fxb += C.kf * uxb;
+        Fyb += C.kf * uyb;
+    }
+    // F = -phi grad mu + (rho - rho_ref) g, rho(phi)
+    phib -= s.gmx * Fxb + s.gmy * Fyb;
+    rhob += Pr.gxa * Fxb + Pr.gya * Fyb;
+    B.phi = phib + Pr.drho * rhob;
+    B.gmx = -s.phi * Fxb;
+    B.gmy = -s.phi * Fyb;
+    B.gfx = gfxb;
+    B.gfy = gfyb;
+    B.mu = mub;
+    B.lmu = lmub;
+    B.ux = uxb;
+    B.uy = uyb;
+    B.p = pb;
+    return CELL ? T(36) * b : a;
+}
+
+template <typename T>
+__device__ __forceinline__ const AxisRecT<T> &rec(const InstDev &I, const AxisRecT<T> *__restrict__ geo, int axis, int k)
+{
+    return geo[(axis == 0 ? I.gx_off : I.gy_off) + k];
+}
+
+// Index of the face at a low wall of axis A, at position t of the other axis.
+__device__ __forceinline__ long long low_face(const InstDev &I, long long N, int A, int t)
+{
+    return N + (A == 0 ? I.gy_off : I.gx_off) + t;
+}
+
+// The high face on axis A of the cell at position n of that axis and t of the
+// other, or the face at the low wall for n = -1.
+template <typename T, int A>
+__device__ __forceinline__ void face_of(const InstDev &I, const AxisRecT<T> *__restrict__ geo, const Planes<T> &P, const AdjPlanes<T> &Ad,
+                                        int n, int t, T &lam)
+{
+    const ParT<T> &Pr = par<T>(I);
+    const long long N = P.N;
+    auto cell = [&](int nn, int tt) -> long long { return A == 0 ? cell_of(I, nn, tt) : cell_of(I, tt, nn); };
+    const AxisRecT<T> &rt = rec<T>(I, geo, 1 - A, t);
+    const T em = rt.e1m, e0 = rt.e10, ep = rt.e1p, h = Pr.h;
+    const int nc = n < 0 ? 0 : n;
+    const AxisRecT<T> &rn = rec<T>(I, geo, A, nc);
+    const int side = n < 0 ? -1 : rn.hi_wall ? 1 : 0;
+    const long long cL = cell(nc, t), cLm = cell(nc, rt.km), cLp = cell(nc, rt.kp);
+    T fb[Q], gb[Q], ob[Q], yb[Q];
+    APt<T> s, B;
+    T fsum = 0;
+#pragma unroll
+    for (int q = 0; q < Q; q++) ob[q] = yb[q] = T(0);
+    if (side == 0) {
+        const int nR = rn.kp;
+        const long long cR = cell(nR, t), cRm = cell(nR, rt.km), cRp = cell(nR, rt.kp);
+        const T wL = rn.wL, wR = rn.wR, k = h * rn.invd;
+        const T Lm = h * wL * em, Lp = h * wL * ep, L0 = h * wL * e0, Rm = h * wR * em, Rp = h * wR * ep, R0 = h * wR * e0;
+        const T kL = Pr.dt * recip(rn.d), kR = Pr.dt * recip(rec<T>(I, geo, A, nR).d);
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const int nq = ca(q, A), tq = ca(q, 1 - A);
+            const T cl = wL + T(nq) * k - T(tq) * L0, cr = wR - T(nq) * k - T(tq) * R0;
+            const T *Pf = P.fbp + q * N, *Pg = P.gbp + q * N;
+            T vf = cl * Pf[cL] + cr * Pf[cR], vg = cl * Pg[cL] + cr * Pg[cR];
+            if (tq) {
+                const T sg = T(-tq);
+                vf += sg * (Lm * Pf[cLm] + Lp * Pf[cLp] + Rm * Pf[cRm] + Rp * Pf[cRp]);
+                vg += sg * (Lm * Pg[cLm] + Lp * Pg[cLp] + Rm * Pg[cRm] + Rp * Pg[cRp]);
+            }
+            fb[q] = vf;
+            gb[q] = vg;
+            if (nq) {   // the flux enters J_L with + and J_R with -; J-bar = -dt/|V| x-bar
+                ob[q] = T(nq) * (kR * Ad.xf[q * N + cR] - kL * Ad.xf[q * N + cL]);
+                yb[q] = T(nq) * (kR * Ad.xg[q * N + cR] - kL * Ad.xg[q * N + cL]);
+                fsum += vf * ob[q];
+            }
+        }
+        s.mu = wL * P.mu[cL] + wR * P.mu[cR];
+        s.lmu = wL * P.lapmu[cL] + wR * P.lapmu[cR];
+        s.gmx = wL * P.gmux[cL] + wR * P.gmux[cR];
+        s.gmy = wL * P.gmuy[cL] + wR * P.gmuy[cR];
+        s.gfx = wL * P.gphix[cL] + wR * P.gphix[cR];
+        s.gfy = wL * P.gphiy[cL] + wR * P.gphiy[cR];
+        s.gpx = wL * P.gpx[cL] + wR * P.gpx[cR];
+        s.gpy = wL * P.gpy[cL] + wR * P.gpy[cR];
+    } else {
+        // wall face: Taylor reconstruction of the outgoing and parallel directions,
+        // bounce-back of the incoming ones
+        const long long cnm = cell(rn.km, t), cnp = cell(rn.kp, t);
+        const T half = T(0.5) * rn.d, kc = Pr.dt * recip(rn.d);
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            if (ca(q, A) * side < 0) continue;
+            const T off = T(side) * half - h * T(ca(q, A)), ht = h * T(ca(q, 1 - A));
+            const T *Pf = P.fbp + q * N, *Pg = P.gbp + q * N;
+            const T bf = Pf[cL], bg = Pg[cL];
+            fb[q] = bf + off * (rn.e1m * Pf[cnm] + rn.e10 * bf + rn.e1p * Pf[cnp]) - ht * (em * Pf[cLm] + e0 * bf + ep * Pf[cLp]);
+            gb[q] = bg + off * (rn.e1m * Pg[cnm] + rn.e10 * bg + rn.e1p * Pg[cnp]) - ht * (em * Pg[cLm] + e0 * bg + ep * Pg[cLp]);
+            if (ca(q, A) * side > 0) {   // carries its own flux and its opposite's
+                const int o = opp(q);
+                ob[q] = kc * (Ad.xf[o * N + cL] - Ad.xf[q * N + cL]);
+                yb[q] = kc * (Ad.xg[o * N + cL] - Ad.xg[q * N + cL]);
+                fsum += fb[q] * ob[q];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            if (ca(q, A) * side < 0) {
+                fb[q] = fb[opp(q)];
+                gb[q] = gb[opp(q)];
+            }
+        }
+        s.mu = P.mu[cL];
+        s.lmu = P.lapmu[cL];
+        s.gmx = A == 0 ? T(0) : P.gmux[cL];
+        s.gmy = A == 1 ? T(0) : P.gmuy[cL];
+        s.gfx = A == 0 ? T(0) : P.gphix[cL];
+        s.gfy = A == 1 ? T(0) : P.gphiy[cL];
+        s.gpx = A == 0 ? T(0) : P.gpx[cL];
+        s.gpy = A == 1 ? T(0) : P.gpy[cL];
+    }
+    // face macros (Eq. conservedVariable with h)
+    const PtC<T> &C = facec<T>(I);
+    T sf = 0, mx = 0, my = 0;
+    s.phi = 0;
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        s.phi += gb[q];
+        sf += fb[q];
+        if (cx(q)) mx += T(cx(q)) * fb[q];
+        if (cy(q)) my += T(cy(q)) * fb[q];
+    }
+    const T rho = Pr.rhoB + Pr.drho * (s.phi - Pr.phiB), r3 = T(3) * recip(rho);
+    s.ux = (mx + C.kf * (-s.phi * s.gmx + (rho - Pr.rho_ref) * Pr.gxa)) * r3;
+    s.uy = (my + C.kf * (-s.phi * s.gmy + (rho - Pr.rho_ref) * Pr.gya)) * r3;
+    if (side != 0) s.ux = s.uy = T(0);
+    s.p = sf + C.kp1 * (s.ux * s.gfx + s.uy * s.gfy) - C.kp2 * rho * s.lmu;
+    const T a = point_adj<T, A>(I, s, ob, yb, fsum, side != 0, B, lam);
+    // gifts: bar f_q gets a ob_q + p-bar + xi_q . m-bar, bar g_q gets ga yb_q + phi-bar;
+    // a wall's incoming bars are copies of the outgoing ones
+    T *F = Ad.face[A];
+    const long long NF = Ad.NF, at = n < 0 ? low_face(I, N, A, t) : cL;
+    const T two = side != 0 ? T(2) : T(1);
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int q = fset<A>(k);
+        const bool in = ca(q, A) * side < 0;
+        const T m = T(cx(q)) * B.ux + T(cy(q)) * B.uy;
+        F[(AF + k) * NF + at] = in ? T(0) : a * ob[q] + two * B.p + m;
+        F[(AG + k) * NF + at] = in ? T(0) : C.ga * yb[q] + two * B.phi;
+    }
+    F[AS * NF + at] = B.p;
+    F[AM * NF + at] = A == 0 ? B.uy : B.ux;
+    F[AP * NF + at] = B.phi;
+    const bool wx = side != 0 && A == 0, wy = side != 0 && A == 1;   // aux normal to a wall: not the cell's
+    const T v[8] = {B.mu, B.lmu, wx ? T(0) : B.gmx, wy ? T(0) : B.gmy, wx ? T(0) : B.gfx, wy ? T(0) : B.gfy,
+                    wx ? T(0) : B.gpx, wy ? T(0) : B.gpy};
+#pragma unroll
+    for (int k = 0; k < 8; k++) F[(AX + k) * NF + at] = v[k];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) ka_face(const InstDev *__restrict__ insts, const AdjSeg *__restrict__ segs, int n_seg,
+                                               const AxisRecT<T> *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
+{
+    const int sg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (sg >= n_seg) return;
+    const AdjSeg g = segs[sg];
+    const InstDev &I = insts[g.inst];
+    const int i = g.i + (threadIdx.x & 31);
+    T lam = 0;
+    if (i < I.nx) {
+        if (g.axis == 0) face_of<T, 0>(I, geo, P, Ad, i, g.j, lam);
+        else face_of<T, 1>(I, geo, P, Ad, g.j, i, lam);
+    }
+    slot_add(Ad.lam_face + sg, lam);
+}
+
+// What the faces of axis A give the bar values p of one kind (0 f, 1 g) and four of
+// the aux fields (0: mu, lap mu, grad mu; 1: grad phi, grad p) of a cell at position
+// n of that axis and t of the other: the transpose of the reconstruction.  With T = (interpolation weight) E + (weight) W of the cell's
+// high and low face values, an interior cell gets T + h xi_n (E - W) / distance
+// - h xi_t (e0 T + e1m T of the next row + e1p T of the row before).
+template <typename T, int A, int KIND>
+__device__ __forceinline__ void gather(const InstDev &I, const AxisRecT<T> *__restrict__ geo, const AdjPlanes<T> &Ad, int n, int t,
+                                       T (&p)[Q], T (&x)[4])
+{
+    const long long N = Ad.N, NF = Ad.NF;
+    const T h = par<T>(I).h;
+    const T *F = Ad.face[A];
+    auto cell = [&](int nn, int tt) -> long long { return A == 0 ? cell_of(I, nn, tt) : cell_of(I, tt, nn); };
+    const AxisRecT<T> &rn = rec<T>(I, geo, A, n), &rt = rec<T>(I, geo, 1 - A, t);
+    const int km = rn.km, kp = rn.kp;
+    const bool lo = rn.lo_wall, hi = rn.hi_wall;
+    const AxisRecT<T> &rm = rec<T>(I, geo, A, km), &rp = rec<T>(I, geo, A, kp);
+    // weights of the high (E) and low (W) face; a wall's face is the cell's alone
+    const T aE = hi ? T(1) : rn.wL, aW = lo ? T(1) : rm.wR;
+    const T kE = hi ? T(0) : h * rn.invd, kW = lo ? T(0) : h * rm.invd;
+    const long long E0 = cell(n, t), W0 = lo ? low_face(I, N, A, t) : cell(km, t);
+    // the rows whose tangential derivative reads this cell
+    const bool hm = rt.km != t, hp = rt.kp != t;
+    const long long Em = cell(n, rt.km), Ep = cell(n, rt.kp);
+    const long long Wm = lo ? low_face(I, N, A, rt.km) : cell(km, rt.km), Wp = lo ? low_face(I, N, A, rt.kp) : cell(km, rt.kp);
+    const T e0 = h * (rt.e10 + (hm ? T(0) : rt.e1m) + (hp ? T(0) : rt.e1p));
+    const T em = hp ? h * rec<T>(I, geo, 1 - A, rt.kp).e1m : T(0);   // the next row's low neighbour
+    const T ep = hm ? h * rec<T>(I, geo, 1 - A, rt.km).e1p : T(0);   // the row before's high neighbour
+    auto at = [&](int pl, long long e, long long w) -> T { return aE * F[pl * NF + e] + aW * F[pl * NF + w]; };
+    auto tang = [&](int pl, T c0) -> T { return e0 * c0 + em * at(pl, Ep, Wp) + ep * at(pl, Em, Wm); };
+    // wall terms of direction q: the normal derivative of the wall's cell reads it
+    // and its inner neighbour
+    const bool nearw = lo || hi || rm.lo_wall || rp.hi_wall;
+    auto normal = [&](int pl, int xn) -> T {
+        T v = T(xn) * (kE * F[pl * NF + E0] - kW * F[pl * NF + W0]);
+        if (nearw) {
+            if (hi) v += (T(0.5) * rn.d - h * T(xn)) * rn.e10 * F[pl * NF + E0];
+            else if (rp.hi_wall) v += (T(0.5) * rp.d - h * T(xn)) * rp.e1m * F[pl * NF + cell(kp, t)];
+            if (lo) v += (T(-0.5) * rn.d - h * T(xn)) * rn.e10 * F[pl * NF + W0];
+            else if (rm.lo_wall) v += (T(-0.5) * rm.d - h * T(xn)) * rm.e1p * F[pl * NF + low_face(I, N, A, t)];
+        }
+        return v;
+    };
+    constexpr int F0 = KIND == 0 ? AF : AG;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const int q = fset<A>(k), xn = ca(q, A), xt = ca(q, 1 - A);
+        const T c = at(F0 + k, E0, W0);
+        p[q] = c + normal(F0 + k, xn);
+        if (xt) p[q] -= T(xt) * tang(F0 + k, c);
+    }
+    constexpr int tp = A == 0 ? 2 : 1, tn = A == 0 ? 4 : 3;   // along the face
+    if (KIND == 0) {
+        const T cS = at(AS, E0, W0), cM = at(AM, E0, W0);
+        const T nS = cS + normal(AS, 0), nM = cM + normal(AM, 0), yS = tang(AS, cS), yM = tang(AM, cM);
+        p[0] = nS;
+        p[tp] = (nS + nM) - (yS + yM);
+        p[tn] = (nS - nM) + (yS - yM);
+    } else {
+        const T cP = at(AP, E0, W0), nP = cP + normal(AP, 0), yP = tang(AP, cP);
+        p[0] = nP;
+        p[tp] = nP - yP;
+        p[tn] = nP + yP;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) x[k] = at(AX + 4 * KIND + k, E0, W0);
+}
+
+// bar-plus at the cell centre (Eq. relations1) after its faces, and the update
+// x_new = 4/3 bar-plus - 1/3 x - dt/|V| J (Eqs. relations2, updatef).  A warp per
+// run of 32 cells, or (SPLIT) a block: its four warps gather the two kinds from the
+// two axes, then one of them (another one in the next block, so that the FP64 work of
+// an SM's blocks spreads over its sub-partitions) transposes the point.  The split
+// shortens the longest path (FP64 48x96: 43 -> 31 us), and leaves three of four warps
+// without work at the end (FP32 256x512: 34 -> 54 us): it is for meshes of few runs.
+template <typename T, bool SPLIT>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 && !SPLIT ? 4 : 2) ka_cell(const InstDev *__restrict__ insts,
+                                                                                 const AdjSeg *__restrict__ segs, int n_seg,
+                                                                                 const AxisRecT<T> *__restrict__ geo,
+                                                                                 Planes<T> P, AdjPlanes<T> Ad)
+{
+    __shared__ T Gs[SPLIT ? 2 : 1][2][Q][32], Xs[SPLIT ? 2 : 1][8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sg = SPLIT ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + warp;
+    if (sg >= n_seg) return;
+    const AdjSeg g = segs[sg];
+    const InstDev &I = insts[g.inst];
+    const int i = g.i + lane, j = g.j;
+    const bool own = i < I.nx;
+    T Gf[Q], Gg[Q], X[8];
+    if (own) {
+        T v[Q], x[4];
+        if constexpr (SPLIT) {
+            if (warp == 0) gather<T, 0, 0>(I, geo, Ad, i, j, v, x);
+            else if (warp == 1) gather<T, 0, 1>(I, geo, Ad, i, j, v, x);
+            else if (warp == 2) gather<T, 1, 0>(I, geo, Ad, j, i, v, x);
+            else gather<T, 1, 1>(I, geo, Ad, j, i, v, x);
+#pragma unroll
+            for (int q = 0; q < Q; q++) Gs[warp >> 1][warp & 1][q][lane] = v[q];
+#pragma unroll
+            for (int k = 0; k < 4; k++) Xs[warp >> 1][4 * (warp & 1) + k][lane] = x[k];
+        } else {
+            gather<T, 0, 0>(I, geo, Ad, i, j, Gf, x);
+            T y[4];
+            gather<T, 1, 0>(I, geo, Ad, j, i, v, y);
+#pragma unroll
+            for (int q = 0; q < Q; q++) Gf[q] += v[q];
+#pragma unroll
+            for (int k = 0; k < 4; k++) X[k] = x[k] + y[k];
+            gather<T, 0, 1>(I, geo, Ad, i, j, Gg, x);
+            gather<T, 1, 1>(I, geo, Ad, j, i, v, y);
+#pragma unroll
+            for (int q = 0; q < Q; q++) Gg[q] += v[q];
+#pragma unroll
+            for (int k = 0; k < 4; k++) X[4 + k] = x[k] + y[k];
+        }
+    }
+    if constexpr (SPLIT) {
+        __syncthreads();
+        if (warp != (int)(blockIdx.x & 3)) return;
+        if (own) {
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                Gf[q] = Gs[0][0][q][lane] + Gs[1][0][q][lane];
+                Gg[q] = Gs[0][1][q][lane] + Gs[1][1][q][lane];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; k++) X[k] = Xs[0][k][lane] + Xs[1][k][lane];
+        }
+    }
+    T lam = 0;
+    if (own) {
+        const long long c = cell_of(I, i, j), N = P.N;
+        APt<T> s, B;
+        s.phi = T(phi_val(P.phi[c]));
+        s.ux = P.ux[c];
+        s.uy = P.uy[c];
+        s.p = P.p[c];
+        s.mu = P.mu[c];
+        s.lmu = P.lapmu[c];
+        s.gmx = P.gmux[c];
+        s.gmy = P.gmuy[c];
+        s.gfx = P.gphix[c];
+        s.gfy = P.gphiy[c];
+        s.gpx = P.gpx[c];
+        s.gpy = P.gpy[c];
+        T pf[Q], pg[Q], xf[Q], xg[Q];
+        T fsum = 0;
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            xf[q] = Ad.xf[q * N + c];
+            xg[q] = Ad.xg[q * N + c];
+            pf[q] = T(4.0 / 3.0) * xf[q] + Gf[q];
+            pg[q] = T(4.0 / 3.0) * xg[q] + Gg[q];
+            fsum += P.f[q * N + c] * pf[q];
+        }
+        const T b = point_adj<T, -1>(I, s, pf, pg, fsum, false, B, lam);
+        // a p - x / 3 with p = 4/3 x + G and a = 1 - b: as an increment of x, so that
+        // a uniform adjoint passes the step unchanged (4/3, 1/3 and a rounded one by
+        // one would leave a bias that grows with the steps)
+        const T bg = cellc<T>(I).gb36;
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            Ad.af[q * N + c] = xf[q] + (Gf[q] - b * pf[q]);
+            Ad.ag[q * N + c] = xg[q] + (Gg[q] - bg * pg[q]);
+        }
+        T *const out[8] = {Ad.mu, Ad.lapmu, Ad.gmx, Ad.gmy, Ad.gfx, Ad.gfy, Ad.gpx, Ad.gpy};
+        const T v[8] = {B.mu, B.lmu, B.gmx, B.gmy, B.gfx, B.gfy, B.gpx, B.gpy};
+#pragma unroll
+        for (int k = 0; k < 8; k++) out[k][c] = X[k] + v[k];
+        Ad.phi[c] = B.phi;
+        Ad.p[c] = B.p;
+        Ad.ux[c] = B.ux;
+        Ad.uy[c] = B.uy;
+    }
+    slot_add(Ad.lam_cell + sg, lam);
+}
 
 template <typename T>
 struct PtBar {
@@ -134,450 +640,6 @@ __device__ __forceinline__ void pt_inv_adj(const ParT<T> &Pr, const Pt<T> &s, co
     sb.gry += cs2 * vb.cgy;
 }
 
-// transpose of tau_f(phi, rho) = 3 mu_mix(phi) / rho (Eqs. mixvis, kineticandmobility)
-template <typename T>
-__device__ __forceinline__ void tauf_adj(const ParT<T> &Pr, T phi, T rho, T taub, T &phib, T &rhob)
-{
-    const T K = Pr.muA * Pr.muB * (Pr.phiA - Pr.phiB);
-    const T den = (phi - Pr.phiB) * Pr.muB + (Pr.phiA - phi) * Pr.muA;
-    const T mu = K / den;
-    phib += taub * T(3) / rho * (-K * (Pr.muB - Pr.muA) / (den * den));
-    rhob -= taub * T(3) * mu / (rho * rho);
-}
-
-// Face of axis A: forward face macros and originals (as face_originals) and
-// their transpose.  Ffb/Fgb are the adjoints of the flux values
-// (xi . e_A) phi_i |S| of the six flux-carrying directions; outputs are the
-// adjoints of the nine bar distributions of each kind and of the face aux.
-template <typename T, int A>
-__device__ void face_adj(const ParT<T> &Pr, const T (&fb)[Q], const T (&gb)[Q], const FaceAux<T> &ax, bool wall,
-                         int side, T area, const T (&Ffb)[6], const T (&Fgb)[6], T (&fbb)[Q], T (&gbb)[Q],
-                         FaceAux<T> &axb, T &lamb)
-{
-    const T cs2 = Cst<T>::cs2;
-    const T h = Pr.h;
-    T phi = 0, sf = 0, mx = 0, my = 0;
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        phi += gb[q];
-        sf += fb[q];
-        if (cx(q)) mx += T(cx(q)) * fb[q];
-        if (cy(q)) my += T(cy(q)) * fb[q];
-    }
-    Pt<T> s;
-    s.phi = phi;
-    s.rho = Pr.rhoB + Pr.drho * (phi - Pr.phiB);
-    const T irho = T(1) / s.rho;
-    s.Fx = -phi * ax.gmux + (s.rho - Pr.rho_ref) * Pr.gxa;
-    s.Fy = -phi * ax.gmuy + (s.rho - Pr.rho_ref) * Pr.gya;
-    s.grx = Pr.drho * ax.gphix;
-    s.gry = Pr.drho * ax.gphiy;
-    if (wall) {
-        s.ux = 0;
-        s.uy = 0;
-    } else {
-        s.ux = (T(3) * mx + T(0.5) * h * s.Fx) * irho;
-        s.uy = (T(3) * my + T(0.5) * h * s.Fy) * irho;
-    }
-    s.p = sf + T(0.5) * h * cs2 * (s.ux * s.grx + s.uy * s.gry - Pr.gamma * s.rho * Pr.lambda * ax.lapmu);
-    s.mu = ax.mu;
-    s.lapmu = ax.lapmu;
-    s.gpx = ax.gpx;
-    s.gpy = ax.gpy;
-    const T K = Pr.muA * Pr.muB * (Pr.phiA - Pr.phiB);
-    const T tf = T(3) * (K / ((phi - Pr.phiB) * Pr.muB + (Pr.phiA - phi) * Pr.muA)) / s.rho;
-    const T tg = Pr.tau_g;
-    const PtInv<T> v = pt_inv_p<T>(Pr, s);
-    const T r1 = T(1) / (T(2) * tf + h), r2 = T(1) / (T(2) * tg + h);
-    const T a1 = T(2) * tf * r1, b1 = h * r1, c1 = tf * h * r1;
-    const T a2 = T(2) * tg * r2, b2 = h * r2, c2 = tg * h * r2;
-    // adjoints of the originals
-    T fob[Q], gob[Q];
-#pragma unroll
-    for (int q = 0; q < Q; q++) { fob[q] = 0; gob[q] = 0; fbb[q] = 0; gbb[q] = 0; }
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int q = fset<A>(k);
-        const T vf = T(ca(q, A)) * area * Ffb[k], vg = T(ca(q, A)) * area * Fgb[k];
-        const int dst = (wall && ca(q, A) * side < 0) ? opp(q) : q;
-        fob[dst] += vf;
-        gob[dst] += vg;
-    }
-    PtBar<T> sb = ptbar_zero<T>();
-    InvBar<T> vb = invbar_zero<T>();
-    T a1b = 0, b1b = 0, c1b = 0;
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int q = fset<A>(k);
-        if (wall && ca(q, A) * side < 0) continue;
-        T feq, geq, F1, F2;
-        eq_src<T>(s, v, q, feq, geq, F1, F2);
-        fbb[q] += a1 * fob[q];
-        a1b += fb[q] * fob[q];
-        b1b += feq * fob[q];
-        c1b += F1 * fob[q];
-        gbb[q] += a2 * gob[q];
-        eq_src_adj<T>(s, v, q, b1 * fob[q], b2 * gob[q], c1 * fob[q], c2 * gob[q], sb, vb);
-    }
-    // a1 = 2 tf r1, b1 = h r1, c1 = tf h r1 with r1 = 1 / (2 tf + h)
-    const T taub = (a1b - b1b) * T(2) * h * r1 * r1 + c1b * h * h * r1 * r1;
-    pt_inv_adj<T>(Pr, s, v, vb, sb, lamb);
-    tauf_adj<T>(Pr, phi, s.rho, taub, sb.phi, sb.rho);
-    // p = sf + h/2 c_s^2 (u . grad rho - gamma rho lambda lap mu)
-    const T pk = T(0.5) * h * cs2 * sb.p;
-    const T sfb = sb.p;
-    T uxb = sb.ux + pk * s.grx, uyb = sb.uy + pk * s.gry;
-    T grxb = sb.grx + pk * s.ux, gryb = sb.gry + pk * s.uy;
-    T rhob = sb.rho - pk * Pr.gamma * Pr.lambda * ax.lapmu;
-    const T lapmub = sb.lapmu - pk * Pr.gamma * s.rho * Pr.lambda;
-    lamb -= pk * Pr.gamma * s.rho * ax.lapmu;
-    // u = (3 m + h/2 F) / rho
-    T mxb = 0, myb = 0, Fxb = sb.Fx, Fyb = sb.Fy;
-    if (!wall) {
-        mxb = T(3) * irho * uxb;
-        myb = T(3) * irho * uyb;
-        Fxb += T(0.5) * h * irho * uxb;
-        Fyb += T(0.5) * h * irho * uyb;
-        rhob -= (s.ux * uxb + s.uy * uyb) * irho;
-    }
-    // F = -phi grad mu + (rho - rho_ref) g
-    T phib = sb.phi - ax.gmux * Fxb - ax.gmuy * Fyb;
-    rhob += Pr.gxa * Fxb + Pr.gya * Fyb;
-    axb.gmux = -phi * Fxb;
-    axb.gmuy = -phi * Fyb;
-    axb.gphix = Pr.drho * grxb;
-    axb.gphiy = Pr.drho * gryb;
-    phib += Pr.drho * rhob;
-    axb.mu = sb.mu;
-    axb.lapmu = lapmub;
-    axb.gpx = sb.gpx;
-    axb.gpy = sb.gpy;
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        fbb[q] += sfb + T(cx(q)) * mxb + T(cy(q)) * myb;
-        gbb[q] += phib;
-    }
-}
-
-
-// sum over a block of one instance's per-thread parameter adjoint, added in FP64
-template <typename T>
-__device__ __forceinline__ void block_add_param(double *dst, T v)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(dst, (double)v);
-}
-
-// ---------------------------------------------------------------------------
-// faces: the transposes of the interior and wall faces (Eqs. fbar_h,
-// conservedVariable with h, original-function, microfluxf) for a TX x TY tile
-// per thread block.  Bar-plus, the face aux fields and the incoming adjoints
-// of the tile and its one-cell ring are staged in shared memory with
-// coalesced loads, the scatter of the face transposes goes into shared
-// accumulators, and each accumulator slot is added to global memory once.
-// Each cell owns its west and south faces, and the wall faces at the high end.
-// ---------------------------------------------------------------------------
-template <typename T>
-struct AdjTile {
-    static constexpr int W = TX + 2, H = TY + 2, A = W * H;   // region: columns -1..TX, rows -1..TY
-    static constexpr int NG = W + H;                          // geometry entries: columns, then rows
-    static constexpr int BP = 0, AUX = 2 * Q, XF = 2 * Q + 8, XG = 3 * Q + 8;
-    static constexpr int NIN = 4 * Q + 8;                     // staged planes
-    static constexpr int NACC = 2 * Q + 8;                    // accumulators: bar-plus, then aux adjoints
-    static constexpr size_t al(size_t v) { return (v + 15) / 16 * 16; }
-    static constexpr size_t o_in = al((sizeof(T) * 7 + sizeof(int) * 2) * NG);
-    static constexpr size_t o_acc = al(o_in + sizeof(T) * NIN * A);
-    static constexpr size_t bytes = al(o_acc + sizeof(T) * NACC * A);
-    static __device__ __forceinline__ int ri(int x, int y) { return (y + 1) * W + (x + 1); }
-    static __device__ __forceinline__ int ex(int x) { return x + 1; }
-    static __device__ __forceinline__ int ey(int y) { return W + y + 1; }
-};
-
-template <typename T>
-struct AdjTileView {
-    using AT = AdjTile<T>;
-    const T *ga;     // [7][NG]: d, e1m, e10, e1p, wL, wR, invd
-    const int *gf;   // [NG] flags: 1 low neighbour, 2 high neighbour, 4 low wall, 8 high wall
-    const T *in;     // [NIN][A]
-    T *acc;          // [NACC][A]
-    __device__ __forceinline__ T g(int k, int e) const { return ga[k * AT::NG + e]; }
-    __device__ __forceinline__ T v(int plane, int r) const { return in[plane * AT::A + r]; }
-    __device__ __forceinline__ void add(int plane, int r, T val) const { atomicAdd(acc + plane * AT::A + r, val); }
-};
-
-template <typename T, int A>
-__device__ void interior_face_adj_t(const ParT<T> &Pr, const AdjTileView<T> &V, int xL, int yL, int xR, int yR, T &lamb)
-{
-    using AT = AdjTile<T>;
-    const int rL = AT::ri(xL, yL), rR = AT::ri(xR, yR);
-    const int en = A == 0 ? AT::ex(xL) : AT::ey(yL);     // normal axis: the high face of L
-    const int et = A == 0 ? AT::ey(yL) : AT::ex(xL);     // tangential axis
-    const T wL = V.g(4, en), wR = V.g(5, en), invd = V.g(6, en);
-    const T em = V.g(1, et), e0 = V.g(2, et), ep = V.g(3, et);
-    const T area = V.g(0, et);
-    const int ft = V.gf[et], tstep = A == 0 ? AT::W : 1;
-    const int tm = (ft & 1) ? -tstep : 0, tp = (ft & 2) ? tstep : 0;   // a wall ghost is the cell itself
-    const T h = Pr.h;
-    T fb[Q], gb[Q];
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-#pragma unroll
-        for (int kind = 0; kind < 2; kind++) {
-            const int pl = AT::BP + kind * Q + q;
-            const T bL = V.v(pl, rL), bR = V.v(pl, rR);
-            const T tL = em * V.v(pl, rL + tm) + e0 * bL + ep * V.v(pl, rL + tp);
-            const T tR = em * V.v(pl, rR + tm) + e0 * bR + ep * V.v(pl, rR + tp);
-            (kind == 0 ? fb : gb)[q] = (wL * bL + wR * bR) - h * (T(ca(q, A)) * ((bR - bL) * invd) + T(ca(q, 1 - A)) * (wL * tL + wR * tR));
-        }
-    }
-    FaceAux<T> ax;
-    ax.mu = wL * V.v(AT::AUX + 0, rL) + wR * V.v(AT::AUX + 0, rR);
-    ax.lapmu = wL * V.v(AT::AUX + 1, rL) + wR * V.v(AT::AUX + 1, rR);
-    ax.gmux = wL * V.v(AT::AUX + 2, rL) + wR * V.v(AT::AUX + 2, rR);
-    ax.gmuy = wL * V.v(AT::AUX + 3, rL) + wR * V.v(AT::AUX + 3, rR);
-    ax.gpx = wL * V.v(AT::AUX + 4, rL) + wR * V.v(AT::AUX + 4, rR);
-    ax.gpy = wL * V.v(AT::AUX + 5, rL) + wR * V.v(AT::AUX + 5, rR);
-    ax.gphix = wL * V.v(AT::AUX + 6, rL) + wR * V.v(AT::AUX + 6, rR);
-    ax.gphiy = wL * V.v(AT::AUX + 7, rL) + wR * V.v(AT::AUX + 7, rR);
-    // the flux value enters J_L with + and J_R with -; J-bar = -dt/|V| x-bar
-    const T dtvL = Pr.dt / (V.g(0, AT::ex(xL)) * V.g(0, AT::ey(yL)));
-    const T dtvR = Pr.dt / (V.g(0, AT::ex(xR)) * V.g(0, AT::ey(yR)));
-    T Ffb[6], Fgb[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int q = fset<A>(k);
-        Ffb[k] = dtvR * V.v(AT::XF + q, rR) - dtvL * V.v(AT::XF + q, rL);
-        Fgb[k] = dtvR * V.v(AT::XG + q, rR) - dtvL * V.v(AT::XG + q, rL);
-    }
-    T fbb[Q], gbb[Q];
-    FaceAux<T> axb;
-    face_adj<T, A>(Pr, fb, gb, ax, false, 0, area, Ffb, Fgb, fbb, gbb, axb, lamb);
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-#pragma unroll
-        for (int kind = 0; kind < 2; kind++) {
-            const T bb = (kind == 0 ? fbb : gbb)[q];
-            const int pl = kind * Q + q;
-            const T k1 = h * T(ca(q, A)) * invd;
-            V.add(pl, rL, (wL + k1) * bb);
-            V.add(pl, rR, (wR - k1) * bb);
-            if (ca(q, 1 - A)) {
-                const T kt = -h * T(ca(q, 1 - A)) * bb;
-                V.add(pl, rL + tm, kt * wL * em);
-                V.add(pl, rL, kt * wL * e0);
-                V.add(pl, rL + tp, kt * wL * ep);
-                V.add(pl, rR + tm, kt * wR * em);
-                V.add(pl, rR, kt * wR * e0);
-                V.add(pl, rR + tp, kt * wR * ep);
-            }
-        }
-    }
-    const T vals[8] = {axb.mu, axb.lapmu, axb.gmux, axb.gmuy, axb.gpx, axb.gpy, axb.gphix, axb.gphiy};
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        V.add(2 * Q + k, rL, wL * vals[k]);
-        V.add(2 * Q + k, rR, wR * vals[k]);
-    }
-}
-
-template <typename T, int A>
-__device__ void wall_face_adj_t(const ParT<T> &Pr, const AdjTileView<T> &V, int x, int y, int side, T &lamb)
-{
-    using AT = AdjTile<T>;
-    const int r = AT::ri(x, y);
-    const int en = A == 0 ? AT::ex(x) : AT::ey(y), et = A == 0 ? AT::ey(y) : AT::ex(x);
-    const int fn = V.gf[en], ft = V.gf[et];
-    const int nstep = A == 0 ? 1 : AT::W, tstep = A == 0 ? AT::W : 1;
-    const int nmo = (fn & 1) ? -nstep : 0, npo = (fn & 2) ? nstep : 0;   // a wall ghost is the cell itself
-    const int tmo = (ft & 1) ? -tstep : 0, tpo = (ft & 2) ? tstep : 0;
-    const T h = Pr.h, half_d = T(0.5) * V.g(0, en);
-    const T nm = V.g(1, en), n0 = V.g(2, en), np = V.g(3, en);
-    const T tm = V.g(1, et), t0 = V.g(2, et), tp = V.g(3, et);
-    const T area = V.g(0, et);
-    T fb[Q], gb[Q];
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        if (ca(q, A) * side < 0) continue;
-        const T off = T(side) * half_d - h * T(ca(q, A));
-        const T ht = h * T(ca(q, 1 - A));
-#pragma unroll
-        for (int kind = 0; kind < 2; kind++) {
-            const int pl = AT::BP + kind * Q + q;
-            const T b = V.v(pl, r);
-            (kind == 0 ? fb : gb)[q] = b + off * (nm * V.v(pl, r + nmo) + n0 * b + np * V.v(pl, r + npo))
-                                     - ht * (tm * V.v(pl, r + tmo) + t0 * b + tp * V.v(pl, r + tpo));
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        if (ca(q, A) * side < 0) {
-            fb[q] = fb[opp(q)];
-            gb[q] = gb[opp(q)];
-        }
-    }
-    FaceAux<T> ax;
-    ax.mu = V.v(AT::AUX + 0, r);
-    ax.lapmu = V.v(AT::AUX + 1, r);
-    ax.gmux = (A == 0) ? T(0) : V.v(AT::AUX + 2, r);
-    ax.gmuy = (A == 1) ? T(0) : V.v(AT::AUX + 3, r);
-    ax.gpx = (A == 0) ? T(0) : V.v(AT::AUX + 4, r);
-    ax.gpy = (A == 1) ? T(0) : V.v(AT::AUX + 5, r);
-    ax.gphix = (A == 0) ? T(0) : V.v(AT::AUX + 6, r);
-    ax.gphiy = (A == 1) ? T(0) : V.v(AT::AUX + 7, r);
-    // the flux value enters J_c with the sign of the side
-    const T dtv = Pr.dt / (V.g(0, AT::ex(x)) * V.g(0, AT::ey(y)));
-    T Ffb[6], Fgb[6];
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-        const int q = fset<A>(k);
-        Ffb[k] = -T(side) * dtv * V.v(AT::XF + q, r);
-        Fgb[k] = -T(side) * dtv * V.v(AT::XG + q, r);
-    }
-    T fbb[Q], gbb[Q];
-    FaceAux<T> axb;
-    face_adj<T, A>(Pr, fb, gb, ax, true, side, area, Ffb, Fgb, fbb, gbb, axb, lamb);
-    // incoming bars were copies of the opposite outgoing ones
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        if (ca(q, A) * side < 0) {
-            fbb[opp(q)] += fbb[q];
-            gbb[opp(q)] += gbb[q];
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < Q; q++) {
-        if (ca(q, A) * side < 0) continue;
-        const T off = T(side) * half_d - h * T(ca(q, A));
-        const T ht = h * T(ca(q, 1 - A));
-#pragma unroll
-        for (int kind = 0; kind < 2; kind++) {
-            const T bb = (kind == 0 ? fbb : gbb)[q];
-            const int pl = kind * Q + q;
-            V.add(pl, r, (T(1) + off * n0 - ht * t0) * bb);
-            V.add(pl, r + nmo, off * nm * bb);
-            V.add(pl, r + npo, off * np * bb);
-            V.add(pl, r + tmo, -ht * tm * bb);
-            V.add(pl, r + tpo, -ht * tp * bb);
-        }
-    }
-    V.add(2 * Q + 0, r, axb.mu);
-    V.add(2 * Q + 1, r, axb.lapmu);
-    if (A == 1) { V.add(2 * Q + 2, r, axb.gmux); V.add(2 * Q + 4, r, axb.gpx); V.add(2 * Q + 6, r, axb.gphix); }
-    if (A == 0) { V.add(2 * Q + 3, r, axb.gmuy); V.add(2 * Q + 5, r, axb.gpy); V.add(2 * Q + 7, r, axb.gphiy); }
-}
-
-// update and faces of a tile: x_new = 4/3 bar-plus - 1/3 x - dt/|V| J
-// (Eqs. relations2, updatef)
-template <typename T>
-__global__ void __launch_bounds__(TX *TY, sizeof(T) == 4 ? 2 : 1)
-    ka_face_t(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, const AxisRecT<T> *__restrict__ geo,
-              Planes<T> P, AdjPlanes<T> Ad)
-{
-    using AT = AdjTile<T>;
-    extern __shared__ __align__(16) unsigned char smem[];
-    T *ga = (T *)smem;
-    int *gg = (int *)(ga + 7 * AT::NG), *gf = gg + AT::NG;
-    T *in = (T *)(smem + AT::o_in);
-    T *acc = (T *)(smem + AT::o_acc);
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
-    const ParT<T> &Pr = par<T>(I);
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    const int i0 = t.y, j0 = t.z;
-    const long long N = P.N;
-    // geometry of the region's columns and rows (wrapped on a periodic axis,
-    // -1 outside the domain)
-    for (int e = tid; e < AT::NG; e += TX * TY) {
-        const bool isx = e < AT::W;
-        const int n = isx ? I.nx : I.ny;
-        int g = isx ? i0 + e - 1 : j0 + (e - AT::W) - 1;
-        if ((isx ? I.bcx : I.bcy) == 0) {
-            while (g < 0) g += n;
-            while (g >= n) g -= n;
-        } else if (g < 0 || g >= n) {
-            g = -1;
-        }
-        T v[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-        int fl = 0;
-        if (g >= 0) {
-            const AxisRecT<T> &R = geo[(isx ? I.gx_off : I.gy_off) + g];
-            v[0] = R.d; v[1] = R.e1m; v[2] = R.e10; v[3] = R.e1p; v[4] = R.wL; v[5] = R.wR; v[6] = R.invd;
-            fl = (R.km == g ? 0 : 1) | (R.kp == g ? 0 : 2) | (R.lo_wall ? 4 : 0) | (R.hi_wall ? 8 : 0);
-        }
-#pragma unroll
-        for (int k = 0; k < 7; k++) ga[k * AT::NG + e] = v[k];
-        gg[e] = g;
-        gf[e] = fl;
-    }
-    __syncthreads();
-    // staged planes; the accumulators start from the update's 4/3 x-bar in the
-    // tile's own cells, whose new x-bar (-1/3 x-bar) is written here
-    for (int r = tid; r < AT::A; r += TX * TY) {
-        const int x = r % AT::W - 1, y = r / AT::W - 1;
-        const int gi = gg[AT::ex(x)], gj = gg[AT::ey(y)];
-        const bool inside = gi >= 0 && gj >= 0;
-        const bool own = x >= 0 && x < TX && y >= 0 && y < TY && i0 + x < I.nx && j0 + y < I.ny;
-        const long long c = inside ? cell_of(I, gi, gj) : 0;
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            const T xf = inside ? Ad.xf[q * N + c] : T(0), xg = inside ? Ad.xg[q * N + c] : T(0);
-            in[(AT::BP + q) * AT::A + r] = inside ? P.fbp[q * N + c] : T(0);
-            in[(AT::BP + Q + q) * AT::A + r] = inside ? P.gbp[q * N + c] : T(0);
-            in[(AT::XF + q) * AT::A + r] = xf;
-            in[(AT::XG + q) * AT::A + r] = xg;
-            acc[q * AT::A + r] = own ? T(4.0 / 3.0) * xf : T(0);
-            acc[(Q + q) * AT::A + r] = own ? T(4.0 / 3.0) * xg : T(0);
-            if (own) {
-                Ad.af[q * N + c] = -T(1.0 / 3.0) * xf;
-                Ad.ag[q * N + c] = -T(1.0 / 3.0) * xg;
-            }
-        }
-        const T *aux[8] = {P.mu, P.lapmu, P.gmux, P.gmuy, P.gpx, P.gpy, P.gphix, P.gphiy};
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            in[(AT::AUX + k) * AT::A + r] = inside ? aux[k][c] : T(0);
-            acc[(2 * Q + k) * AT::A + r] = T(0);
-        }
-    }
-    __syncthreads();
-    const AdjTileView<T> V{ga, gf, in, acc};
-    T lamb = 0;
-    {
-        const int x = threadIdx.x, y = threadIdx.y;
-        if (i0 + x < I.nx && j0 + y < I.ny) {
-            const int fx = gf[AT::ex(x)], fy = gf[AT::ey(y)];
-            if (fx & 4) wall_face_adj_t<T, 0>(Pr, V, x, y, -1, lamb);
-            else interior_face_adj_t<T, 0>(Pr, V, x - 1, y, x, y, lamb);
-            if (fx & 8) wall_face_adj_t<T, 0>(Pr, V, x, y, +1, lamb);
-            if (fy & 4) wall_face_adj_t<T, 1>(Pr, V, x, y, -1, lamb);
-            else interior_face_adj_t<T, 1>(Pr, V, x, y - 1, x, y, lamb);
-            if (fy & 8) wall_face_adj_t<T, 1>(Pr, V, x, y, +1, lamb);
-        }
-    }
-    __syncthreads();
-    // every accumulator slot of a cell of the domain, added once
-    T *const aux_out[8] = {Ad.mu, Ad.lapmu, Ad.gmx, Ad.gmy, Ad.gpx, Ad.gpy, Ad.gfx, Ad.gfy};
-    for (int r = tid; r < AT::A; r += TX * TY) {
-        const int gi = gg[AT::ex(r % AT::W - 1)], gj = gg[AT::ey(r / AT::W - 1)];
-        if (gi < 0 || gj < 0) continue;
-        const long long c = cell_of(I, gi, gj);
-#pragma unroll
-        for (int k = 0; k < 2 * Q; k++) {
-            const T v = acc[k * AT::A + r];
-            if (v != T(0)) atomicAdd(Ad.bp + k * N + c, v);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const T v = acc[(2 * Q + k) * AT::A + r];
-            if (v != T(0)) atomicAdd(aux_out[k] + c, v);
-        }
-    }
-    block_add_param(Ad.pk + 2 * t.x, lamb);
-}
-
-// ---------------------------------------------------------------------------
-// cells
-// ---------------------------------------------------------------------------
 // transpose of F = -phi grad mu + (rho - rho_ref) g and grad rho = drho grad phi
 template <typename T>
 __device__ __forceinline__ void force_adj(const ParT<T> &Pr, T phi, T gmx, T gmy, PtBar<T> &sb, T &gmxb, T &gmyb,
@@ -591,174 +653,180 @@ __device__ __forceinline__ void force_adj(const ParT<T> &Pr, T phi, T gmx, T gmy
     gfyb += Pr.drho * sb.gry;
 }
 
-// bar-plus at the cell centre (Eq. relations1) and its equilibria and sources
-template <typename T>
-__global__ void __launch_bounds__(TX *TY, sizeof(T) == 4 ? 2 : 1) ka_cell(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                  const AxisRec *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
-{
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
-    const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
-    T lamb = 0;
-    if (i < I.nx && j < I.ny) {
-        const long long c = cell_of(I, i, j);
-        const long long N = P.N;
-        Pt<T> s;
-        cell_point(I, P, c, P.gpx[c], P.gpy[c], s);
-        const PtInv<T> v = pt_inv_p<T>(Pr, s);
-        const T dt = Pr.dt, h = Pr.h, tf = s.tauf, tg = Pr.tau_g;
-        const T rf = T(1) / (T(2) * tf + dt), rg = T(1) / (T(2) * tg + dt);
-        const T af = (T(2) * tf - h) * rf, bf = T(3) * h * rf, cf = T(3) * tf * h * rf;
-        const T ag = (T(2) * tg - h) * rg, bg = T(3) * h * rg, cg = T(3) * tg * h * rg;
-        PtBar<T> sb = ptbar_zero<T>();
-        InvBar<T> vb = invbar_zero<T>();
-        T afb = 0, bfb = 0, cfb = 0;
-        // every input of the nine directions is loaded before any store, so
-        // that the loads are in flight together
-        T pf[Q], pg[Q], fv[Q], xa[Q], xg[Q];
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            pf[q] = Ad.bp[q * N + c];
-            pg[q] = Ad.bp[(Q + q) * N + c];
-            fv[q] = P.f[q * N + c];
-            xa[q] = Ad.af[q * N + c];
-            xg[q] = Ad.ag[q * N + c];
-        }
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            T feq, geq, Ff, Fg;
-            eq_src<T>(s, v, q, feq, geq, Ff, Fg);
-            afb += fv[q] * pf[q];
-            bfb += feq * pf[q];
-            cfb += Ff * pf[q];
-            eq_src_adj<T>(s, v, q, bf * pf[q], bg * pg[q], cf * pf[q], cg * pg[q], sb, vb);
-        }
-#pragma unroll
-        for (int q = 0; q < Q; q++) {
-            Ad.af[q * N + c] = xa[q] + af * pf[q];
-            Ad.ag[q * N + c] = xg[q] + ag * pg[q];
-        }
-        // af = (2 tf - h) rf, bf = 3 h rf, cf = 3 tf h rf, rf = 1 / (2 tf + dt)
-        const T taub = afb * T(3) * dt * rf * rf - bfb * T(6) * h * rf * rf + cfb * T(3) * h * dt * rf * rf;
-        pt_inv_adj<T>(Pr, s, v, vb, sb, lamb);
-        tauf_adj<T>(Pr, s.phi, s.rho, taub, sb.phi, sb.rho);
-        T gmxb = 0, gmyb = 0, gfxb = 0, gfyb = 0;
-        force_adj<T>(Pr, s.phi, P.gmux[c], P.gmuy[c], sb, gmxb, gmyb, gfxb, gfyb);
-        sb.phi += Pr.drho * sb.rho;
-        Ad.phi[c] += sb.phi;
-        Ad.mu[c] += sb.mu;
-        Ad.lapmu[c] += sb.lapmu;
-        Ad.gmx[c] += gmxb;
-        Ad.gmy[c] += gmyb;
-        Ad.gfx[c] += gfxb;
-        Ad.gfy[c] += gfyb;
-        Ad.gpx[c] += sb.gpx;
-        Ad.gpy[c] += sb.gpy;
-        Ad.p[c] = sb.p;
-        Ad.ux[c] = sb.ux;
-        Ad.uy[c] = sb.uy;
-    }
-    block_add_param(Ad.pk + 2 * t.x, lamb);
-}
-
 // Transpose of a three-point stencil along axis a: the sum over the cells whose
 // stencil reads cell (i, j), of their coefficient times the adjoint there.
 // KIND 0: first derivative (c1m, c10, c1p); 1: first derivative in difference
 // form (centre weight -(c1m + c1p)); 2: second derivative (c2m, c20, c2p);
 // 3: second derivative in difference form.
-template <int KIND>
-__device__ __forceinline__ double coef(const AxisRec &r, int which)
+template <typename T, int KIND>
+__device__ __forceinline__ T coef(const AxisRecT<T> &r, int which)
 {
-    const double m = (KIND < 2) ? r.c1m : r.c2m, p = (KIND < 2) ? r.c1p : r.c2p;
-    const double z = (KIND == 0) ? r.c10 : (KIND == 2) ? r.c20 : -(m + p);
+    const T m = (KIND < 2) ? r.c1m : r.c2m, p = (KIND < 2) ? r.c1p : r.c2p;
+    const T z = (KIND == 0) ? r.c10 : (KIND == 2) ? r.c20 : -(m + p);
     return which < 0 ? m : which > 0 ? p : z;
 }
 
 template <typename T, int KIND>
-__device__ __forceinline__ T stencil_t(const InstDev &I, const AxisRec *__restrict__ geo, const T *__restrict__ Ab,
+__device__ __forceinline__ T stencil_t(const InstDev &I, const AxisRecT<T> *__restrict__ geo, const T *__restrict__ Ab,
                                        int a, int i, int j)
 {
     const long long off = a == 0 ? I.gx_off : I.gy_off;
     const int k = a == 0 ? i : j;
-    const AxisRec &r = geo[off + k];
+    const AxisRecT<T> &r = geo[off + k];
     auto at = [&](int kk) -> T { return Ab[a == 0 ? cell_of(I, kk, j) : cell_of(I, i, kk)]; };
-    T s = T(coef<KIND>(r, 0)) * at(k);
-    if (r.km == k) s += T(coef<KIND>(r, -1)) * at(k);
-    else s += T(coef<KIND>(geo[off + r.km], +1)) * at(r.km);
-    if (r.kp == k) s += T(coef<KIND>(r, +1)) * at(k);
-    else s += T(coef<KIND>(geo[off + r.kp], -1)) * at(r.kp);
+    T s = coef<T, KIND>(r, 0) * at(k);
+    if (r.km == k) s += coef<T, KIND>(r, -1) * at(k);
+    else s += coef<T, KIND>(geo[off + r.km], +1) * at(r.km);
+    if (r.kp == k) s += coef<T, KIND>(r, +1) * at(k);
+    else s += coef<T, KIND>(geo[off + r.kp], -1) * at(r.kp);
     return s;
 }
 
-// p, u, F of the cell (Eqs. u, P), after the transpose of grad p
-template <typename T>
-__global__ void __launch_bounds__(TX *TY) ka_macro(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                   const AxisRec *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
+// Stencil transpose (see stencil_t) on a shared plane S of pitch W at entry e; st: the
+// step to the next position of the axis, r, rm, rp: the records of the position and of
+// its neighbours.
+template <typename T, int KIND>
+__device__ __forceinline__ T stencil_s(const T *S, int e, int st, const AxisRecT<T> &r, const AxisRecT<T> &rm, const AxisRecT<T> &rp,
+                                       bool hm, bool hp)
 {
+    T s = coef<T, KIND>(r, 0) * S[e];
+    s += hm ? coef<T, KIND>(rm, +1) * S[e - st] : coef<T, KIND>(r, -1) * S[e];
+    s += hp ? coef<T, KIND>(rp, -1) * S[e + st] : coef<T, KIND>(r, +1) * S[e];
+    return s;
+}
+
+// The rest of the step's transpose for a BX x BY tile per thread block, each on the
+// ring that the next one reads: grad p, then p, u, F (Eqs. u, P) on a 2-cell ring;
+// grad mu and lap mu, then mu = psi'(phi) - kappa lap(phi) (Eq. chemicalpotential) on
+// a 1-cell ring; grad phi and lap phi, then phi = sum g~ on the tile.  As three
+// kernels these took 14 + 7 + 11 us of a 256x512 FP32 step, most of it to add to planes
+// in memory one after the other.
+template <typename T, int BX, int BY, int NT>
+__global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
+                                              const AxisRecT<T> *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
+{
+    constexpr int W2 = BX + 4, A2 = W2 * (BY + 4), W1 = BX + 2, A1 = W1 * (BY + 2);
+    __shared__ T gmx[A2], gmy[A2], lmu[A2], gfx[A2], gfy[A2], lph[A1], phb[BX * BY];
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
-    T lamb = 0;
-    if (i < I.nx && j < I.ny) {
+    const int i0 = t.y, j0 = t.z, tid = threadIdx.x;
+    const long long N = P.N;
+    // global index of a position (-1 outside)
+    auto wrap = [](int g, int n, int bc) -> int {
+        if (bc == 0) {
+            while (g < 0) g += n;
+            while (g >= n) g -= n;
+            return g;
+        }
+        return g < 0 || g >= n ? -1 : g;
+    };
+    const T cs2 = Cst<T>::cs2, hdt = T(0.5) * Pr.dt;
+    T lamb = 0, kapb = 0;
+    for (int r = tid; r < A2; r += NT) {
+        const int x = r % W2 - 2, y = r / W2 - 2;
+        const int i = wrap(i0 + x, I.nx, I.bcx), j = wrap(j0 + y, I.ny, I.bcy);
+        if (i < 0 || j < 0) continue;
+        const bool own = x >= 0 && x < BX && y >= 0 && y < BY && i0 + x < I.nx && j0 + y < I.ny;
         const long long c = cell_of(I, i, j);
-        const long long N = P.N;
-        const T cs2 = Cst<T>::cs2;
-        const T hdt = T(0.5) * Pr.dt;
         const T pb = Ad.p[c] + stencil_t<T, 0>(I, geo, Ad.gpx, 0, i, j) + stencil_t<T, 0>(I, geo, Ad.gpy, 1, i, j);
         T uxb = Ad.ux[c], uyb = Ad.uy[c];
         const T phi = T(phi_val(P.phi[c]));
         const T rho = Pr.rhoB + Pr.drho * (phi - Pr.phiB);
         const T ux = P.ux[c], uy = P.uy[c];
         const T grx = Pr.drho * P.gphix[c], gry = Pr.drho * P.gphiy[c];
-        const T lmu = P.lapmu[c];
+        const T lm = P.lapmu[c];
         const T pk = hdt * cs2 * pb;
         // p = sum f + dt/2 c_s^2 (u . grad rho - gamma rho lambda lap mu)
-        const T sfb = pb;
         uxb += pk * grx;
         uyb += pk * gry;
         PtBar<T> sb = ptbar_zero<T>();
         sb.grx = pk * ux;
         sb.gry = pk * uy;
-        sb.rho = -pk * Pr.gamma * Pr.lambda * lmu;
-        const T lmub = -pk * Pr.gamma * rho * Pr.lambda;
-        lamb -= pk * Pr.gamma * rho * lmu;
+        sb.rho = -pk * Pr.gamma * Pr.lambda * lm;
         // u = (3 m + dt/2 F) / rho
-        const T mxb = T(3) * uxb / rho, myb = T(3) * uyb / rho;
-        sb.Fx = hdt * uxb / rho;
-        sb.Fy = hdt * uyb / rho;
-        sb.rho -= (ux * uxb + uy * uyb) / rho;
+        const T irho = recip(rho);
+        const T mxb = T(3) * uxb * irho, myb = T(3) * uyb * irho;
+        sb.Fx = hdt * uxb * irho;
+        sb.Fy = hdt * uyb * irho;
+        sb.rho -= (ux * uxb + uy * uyb) * irho;
         T gmxb = 0, gmyb = 0, gfxb = 0, gfyb = 0;
         force_adj<T>(Pr, phi, P.gmux[c], P.gmuy[c], sb, gmxb, gmyb, gfxb, gfyb);
-        sb.phi += Pr.drho * sb.rho;
+        gmx[r] = Ad.gmx[c] + gmxb;
+        gmy[r] = Ad.gmy[c] + gmyb;
+        lmu[r] = Ad.lapmu[c] - pk * Pr.gamma * rho * Pr.lambda;
+        gfx[r] = Ad.gfx[c] + gfxb;
+        gfy[r] = Ad.gfy[c] + gfyb;
+        if (own) {
+            lamb -= pk * Pr.gamma * rho * lm;
+            phb[y * BX + x] = Ad.phi[c] + (sb.phi + Pr.drho * sb.rho);
 #pragma unroll
-        for (int q = 0; q < Q; q++) Ad.af[q * N + c] += sfb + T(cx(q)) * mxb + T(cy(q)) * myb;
-        Ad.phi[c] += sb.phi;
-        Ad.gmx[c] += gmxb;
-        Ad.gmy[c] += gmyb;
-        Ad.gfx[c] += gfxb;
-        Ad.gfy[c] += gfyb;
-        Ad.lapmu[c] += lmub;
+            for (int q = 0; q < Q; q++) Ad.af[q * N + c] += pb + T(cx(q)) * mxb + T(cy(q)) * myb;
+        }
     }
-    block_add_param(Ad.pk + 2 * t.x, lamb);
+    __syncthreads();
+    for (int r = tid; r < A1; r += NT) {
+        const int x = r % W1 - 1, y = r / W1 - 1;
+        const int i = wrap(i0 + x, I.nx, I.bcx), j = wrap(j0 + y, I.ny, I.bcy);
+        if (i < 0 || j < 0) continue;
+        const bool own = x >= 0 && x < BX && y >= 0 && y < BY && i0 + x < I.nx && j0 + y < I.ny;
+        const long long c = cell_of(I, i, j);
+        const AxisRecT<T> &ax = rec<T>(I, geo, 0, i), &ay = rec<T>(I, geo, 1, j);
+        const AxisRecT<T> &axm = rec<T>(I, geo, 0, ax.km), &axp = rec<T>(I, geo, 0, ax.kp);
+        const AxisRecT<T> &aym = rec<T>(I, geo, 1, ay.km), &ayp = rec<T>(I, geo, 1, ay.kp);
+        const bool xm = !ax.lo_wall, xp = !ax.hi_wall, ym = !ay.lo_wall, yp = !ay.hi_wall;
+        const int e = (y + 2) * W2 + x + 2;
+        const T mub = Ad.mu[c] + stencil_s<T, 0>(gmx, e, 1, ax, axm, axp, xm, xp) + stencil_s<T, 0>(gmy, e, W2, ay, aym, ayp, ym, yp)
+                    + stencil_s<T, 2>(lmu, e, 1, ax, axm, axp, xm, xp) + stencil_s<T, 2>(lmu, e, W2, ay, aym, ayp, ym, yp);
+        lph[r] = -Pr.kappa * mub;
+        if (own) {
+            const phi_t<T> p0 = P.phi[c];
+            const T phi = T(phi_val(p0));
+            const T a = phi - Pr.phiA, b = phi - Pr.phiB, m = phi - T(0.5) * (Pr.phiA + Pr.phiB);
+            const T d2psi = T(4) * Pr.beta * (b * m + a * m + a * b);
+            const T lap = (ax.c2m * phi_sub(P.phi[cell_of(I, ax.km, j)], p0) + ax.c2p * phi_sub(P.phi[cell_of(I, ax.kp, j)], p0))
+                        + (ay.c2m * phi_sub(P.phi[cell_of(I, i, ay.km)], p0) + ay.c2p * phi_sub(P.phi[cell_of(I, i, ay.kp)], p0));
+            phb[y * BX + x] += d2psi * mub;
+            kapb -= lap * mub;
+        }
+    }
+    __syncthreads();
+    for (int r = tid; r < BX * BY; r += NT) {
+        const int x = r % BX, y = r / BX, i = i0 + x, j = j0 + y;
+        if (i >= I.nx || j >= I.ny) continue;
+        const long long c = cell_of(I, i, j);
+        const AxisRecT<T> &ax = rec<T>(I, geo, 0, i), &ay = rec<T>(I, geo, 1, j);
+        const AxisRecT<T> &axm = rec<T>(I, geo, 0, ax.km), &axp = rec<T>(I, geo, 0, ax.kp);
+        const AxisRecT<T> &aym = rec<T>(I, geo, 1, ay.km), &ayp = rec<T>(I, geo, 1, ay.kp);
+        const bool xm = !ax.lo_wall, xp = !ax.hi_wall, ym = !ay.lo_wall, yp = !ay.hi_wall;
+        const int e2 = (y + 2) * W2 + x + 2, e1 = (y + 1) * W1 + x + 1;
+        const T phib = phb[r] + stencil_s<T, 1>(gfx, e2, 1, ax, axm, axp, xm, xp) + stencil_s<T, 1>(gfy, e2, W2, ay, aym, ayp, ym, yp)
+                     + stencil_s<T, 3>(lph, e1, 1, ax, axm, axp, xm, xp) + stencil_s<T, 3>(lph, e1, W1, ay, aym, ayp, ym, yp);
+#pragma unroll
+        for (int q = 0; q < Q; q++) Ad.ag[q * N + c] += phib;
+    }
+    const int w = blockIdx.x * (NT / 32) + tid / 32;
+    slot_add(Ad.lam_macro + w, lamb);
+    slot_add(Ad.kap + w, kapb);
 }
 
-// mu = psi'(phi) - kappa lap(phi) (Eq. chemicalpotential), after the transposes
-// of grad mu and lap mu; writes the adjoint of lap(phi)
+// The initialisation's mu = psi'(phi) - kappa lap(phi) (Eq. chemicalpotential),
+// after the transposes of grad mu and lap mu; writes the adjoint of lap(phi)
 template <typename T>
-__global__ void __launch_bounds__(TX *TY) ka_mu(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                const AxisRec *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
+__global__ void __launch_bounds__(128) ka_mu(const InstDev *__restrict__ insts, const AdjSeg *__restrict__ segs, int n_seg,
+        const AxisRecT<T> *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
 {
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
+    const int sg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (sg >= n_seg) return;
+    const AdjSeg g = segs[sg];
+    const InstDev &I = insts[g.inst];
     const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
+    const int i = g.i + (threadIdx.x & 31), j = g.j;
     T kapb = 0;
-    if (i < I.nx && j < I.ny) {
+    if (i < I.nx) {
         const long long c = cell_of(I, i, j);
-        const AxisRec &ax = geo[I.gx_off + i];
-        const AxisRec &ay = geo[I.gy_off + j];
+        const AxisRecT<T> &ax = geo[I.gx_off + i];
+        const AxisRecT<T> &ay = geo[I.gy_off + j];
         const T mub = Ad.mu[c] + stencil_t<T, 0>(I, geo, Ad.gmx, 0, i, j) + stencil_t<T, 0>(I, geo, Ad.gmy, 1, i, j)
                     + stencil_t<T, 2>(I, geo, Ad.lapmu, 0, i, j) + stencil_t<T, 2>(I, geo, Ad.lapmu, 1, i, j);
         const phi_t<T> p0 = P.phi[c];
@@ -771,46 +839,44 @@ __global__ void __launch_bounds__(TX *TY) ka_mu(const InstDev *__restrict__ inst
         Ad.lapphi[c] = -Pr.kappa * mub;
         kapb = -lap * mub;
     }
-    block_add_param(Ad.pk + 2 * t.x + 1, kapb);
+    slot_add(Ad.kap0 + sg, kapb);
 }
 
-// phi = sum_i g~_i, after the transposes of grad phi and lap phi
+// The initialisation's phi, after the transposes of grad phi and lap phi: the
+// gradient with respect to the input field
 template <typename T>
-__global__ void __launch_bounds__(TX *TY) ka_phi(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                 const AxisRec *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad,
-                                                 double *phi0_out, const long long *__restrict__ dense0)
+__global__ void __launch_bounds__(128) ka_phi0(const InstDev *__restrict__ insts, const AdjSeg *__restrict__ segs, int n_seg,
+                                               const AxisRecT<T> *__restrict__ geo, AdjPlanes<T> Ad, double *phi0_out,
+                                               const long long *__restrict__ dense0)
 {
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
-    if (i >= I.nx || j >= I.ny) return;
+    const int sg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (sg >= n_seg) return;
+    const AdjSeg g = segs[sg];
+    const InstDev &I = insts[g.inst];
+    const int i = g.i + (threadIdx.x & 31), j = g.j;
+    if (i >= I.nx) return;
     const long long c = cell_of(I, i, j);
-    const long long N = P.N;
-    const T phib = Ad.phi[c] + stencil_t<T, 1>(I, geo, Ad.gfx, 0, i, j) + stencil_t<T, 1>(I, geo, Ad.gfy, 1, i, j)
-                 + stencil_t<T, 3>(I, geo, Ad.lapphi, 0, i, j) + stencil_t<T, 3>(I, geo, Ad.lapphi, 1, i, j);
-    if (phi0_out) {
-        // initialisation: phi is the input field itself
-        phi0_out[dense0[t.x] + (long long)j * I.nx + i] = (double)phib;
-        return;
-    }
-#pragma unroll
-    for (int q = 0; q < Q; q++) Ad.ag[q * N + c] += phib;
+    phi0_out[dense0[g.inst] + (long long)j * I.nx + i] =
+        (double)(Ad.phi[c] + stencil_t<T, 1>(I, geo, Ad.gfx, 0, i, j) + stencil_t<T, 1>(I, geo, Ad.gfy, 1, i, j)
+                 + stencil_t<T, 3>(I, geo, Ad.lapphi, 0, i, j) + stencil_t<T, 3>(I, geo, Ad.lapphi, 1, i, j));
 }
 
 // Step 1 (Eq. auxf a with the original distribution at equilibrium):
 // tilde = eq - dt/2 F; the adjoint of the tracked state is in xf, xg.
 template <typename T>
-__global__ void __launch_bounds__(TX *TY) ka_init(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                  const AxisRec *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
+__global__ void __launch_bounds__(128) ka_init(const InstDev *__restrict__ insts, const AdjSeg *__restrict__ segs, int n_seg,
+                                                  const AxisRecT<T> *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
 {
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
+    const int sg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (sg >= n_seg) return;
+    const AdjSeg g = segs[sg];
+    const InstDev &I = insts[g.inst];
     const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
+    const int i = g.i + (threadIdx.x & 31), j = g.j;
     T lamb = 0;
-    if (i < I.nx && j < I.ny) {
-        const AxisRec &ax = geo[I.gx_off + i];
-        const AxisRec &ay = geo[I.gy_off + j];
+    if (i < I.nx) {
+        const AxisRecT<T> &ax = geo[I.gx_off + i];
+        const AxisRecT<T> &ay = geo[I.gy_off + j];
         const long long c = cell_of(I, i, j);
         const long long N = P.N;
         Pt<T> s;
@@ -854,7 +920,44 @@ __global__ void __launch_bounds__(TX *TY) ka_init(const InstDev *__restrict__ in
         Ad.gfx[c] = gfxb;
         Ad.gfy[c] = gfyb;
     }
-    block_add_param(Ad.pk + 2 * t.x, lamb);
+    slot_add(Ad.lam_cell + sg, lamb);
+}
+
+// d/dlambda and d/dkappa of each instance from the slots of its warps, in a fixed
+// order; rng = {first face run, face runs, first cell run, cell runs}, trng = {first
+// slot of its tiles' warps, slots}.
+__global__ void __launch_bounds__(256) ka_params(const int4 *__restrict__ rng, const int2 *__restrict__ trng,
+                                                 const double *__restrict__ lam_face, const double *__restrict__ lam_cell,
+                                                 const double *__restrict__ kap0, const double *__restrict__ lam_macro,
+                                                 const double *__restrict__ kap, double *pk)
+{
+    __shared__ double s[2][256];
+    const int4 r = rng[blockIdx.x];
+    double l = 0.0, k = 0.0;
+    for (int w = threadIdx.x; w < r.y; w += 256) l += lam_face[r.x + w];
+    for (int w = threadIdx.x; w < r.w; w += 256) {
+        l += lam_cell[r.z + w];
+        k += kap0[r.z + w];
+    }
+    const int2 u = trng[blockIdx.x];
+    for (int w = threadIdx.x; w < u.y; w += 256) {
+        l += lam_macro[u.x + w];
+        k += kap[u.x + w];
+    }
+    s[0][threadIdx.x] = l;
+    s[1][threadIdx.x] = k;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) {
+            s[0][threadIdx.x] += s[0][threadIdx.x + o];
+            s[1][threadIdx.x] += s[1][threadIdx.x + o];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        pk[2 * blockIdx.x] = s[0][0];
+        pk[2 * blockIdx.x + 1] = s[1][0];
+    }
 }
 
 // L = sum_cells (phi - phi*)^2: per-tile FP64 partial loss and the seed

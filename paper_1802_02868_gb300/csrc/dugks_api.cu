@@ -85,6 +85,12 @@ struct dugks_sim {
     int *d_flow_nbr = nullptr;
     unsigned flow_base = 0;
     bool flow_off = false;        // the cooperative launch was refused
+    // adjoint: runs of cells and of faces, and each instance's ranges of them;
+    // built by the first dugks_adjoint
+    AdjSeg *d_cseg = nullptr, *d_fseg = nullptr;
+    int4 *d_segrng = nullptr;
+    int n_cseg = 0, n_fseg = 0;
+    long long n_geo = 0;          // geometry records of all instances
     double2 *d_partials = nullptr;
     RedTile *d_red = nullptr;     // FP32 sims: one record per tile for the conservation sums
     float2 *d_redgeo = nullptr;   // FP32 sims: the widths {d, d_lo} of the geometry records
@@ -657,8 +663,8 @@ int launch_flow(dugks_sim *s, int k, int n)
     constexpr int MB = fused_minb<T, NT, false>();
     static int resident[2] = {0, 0};   // blocks per SM of each class's kernel
     const bool uni = s->n_uni_s[k] > 0;
-    const void *f = uni ? (const void *)k_step<T, BX, BY, NT, MB, true, false, true>
-                        : (const void *)k_step<T, BX, BY, NT, MB, false, false, true>;
+    const void *f = uni ? (const void *)k_step<T, BX, BY, NT, MB, true, false, MODE_FLOW>
+                        : (const void *)k_step<T, BX, BY, NT, MB, false, false, MODE_FLOW>;
     if (!resident[uni]) {
         cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[uni], f, NT, L::bytes);
@@ -965,6 +971,9 @@ void free_sim(dugks_sim *s)
     dfree(s, s->d_status);
     dfree(s, s->d_flow);
     dfree(s, s->d_flow_nbr);
+    dfree(s, s->d_cseg);
+    dfree(s, s->d_fseg);
+    dfree(s, s->d_segrng);
     dfree(s, s->d_partials);
     dfree(s, s->d_red);
     dfree(s, s->d_redgeo);
@@ -1017,166 +1026,273 @@ int sync_status(dugks_sim *s)
 // ---------------------------------------------------------------------------
 // Adjoint: checkpointed forward, then the reverse sweep of dugks_adjoint.cuh
 // ---------------------------------------------------------------------------
+// runs of 32 cells of a row, and of the faces: per axis the high face of each cell
+// and, with walls, the face at the low one
+int ensure_segs(dugks_sim *s)
+{
+    if (s->d_cseg) return DUGKS_OK;
+    std::vector<AdjSeg> cs, fs;
+    std::vector<int4> rng;
+    for (int k = 0; k < s->n_inst; k++) {
+        const InstDev &I = s->h_inst[k];
+        const int f0 = (int)fs.size(), c0 = (int)cs.size();
+        for (int i = 0; i < I.nx; i += 32)
+            for (int j = 0; j < I.ny; j++) cs.push_back({k, i, j, 0});
+        for (int i = I.bcx == DUGKS_BC_WALL ? -1 : 0; i < I.nx; i += 32)
+            for (int j = 0; j < I.ny; j++) fs.push_back({k, i, j, 0});
+        for (int i = 0; i < I.nx; i += 32)
+            for (int j = I.bcy == DUGKS_BC_WALL ? -1 : 0; j < I.ny; j++) fs.push_back({k, i, j, 1});
+        rng.push_back(make_int4(f0, (int)fs.size() - f0, c0, (int)cs.size() - c0));
+    }
+    cudaError_t e = dmalloc(s, (void **)&s->d_fseg, sizeof(AdjSeg) * fs.size());
+    if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_segrng, sizeof(int4) * rng.size());
+    if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_cseg, sizeof(AdjSeg) * cs.size());
+    if (e == cudaSuccess) e = cudaMemcpy(s->d_fseg, fs.data(), sizeof(AdjSeg) * fs.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(s->d_segrng, rng.data(), sizeof(int4) * rng.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(s->d_cseg, cs.data(), sizeof(AdjSeg) * cs.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        dfree(s, s->d_cseg);
+        dfree(s, s->d_fseg);
+        dfree(s, s->d_segrng);
+        s->d_cseg = s->d_fseg = nullptr;
+        s->d_segrng = nullptr;
+        return cuda_status(e);
+    }
+    s->n_cseg = (int)cs.size();
+    s->n_fseg = (int)fs.size();
+    return DUGKS_OK;
+}
+
+template <typename T, int BX, int BY, int NT>
+int launch_planes_shape(dugks_sim *s, int k, const ToPlanes<T> &a)
+{
+    using L = FusedLayout<T, BX, BY, false>;
+    constexpr int MB = fused_minb<T, NT, false>();
+    auto f = k_step<T, BX, BY, NT, MB, false, false, MODE_PLANES>;
+    static bool attr_set = false;
+    if (!attr_set) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+        if (e != cudaSuccess) return cuda_status(e);
+        attr_set = true;
+    }
+    const int rc = ensure_tiles(s, k);
+    if (rc) return rc;
+    f<<<(unsigned)s->n_tiles_s[k], NT, L::bytes, s->stream>>>(s->d_inst, s->d_tiles_s[k], (const AxisRecT<T> *)s->d_geoT, a);
+    return cuda_status(cudaGetLastError());
+}
+
+// tiles of the reverse step: the small ones where the sim's own are small
+// (tile_for_sizes); the index of their table
 template <typename T>
-struct AdjWork {
-    size_t fg_bytes = 0, phi_bytes = 0, state_bytes = 0;
-    void *mem = nullptr;
-    unsigned char *ckpt = nullptr, *seg = nullptr;
-    T *x0 = nullptr, *x1 = nullptr, *bp = nullptr, *scal = nullptr, *fbp = nullptr;
-    double *pk = nullptr, *loss = nullptr, *target = nullptr, *phi0b = nullptr;
-};
+int adj_shape(const dugks_sim *s) { return sizeof(T) == 8 ? (s->tile0 >= 9 ? 9 : 7) : (s->tile0 == 8 ? 8 : 0); }
+
+// bar-plus and the cell fields of a state into the planes of P
+template <typename T>
+int launch_planes(dugks_sim *s, const ToPlanes<T> &a)
+{
+    const int k = adj_shape<T>(s);
+    if constexpr (sizeof(T) == 8)
+        return k == 9 ? launch_planes_shape<T, 8, 4, 128>(s, k, a) : launch_planes_shape<T, 16, 8, 128>(s, k, a);
+    else
+        return k == 8 ? launch_planes_shape<T, 8, 8, 256>(s, k, a) : launch_planes_shape<T, 32, 8, 256>(s, k, a);
+}
 
 template <typename T>
-void copy_state(dugks_sim *s, void *dst_fg, void *dst_phi, const void *src_fg, const void *src_phi, size_t fg_bytes,
-                size_t phi_bytes)
+void launch_tail(dugks_sim *s, const Planes<T> &P, const AdjPlanes<T> &A)
 {
-    cudaMemcpyAsync(dst_fg, src_fg, fg_bytes, cudaMemcpyDeviceToDevice, s->stream);
-    cudaMemcpyAsync(dst_phi, src_phi, phi_bytes, cudaMemcpyDeviceToDevice, s->stream);
+    const int k = adj_shape<T>(s);
+    const unsigned g = (unsigned)s->n_tiles_s[k];
+    const AxisRecT<T> *geo = (const AxisRecT<T> *)s->d_geoT;
+    if constexpr (sizeof(T) == 8) {
+        if (k == 9) ka_tail<T, 8, 4, 128><<<g, 128, 0, s->stream>>>(s->d_inst, s->d_tiles_s[k], geo, P, A);
+        else ka_tail<T, 16, 8, 128><<<g, 128, 0, s->stream>>>(s->d_inst, s->d_tiles_s[k], geo, P, A);
+    } else {
+        if (k == 8) ka_tail<T, 8, 8, 128><<<g, 128, 0, s->stream>>>(s->d_inst, s->d_tiles_s[k], geo, P, A);
+        else ka_tail<T, 32, 8, 256><<<g, 256, 0, s->stream>>>(s->d_inst, s->d_tiles_s[k], geo, P, A);
+    }
 }
+
+template <typename T>
+struct State {   // f, g and phi of one step
+    T *f;
+    phi_t<T> *phi;
+};
 
 template <typename T>
 int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, double *loss_h, double *phi0b_h,
                  double *dkappa_h, double *dlambda_h)
 {
     Planes<T> &P = planes<T>(s);
-    const long long N = P.N, D = s->n_dense;
+    const long long N = P.N, D = s->n_dense, NF = N + (s->n_geo + 31) / 32 * 32;
     const int n = s->n_inst;
-    const dim3 blk(TX, TY);
-    const unsigned g = (unsigned)s->n_tiles;
-    static bool attr_set = false;   // per precision; the tiled face transpose takes more than 48 KB of shared memory
-    if (!attr_set) {
-        const cudaError_t e0 = cudaFuncSetAttribute(ka_face_t<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    (int)AdjTile<T>::bytes);
-        if (e0 != cudaSuccess) return cuda_status(e0);
-        attr_set = true;
+    const int ks = adj_shape<T>(s);
+    int rc = ensure_segs(s);
+    if (!rc) rc = ensure_tiles(s, ks);
+    if (rc) return rc;
+    // warps of the tail's blocks, and each instance's range of them (the tile table
+    // holds the uniform periodic instances' tiles first)
+    const int tw = sizeof(T) == 8 || ks == 8 ? 4 : 8;
+    const size_t n_tslot = (size_t)s->n_tiles_s[ks] * tw;
+    std::vector<int2> trng(n);
+    {
+        int first = 0;
+        for (int pass = 0; pass < 2; pass++)
+            for (int k = 0; k < n; k++) {
+                const InstDev &I = s->h_inst[k];
+                if ((pass == 0) != (s->use_uni && I.uni)) continue;
+                const int c = (I.nx + kShapes[ks].bx - 1) / kShapes[ks].bx * ((I.ny + kShapes[ks].by - 1) / kShapes[ks].by) * tw;
+                trng[k] = make_int2(first, c);
+                first += c;
+            }
     }
-    AdjWork<T> w;
-    w.fg_bytes = sizeof(T) * 2 * Q * (size_t)N;
-    w.phi_bytes = sizeof(phi_t<T>) * (size_t)N;
-    w.state_bytes = w.fg_bytes + w.phi_bytes;
-    const long nck = (nsteps + K - 1) / K;   // checkpoints 0 .. nck (the last is the final state)
-    const size_t scal_planes = 13;
-    const size_t bytes = w.state_bytes * (size_t)(nck + 1 + K) + sizeof(T) * (size_t)N * (2 * 2 * Q + 2 * Q + scal_planes + 2 * Q)
-                       + sizeof(double) * (size_t)(2 * n + n + 2 * D);
-    cudaError_t e = dmalloc(s, (void **)&w.mem, bytes);
+    const size_t fg_bytes = sizeof(T) * 2 * Q * (size_t)N, phi_bytes = sizeof(phi_t<T>) * (size_t)N;
+    const size_t state_bytes = fg_bytes + phi_bytes;   // N is a multiple of 32
+    const long nck = (nsteps + K - 1) / K;             // checkpoints 0 .. nck - 1
+    const long nseg = std::min<long>(K, nsteps) - 1;   // states of a segment after its checkpoint
+    // the sim's own state is kept but for phi, which the initialisation's transpose
+    // takes (the four-kernel step recomputes in place, and needs it all)
+    const size_t keep_bytes = s->fused ? phi_bytes : state_bytes;
+    constexpr int NC = 13;                             // cell planes of the adjoint
+    const size_t n_slot = (size_t)s->n_fseg + 2 * (size_t)s->n_cseg + 2 * n_tslot;
+    const size_t bytes = state_bytes * (size_t)(nck + nseg) + keep_bytes + sizeof(double) * (n_slot + (size_t)(4 * n + 2 * D))
+                       + sizeof(T) * ((size_t)N * (3 * 2 * Q + NC) + (size_t)NF * 2 * NFP) + 16 * 32;
+    void *mem = nullptr;
+    cudaError_t e = dmalloc(s, &mem, bytes);
     if (e != cudaSuccess) return cuda_status(e);
-    unsigned char *m = (unsigned char *)w.mem;
-    w.ckpt = m; m += w.state_bytes * (size_t)(nck + 1);
-    w.seg = m; m += w.state_bytes * (size_t)K;
-    w.x0 = (T *)m; m += w.fg_bytes;
-    w.x1 = (T *)m; m += w.fg_bytes;
-    w.bp = (T *)m; m += sizeof(T) * 2 * Q * (size_t)N;
-    w.scal = (T *)m; m += sizeof(T) * scal_planes * (size_t)N;
-    w.fbp = (T *)m; m += sizeof(T) * 2 * Q * (size_t)N;
-    w.pk = (double *)m; m += sizeof(double) * 2 * n;
-    w.loss = (double *)m; m += sizeof(double) * n;
-    w.target = (double *)m; m += sizeof(double) * D;
-    w.phi0b = (double *)m;
-    T *save_fbp = P.fbp, *save_gbp = P.gbp;
-    P.fbp = w.fbp;
-    P.gbp = w.fbp + (size_t)Q * N;
+    unsigned char *m = (unsigned char *)mem;
+    auto take = [&](size_t b) { unsigned char *r = m; m += (b + 15) / 16 * 16; return r; };
+    unsigned char *ckpt = take(state_bytes * (size_t)nck), *seg = take(state_bytes * (size_t)nseg);
+    unsigned char *keep = take(keep_bytes);
+    double *slots = (double *)take(sizeof(double) * n_slot), *pk = (double *)take(sizeof(double) * 2 * n);
+    double *loss_d = (double *)take(sizeof(double) * n), *target = (double *)take(sizeof(double) * D);
+    double *phi0b = (double *)take(sizeof(double) * D);
+    int2 *trng_d = (int2 *)take(sizeof(int2) * n);
+    T *xb = (T *)take(fg_bytes), *xn = (T *)take(fg_bytes), *fbp = (T *)take(fg_bytes);
+    T *sc = (T *)take(sizeof(T) * (size_t)N * NC);
+    AdjPlanes<T> A;
+    A.N = N;
+    A.NF = NF;
+    for (T *&f : A.face) f = (T *)take(sizeof(T) * (size_t)NF * NFP);
+    T **one[NC] = {&A.phi, &A.mu, &A.lapmu, &A.gmx, &A.gmy, &A.gfx, &A.gfy, &A.gpx, &A.gpy, &A.p, &A.ux, &A.uy, &A.lapphi};
+    for (T **q : one) { *q = sc; sc += N; }
+    A.lam_face = slots;
+    A.lam_cell = slots + s->n_fseg;
+    A.kap0 = A.lam_cell + s->n_cseg;
+    A.lam_macro = A.kap0 + s->n_cseg;
+    A.kap = A.lam_macro + n_tslot;
     const bool timing = s->timing;
     s->timing = false;
-    auto st_fg = [&](long k) { return (void *)(w.ckpt + w.state_bytes * (size_t)k); };
-    auto st_phi = [&](long k) { return (void *)(w.ckpt + w.state_bytes * (size_t)k + w.fg_bytes); };
-    auto sg_fg = [&](long k) { return (void *)(w.seg + w.state_bytes * (size_t)k); };
-    auto sg_phi = [&](long k) { return (void *)(w.seg + w.state_bytes * (size_t)k + w.fg_bytes); };
-    int rc = DUGKS_OK;
+    auto state = [&](unsigned char *at) { return State<T>{(T *)at, (phi_t<T> *)(at + fg_bytes)}; };
+    auto copy = [&](State<T> dst, State<T> src) {
+        cudaMemcpyAsync(dst.f, src.f, fg_bytes, cudaMemcpyDeviceToDevice, s->stream);
+        cudaMemcpyAsync(dst.phi, src.phi, phi_bytes, cudaMemcpyDeviceToDevice, s->stream);
+    };
+    const AxisRecT<T> *geo = (const AxisRecT<T> *)s->d_geoT;
+    // warps per block: single warps spread a small mesh over the SMs
+    const int fw = s->n_fseg >= 16 * s->n_sm ? 4 : 1, cw = s->n_cseg >= 16 * s->n_sm ? 4 : 1;
+    const bool split = s->n_cseg <= 4 * s->n_sm;
+    const unsigned fg = (unsigned)((s->n_fseg + fw - 1) / fw), cg = (unsigned)((s->n_cseg + cw - 1) / cw);
     // forward from the saved init inputs, with checkpoints
     e = cudaMemcpyAsync(s->d_stage, s->d_init_in, sizeof(double) * 4 * D, cudaMemcpyDeviceToDevice, s->stream);
     if (e == cudaSuccess) e = reset_status(s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(w.target, target_h, sizeof(double) * D, cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.pk, 0, sizeof(double) * 3 * n, s->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(target, target_h, sizeof(double) * D, cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(trng_d, trng.data(), sizeof(int2) * n, cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(slots, 0, sizeof(double) * n_slot, s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(loss_d, 0, sizeof(double) * n, s->stream);
     if (e != cudaSuccess) rc = cuda_status(e);
     if (!rc) rc = do_init<T>(s);
     for (long c = 0; c < nck && !rc; c++) {
-        copy_state<T>(s, st_fg(c), st_phi(c), P.f, P.phi, w.fg_bytes, w.phi_bytes);
+        copy(state(ckpt + state_bytes * (size_t)c), State<T>{P.f, P.phi});
         rc = dugks_step(s, std::min<long>(K, nsteps - c * K));
     }
-    if (!rc) copy_state<T>(s, st_fg(nck), st_phi(nck), P.f, P.phi, w.fg_bytes, w.phi_bytes);
-    // loss and the seed adjoint
-    T *xb = w.x0, *xn = w.x1;
     if (!rc) {
-        ka_seed<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, P, xb, xb + (size_t)Q * N, w.target, s->d_dense0, w.loss);
+        if (s->fused) cudaMemcpyAsync(keep, P.phi, phi_bytes, cudaMemcpyDeviceToDevice, s->stream);
+        else copy(state(keep), State<T>{P.f, P.phi});
+        // loss and the seed adjoint
+        ka_seed<T><<<(unsigned)s->n_tiles, dim3(TX, TY), 0, s->stream>>>(s->d_inst, s->d_tiles, P, xb, xb + (size_t)Q * N, target,
+                                                                        s->d_dense0, loss_d);
         s->launches++;
     }
-    AdjPlanes<T> A;
-    A.N = N;
-    A.pk = w.pk;
-    T *sc = w.scal;
-    A.phi = sc; A.mu = sc + N; A.lapmu = sc + 2 * N; A.gmx = sc + 3 * N; A.gmy = sc + 4 * N; A.gfx = sc + 5 * N;
-    A.gfy = sc + 6 * N; A.gpx = sc + 7 * N; A.gpy = sc + 8 * N; A.p = sc + 9 * N; A.ux = sc + 10 * N; A.uy = sc + 11 * N;
-    A.lapphi = sc + 12 * N;
-    A.bp = w.bp;
     // reverse sweep, one checkpoint segment at a time
     for (long c = nck - 1; c >= 0 && !rc; c--) {
         const long len = std::min<long>(K, nsteps - c * K);
-        copy_state<T>(s, P.f, P.phi, st_fg(c), st_phi(c), w.fg_bytes, w.phi_bytes);
-        for (long k = 0; k < len && !rc; k++) {
-            copy_state<T>(s, sg_fg(k), sg_phi(k), P.f, P.phi, w.fg_bytes, w.phi_bytes);
-            if (k + 1 < len) rc = dugks_step(s, 1);
+        auto at = [&](long k) { return state(k == 0 ? ckpt + state_bytes * (size_t)c : seg + state_bytes * (size_t)(k - 1)); };
+        if (!s->fused && len > 1) copy(State<T>{P.f, P.phi}, at(0));
+        for (long k = 0; k + 1 < len && !rc; k++) {
+            const State<T> a = at(k), b = at(k + 1);
+            if (s->fused) {
+                StepIO<T> io = step_io<T>(s);
+                io.f_in = a.f; io.g_in = a.f + (size_t)Q * N; io.phi_in = a.phi;
+                io.f_out = b.f; io.g_out = b.f + (size_t)Q * N; io.phi_out = b.phi;
+                enqueue_fused<T>(s, io, s->stream);
+                s->launches += fused_launches(s);
+                rc = cuda_status(cudaGetLastError());
+            } else {
+                rc = dugks_step(s, 1);
+                if (!rc) copy(b, State<T>{P.f, P.phi});
+            }
         }
         for (long k = len - 1; k >= 0 && !rc; k--) {
-            copy_state<T>(s, P.f, P.phi, sg_fg(k), sg_phi(k), w.fg_bytes, w.phi_bytes);
-            k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P);
-            k_macro<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P, 0);
-            k_cell<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P);
-            cudaMemsetAsync(w.bp, 0, sizeof(T) * 2 * Q * (size_t)N, s->stream);
-            cudaMemsetAsync(w.scal, 0, sizeof(T) * scal_planes * (size_t)N, s->stream);
+            const State<T> a = at(k);
+            ToPlanes<T> tp;
+            tp.io = step_io<T>(s);
+            tp.io.f_in = a.f; tp.io.g_in = a.f + (size_t)Q * N; tp.io.phi_in = a.phi;
+            tp.P = P;
+            tp.P.f = a.f; tp.P.g = a.f + (size_t)Q * N; tp.P.phi = a.phi;
+            tp.P.fbp = fbp; tp.P.gbp = fbp + (size_t)Q * N;
+            const Planes<T> &R = tp.P;
+            rc = launch_planes<T>(s, tp);
+            if (rc) break;
             A.xf = xb; A.xg = xb + (size_t)Q * N;
             A.af = xn; A.ag = xn + (size_t)Q * N;
-            ka_face_t<T><<<g, blk, AdjTile<T>::bytes, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT,
-                                                                  P, A);
-            ka_cell<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A);
-            ka_macro<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A);
-            ka_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A);
-            ka_phi<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A, nullptr, s->d_dense0);
-            s->launches += 8;
+            ka_face<T><<<fg, 32 * fw, 0, s->stream>>>(s->d_inst, s->d_fseg, s->n_fseg, geo, R, A);
+            if (split) ka_cell<T, true><<<(unsigned)s->n_cseg, 128, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, R, A);
+            else ka_cell<T, false><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, R, A);
+            launch_tail<T>(s, R, A);
+            s->launches += 4;
             std::swap(xb, xn);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) rc = cuda_status(e);
+            rc = cuda_status(cudaGetLastError());
         }
     }
     // the initialisation: planes hold phi0, u0, p0 and mu(phi0)
     if (!rc) {
-        const dim3 b2(TX, TY);
-        k_unpack_phi<phi_t<T>><<<g, b2, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in, P.phi, s->d_dense0);
-        k_unpack<T><<<g, b2, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + D, P.ux, s->d_dense0);
-        k_unpack<T><<<g, b2, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 2 * D, P.uy, s->d_dense0);
-        k_unpack<T><<<g, b2, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 3 * D, P.p, s->d_dense0);
-        k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P);
-        cudaMemsetAsync(w.scal, 0, sizeof(T) * scal_planes * (size_t)N, s->stream);
+        const dim3 blk(TX, TY);
+        const unsigned g = (unsigned)s->n_tiles;
+        k_unpack_phi<phi_t<T>><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in, P.phi, s->d_dense0);
+        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + D, P.ux, s->d_dense0);
+        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 2 * D, P.uy, s->d_dense0);
+        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 3 * D, P.p, s->d_dense0);
+        k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P);
         A.xf = xb; A.xg = xb + (size_t)Q * N;
-        ka_init<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A);
-        ka_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A);
-        ka_phi<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P, A, w.phi0b, s->d_dense0);
-        s->launches += 8;
-        e = cudaGetLastError();
-        if (e != cudaSuccess) rc = cuda_status(e);
+        ka_init<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, P, A);
+        ka_mu<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, P, A);
+        ka_phi0<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, A, phi0b, s->d_dense0);
+        ka_params<<<(unsigned)n, 256, 0, s->stream>>>(s->d_segrng, trng_d, A.lam_face, A.lam_cell, A.kap0, A.lam_macro, A.kap, pk);
+        s->launches += 9;
+        // leave the simulation at the final state of the forward run
+        if (s->fused) cudaMemcpyAsync(P.phi, keep, phi_bytes, cudaMemcpyDeviceToDevice, s->stream);
+        else copy(State<T>{P.f, P.phi}, state(keep));
+        rc = cuda_status(cudaGetLastError());
     }
-    // leave the simulation at the final state of the forward run
-    if (!rc) copy_state<T>(s, P.f, P.phi, st_fg(nck), st_phi(nck), w.fg_bytes, w.phi_bytes);
-    std::vector<double> pk(2 * n), loss(n);
+    std::vector<double> pkh(2 * n), loss(n);
     if (!rc) {
-        e = cudaMemcpyAsync(pk.data(), w.pk, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(loss.data(), w.loss, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess && phi0b_h) e = cudaMemcpyAsync(phi0b_h, w.phi0b, sizeof(double) * D, cudaMemcpyDeviceToHost, s->stream);
+        e = cudaMemcpyAsync(pkh.data(), pk, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, s->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(loss.data(), loss_d, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream);
+        if (e == cudaSuccess && phi0b_h) e = cudaMemcpyAsync(phi0b_h, phi0b, sizeof(double) * D, cudaMemcpyDeviceToHost, s->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) rc = cuda_status(e);
     }
     if (!rc) {
         for (int k = 0; k < n; k++) {
             if (loss_h) loss_h[k] = loss[k];
-            if (dlambda_h) dlambda_h[k] = pk[2 * k];
-            if (dkappa_h) dkappa_h[k] = pk[2 * k + 1];
+            if (dlambda_h) dlambda_h[k] = pkh[2 * k];
+            if (dkappa_h) dkappa_h[k] = pkh[2 * k + 1];
         }
         rc = sync_status(s);
     }
     cudaStreamSynchronize(s->stream);
-    P.fbp = save_fbp;
-    P.gbp = save_gbp;
     s->timing = timing;
-    dfree(s, w.mem);
+    dfree(s, mem);
     return rc;
 }
 
@@ -1311,24 +1427,27 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         fill(I.pd);
         fill(I.pf);
         I.b4 = 4.0 * I.beta;
-        I.cd64 = I.drho / 3.0;
-        I.cgl64 = I.gamma * I.lambda / 3.0;
         I.rh64 = 1.0 / I.h;
-        const double K = I.muA * I.muB * (I.phiA - I.phiB), tg = I.tau_g;
-        // half the time tau over which the force of the point's velocity acts,
-        // the weights b and c of Eqs. (relations1), (original-function) over w
-        auto point = [&](PtC64 &C, double tau, double nb, double nc, double ga, double gb, double gc) {
-            C.kf = tau / 3.0;
-            C.kp1 = C.kf * I.drho;
-            C.kp2 = C.kf * I.gamma * I.lambda;
-            C.k6 = 6.0 * K;
-            C.nb = nb / 36.0; C.nc = nc / 36.0;
-            C.ga = ga; C.gb = gb / 36.0; C.gbe = C.gb * I.eta; C.gc = 3.0 * gc / 36.0;
-            C.gb36 = gb; C.gbe36 = gb * I.eta;
+        // tau: the time over which the force of the point's velocity acts; nb, nc
+        // and gb, gc: the numerators of the weights b and c of Eqs. (relations1),
+        // (original-function)
+        auto point = [&](auto &C, double tau, double nb, double nc, double ga, double gb, double gc) {
+            using U = std::remove_reference_t<decltype(C.kf)>;
+            const double K = I.muA * I.muB * (I.phiA - I.phiB), kf = tau / 3.0, deta = 3.0 / I.tau_g;   // d eta / d lambda
+            C.kf = (U)kf; C.kp1 = (U)(kf * I.drho); C.kp2 = (U)(kf * I.gamma * I.lambda);
+            C.k6 = (U)(6.0 * K); C.nb = (U)(nb / 36.0); C.nc = (U)(nc * K / 36.0);
+            C.ga = (U)ga; C.gb = (U)(gb / 36.0); C.gbe = (U)(gb * I.eta / 36.0); C.gc = (U)(3.0 * gc / 36.0);
+            C.gb36 = (U)gb; C.gbe36 = (U)(gb * I.eta);
+            C.cd = (U)(I.drho / 3.0); C.cgl = (U)(I.gamma * I.lambda / 3.0);
+            C.dgbe = (U)(gb * deta / 36.0); C.dkp2 = (U)(kf * I.gamma); C.dcgl = (U)(I.gamma / 3.0);
         };
-        const double gcell = 2.0 * tg + I.dt, gface = 2.0 * tg + I.h;
-        point(I.cell64, 0.5 * I.dt, 3.0, 9.0 * K * I.h, (2.0 * tg - I.h) / gcell, 3.0 * I.h / gcell, 3.0 * tg * I.h / gcell);
-        point(I.face64, 0.5 * I.h, 1.0, 3.0 * K * I.h, 2.0 * tg / gface, I.h / gface, tg * I.h / gface);
+        auto points = [&](auto &cell, auto &face) {
+            const double tg = I.tau_g, gcell = 2.0 * tg + I.dt, gface = 2.0 * tg + I.h;
+            point(cell, 0.5 * I.dt, 3.0, 9.0 * I.h, (2.0 * tg - I.h) / gcell, 3.0 * I.h / gcell, 3.0 * tg * I.h / gcell);
+            point(face, 0.5 * I.h, 1.0, 3.0 * I.h, 2.0 * tg / gface, I.h / gface, tg * I.h / gface);
+        };
+        points(I.cell64, I.face64);
+        points(I.cell32, I.face32);
         I.tile0 = (int)tiles.size();
         for (int ty = 0; ty < m.ny; ty += TY)
             for (int tx = 0; tx < m.nx; tx += TX) tiles.push_back(make_int4(k, tx, ty, 0));
@@ -1336,6 +1455,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         s->h_inst.push_back(I);
     }
     s->N = cell;
+    s->n_geo = (long long)geo.size();
     s->n_dense = dense;
     s->n_tiles = (int)tiles.size();
     choose_shapes(s);

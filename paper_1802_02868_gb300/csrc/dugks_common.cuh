@@ -143,14 +143,18 @@ __device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
 __device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
-// Constants of the FP64 step (dugks_fp64.cuh) at a cell (Eqs. u, P, relations1)
-// or at a face (Eqs. conservedVariable, original-function).  w = 1/36, the
-// diagonals' weight, is part of nb, nc, gb, gbe and gc.
-struct PtC64 {
-    double kf, kp1, kp2;      // c_s^2 tau, with drho, with gamma lambda; tau = dt/2 (cell), h/2 (face)
-    double k6, nb, nc;        // 6K and the numerators w b / X, w c of the f weights (see cell_weights, face_weights)
-    double ga, gb, gbe, gc;   // g weights: a; w b; w b eta; 3 w c
-    double gb36, gbe36;       // b, b eta
+// Constants of the regrouped point arithmetic (dugks_fp64.cuh, dugks_adjoint.cuh)
+// at a cell (Eqs. u, P, relations1) or at a face (Eqs. conservedVariable,
+// original-function).  w = 1/36, the diagonals' weight, is part of nb, nc, gb, gbe
+// and gc.
+template <typename T>
+struct PtC {
+    T kf, kp1, kp2;       // c_s^2 tau, with drho, with gamma lambda; tau = dt/2 (cell), h/2 (face)
+    T k6, nb, nc;         // 6K and the numerators w b / X, w c of the f weights (see cell_weights, face_weights)
+    T ga, gb, gbe, gc;    // g weights: a; w b; w b eta; 3 w c
+    T gb36, gbe36;        // b, b eta
+    T cd, cgl;            // c_s^2 drho, c_s^2 gamma lambda
+    T dgbe, dkp2, dcgl;   // gbe, kp2 and cgl over lambda
 };
 
 // Per-instance constants.
@@ -171,9 +175,9 @@ struct InstDev {
     PhiC cA, cB, cM;
     ParT<double> pd;
     ParT<float> pf;
-    // FP64 step: 4 beta, c_s^2 drho, c_s^2 gamma lambda, 1 / h
-    double b4, cd64, cgl64, rh64;
-    PtC64 cell64, face64;
+    double b4, rh64;   // FP64 step: 4 beta, 1 / h
+    PtC<double> cell64, face64;
+    PtC<float> cell32, face32;
 };
 
 // Flux-carrying directions of x faces (cx != 0) and of y faces (cy != 0).
@@ -188,6 +192,19 @@ template <>
 __device__ __forceinline__ const ParT<double> &par<double>(const InstDev &I) { return I.pd; }
 template <>
 __device__ __forceinline__ const ParT<float> &par<float>(const InstDev &I) { return I.pf; }
+
+template <typename T>
+__device__ __forceinline__ const PtC<T> &cellc(const InstDev &I);
+template <>
+__device__ __forceinline__ const PtC<double> &cellc<double>(const InstDev &I) { return I.cell64; }
+template <>
+__device__ __forceinline__ const PtC<float> &cellc<float>(const InstDev &I) { return I.cell32; }
+template <typename T>
+__device__ __forceinline__ const PtC<T> &facec(const InstDev &I);
+template <>
+__device__ __forceinline__ const PtC<double> &facec<double>(const InstDev &I) { return I.face64; }
+template <>
+__device__ __forceinline__ const PtC<float> &facec<float>(const InstDev &I) { return I.face32; }
 
 // All device planes of a simulation.  Distribution planes are [Q][N], the
 // rest [N], N = total padded cells of all instances.

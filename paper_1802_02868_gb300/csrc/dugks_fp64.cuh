@@ -84,13 +84,13 @@ __device__ __forceinline__ double chem(const InstDev &I, double p0, double dxm, 
 
 // u and p of a point (Eqs. u, P at a cell, Eq. conservedVariable at a face;
 // C.kf = c_s^2 times half the time over which the force acts).
-__device__ __forceinline__ void velocity(const PtC64 &C, const Mom &m, double irho, double Fx, double Fy, double &ux, double &uy)
+__device__ __forceinline__ void velocity(const PtC<double> &C, const Mom &m, double irho, double Fx, double Fy, double &ux, double &uy)
 {
     const double r3 = mu(3.0, irho);
     ux = mu(fm(C.kf, Fx, m.x), r3);
     uy = mu(fm(C.kf, Fy, m.y), r3);
 }
-__device__ __forceinline__ double pressure(const PtC64 &C, double sf, double ux, double uy, double gfx, double gfy, double rho_lmu)
+__device__ __forceinline__ double pressure(const PtC<double> &C, double sf, double ux, double uy, double gfx, double gfy, double rho_lmu)
 {
     return fm(C.kp1, fm(ux, gfx, mu(uy, gfy)), fm(-C.kp2, rho_lmu, sf));
 }
@@ -127,21 +127,21 @@ __device__ __forceinline__ void eq_dirs(double ux, double uy, Eq &E)
 
 // f part: r = 1 / (6K + k X), X the weight variable; CELL: Eq. (relations1), else Eq. (original-function)
 template <bool CELL>
-__device__ __forceinline__ void eq_f(const InstDev &I, const PtC64 &C, double X, double r, double rho, double rho_lmu, double ux,
+__device__ __forceinline__ void eq_f(const InstDev &I, const PtC<double> &C, double X, double r, double rho, double rho_lmu, double ux,
                                      double uy, double p, double Fx, double Fy, double gfx, double gfy, Eq &E)
 {
     E.a = mu(CELL ? sb(C.k6, X) : C.k6, r);
     const double b = mu(X, mu(C.nb, r)), c = mu(C.nc, r);
-    const double FCx = fm(I.cd64, gfx, Fx), FCy = fm(I.cd64, gfy, Fy);
+    const double FCx = fm(C.cd, gfx, Fx), FCy = fm(C.cd, gfy, Fy);
     const double uF = fm(ux, Fx, mu(uy, Fy)), uFC = fm(ux, FCx, mu(uy, FCy));
-    E.K0 = fm(-c, fm(I.cgl64, rho_lmu, uF), mu(b, p));
+    E.K0 = fm(-c, fm(C.cgl, rho_lmu, uF), mu(b, p));
     E.K1 = fm(-c, uFC, mu(b, mu(1.0 / 3.0, rho)));
     E.fx = mu(c, Fx);
     E.fy = mu(c, Fy);
     E.ex = mu(c, FCx);
     E.ey = mu(c, FCy);
 }
-__device__ __forceinline__ void eq_g(const PtC64 &C, double phi, double irho, double ux, double uy, double m, double Gx,
+__device__ __forceinline__ void eq_g(const PtC<double> &C, double phi, double irho, double ux, double uy, double m, double Gx,
                                      double Gy, Eq &E)
 {
     const double P = mu(mu(C.gc, phi), irho);
@@ -177,7 +177,7 @@ __device__ __forceinline__ void pair_f(const Eq &E, double v0, double v1, double
     pair_of<q>(E.a, E.K0, E.K1, E.fx, E.fy, E.ex, E.ey, E, v0, v1, o0, o1);
 }
 template <int q>
-__device__ __forceinline__ void pair_g(const PtC64 &C, const Eq &E, double v0, double v1, double &o0, double &o1)
+__device__ __forceinline__ void pair_g(const PtC<double> &C, const Eq &E, double v0, double v1, double &o0, double &o1)
 {
     pair_of<q>(C.ga, E.A2, E.D2, E.gx, E.gy, E.gx, E.gy, E, v0, v1, o0, o1);
 }
@@ -191,7 +191,7 @@ __device__ __forceinline__ void bar_plus_f(const Eq &E, double (&v)[Q])
     pair_f<5>(E, v[5], v[7], v[5], v[7]);
     pair_f<6>(E, v[6], v[8], v[6], v[8]);
 }
-__device__ __forceinline__ void bar_plus_g(const PtC64 &C, const Eq &E, double phi, double m, double (&v)[Q])
+__device__ __forceinline__ void bar_plus_g(const PtC<double> &C, const Eq &E, double phi, double m, double (&v)[Q])
 {
     // the rest direction's H is phi - (1 - w_0) eta mu
     const double rest = fm(C.gb36, phi, fm(-C.gbe36, m, mu(C.ga, v[0])));
@@ -212,7 +212,7 @@ template <int A>
 __device__ __forceinline__ void originals(const InstDev &I, const double (&fb)[Q], const double (&gb)[Q], const Aux &x, int side,
                                           double2 (&o)[6])
 {
-    const PtC64 &C = I.face64;
+    const PtC<double> &C = I.face64;
     const Mom m = moments(fb);
     const double phi = ad(ad(ad(gb[0], ad(gb[1], gb[3])), ad(gb[2], gb[4])), ad(ad(gb[5], gb[7]), ad(gb[6], gb[8])));
     const double rho = rho_of(I, phi), dr = sb(rho, I.rho_ref);
@@ -299,7 +299,7 @@ template <int KIND, typename TL>
 __device__ __forceinline__ void bar_plus_point(const InstDev &I, const TL &S, int x, int y, double (&f)[Q], double (&g)[Q])
 {
     if (!S.ok(0, x) || !S.ok(1, y)) return;   // no face reads it
-    const PtC64 &C = I.cell64;
+    const PtC<double> &C = I.cell64;
     const int k1 = TL::i1(x, y), k2 = TL::i2(x, y);
     const double phi = S.phi[TL::i4(x, y)], m = S.mu[TL::i3(x, y)], p = S.p[k2];
     const double rho = rho_of(I, phi), dr = sb(rho, I.rho_ref);

@@ -374,8 +374,20 @@ struct Flow {
     int *err;                  // set when a wait ran out
     unsigned limit;            // polls before a wait gives up
 };
+// What k_step does: one step; many steps; or the step up to bar-plus, whose cell
+// fields and bar-plus go to the planes P (for the adjoint's reverse step).
+constexpr int MODE_STEP = 0, MODE_FLOW = 1, MODE_PLANES = 2;
+template <typename T>
+struct ToPlanes {
+    StepIO<T> io;
+    Planes<T> P;
+};
+template <typename T, int MODE>
+using step_arg = std::conditional_t<MODE == MODE_FLOW, Flow<T>, std::conditional_t<MODE == MODE_PLANES, ToPlanes<T>, StepIO<T>>>;
 template <typename T>
 __device__ __forceinline__ const StepIO<T> &step_io_of(const StepIO<T> &io, int) { return io; }
+template <typename T>
+__device__ __forceinline__ const StepIO<T> &step_io_of(const ToPlanes<T> &a, int) { return a.io; }
 template <typename T>
 __device__ __forceinline__ const StepIO<T> &step_io_of(const Flow<T> &fl, int step) { return fl.io[step & 1]; }
 
@@ -393,11 +405,12 @@ __device__ __forceinline__ const StepIO<T> &step_io_of(const Flow<T> &fl, int st
 // dependent kernels (about 2 us) and the geometry set-up every step, and a step of
 // a few waves waited for its last, partly filled one (four 100x100 drops in FP64:
 // 364 tiles of 16x8 on 304 resident blocks, 132 -> 98.6 us per step).
-template <typename T, int BX, int BY, int NT, int MINB, bool UNI, bool SEP, bool FLOW = false>
+template <typename T, int BX, int BY, int NT, int MINB, bool UNI, bool SEP, int MODE = MODE_STEP>
 __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
                                                    const AxisRecT<T> *__restrict__ geo,
-                                                   const __grid_constant__ std::conditional_t<FLOW, Flow<T>, StepIO<T>> arg)
+                                                   const __grid_constant__ step_arg<T, MODE> arg)
 {
+    constexpr bool FLOW = MODE == MODE_FLOW, PLANES = MODE == MODE_PLANES;
     static_assert(NT % 32 == 0 && NT >= BX * BY, "thread count");
     using TL = Tile<T, BX, BY, UNI, SEP>;
     using L = typename TL::L;
@@ -439,7 +452,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     const int4 t = tiles[item];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
-    const StepIO<T> &io = step_io_of(arg, step);
+    const StepIO<T> &io = step_io_of<T>(arg, step);
     const int i0 = t.y, j0 = t.z;
     do {   // left by the threads that have nothing more to do for the tile
     {
@@ -450,7 +463,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
             st = io.status[t.x];
         }
         if (st & ST_NONFINITE) break;   // masked: non-finite instance of a batch
-        if (st & ST_PAUSED) {           // paused: the state passes to the other buffer unchanged
+        if (!PLANES && (st & ST_PAUSED)) {   // paused: the state passes to the other buffer unchanged
             const int x = tid % BX, y = tid / BX;
             if (tid < BX * BY && i0 + x < I.nx && j0 + y < I.ny) {
                 const long long c = I.cell0 + (long long)(j0 + y) * I.nxp + (i0 + x);
@@ -703,6 +716,13 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         s.gry = Pr.drho * gfy;
         s.gpx = gpx;
         s.gpy = gpy;
+        if constexpr (PLANES) {   // no other phase keeps u
+            if (x >= 0 && x < BX && y >= 0 && y < BY && i0 + x < I.nx && j0 + y < I.ny) {
+                const long long c = cell(i0 + x, j0 + y);
+                arg.P.ux[c] = s.ux;
+                arg.P.uy[c] = s.uy;
+            }
+        }
         T af, bf, cf;
         cell_weights<T>(Pr, s.phi, s.rho, af, bf, cf);
         const PtInv<T> v = pt_inv<T>(I, s);
@@ -721,6 +741,36 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         }
     }
     __syncthreads();
+
+    if constexpr (PLANES) {
+        for (int r = tid; r < BX * BY; r += NT) {
+            const int x = r % BX, y = r / BX;
+            if (i0 + x >= I.nx || j0 + y >= I.ny) continue;
+            const long long c = cell(i0 + x, j0 + y);
+            const int k1 = TL::i1(x, y), k2 = TL::i2(x, y), ka = L::F64 ? k2 : k1;
+            const Planes<T> &P = arg.P;
+            P.mu[c] = S.mu[TL::i3(x, y)];
+            P.lapmu[c] = S.lmu[ka];
+            P.gmux[c] = S.gmx[ka];
+            P.gmuy[c] = S.gmy[ka];
+            P.gphix[c] = S.gfx[ka];
+            P.gphiy[c] = S.gfy[ka];
+            P.p[c] = S.p[k2];
+            P.gpx[c] = S.gpx[k1];
+            P.gpy[c] = S.gpy[k1];
+            if constexpr (L::F64) {
+                P.ux[c] = S.ux[k2];
+                P.uy[c] = S.uy[k2];
+            }
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                const pair_t<T> b = S.bp[q * L::A1 + k1];
+                P.fbp[q * N + c] = b.x;
+                P.gbp[q * N + c] = b.y;
+            }
+        }
+    }
+    if (PLANES) break;
 
     // ---- phase 5: every face of the tile once (x faces first in the item space)
     for (int k = tid; k < L::NFT; k += NT) {
