@@ -960,7 +960,7 @@ __global__ void __launch_bounds__(256) ka_params(const int4 *__restrict__ rng, c
     }
 }
 
-// L = sum_cells (phi - phi*)^2: per-tile FP64 partial loss and the seed
+// L = sum_cells (phi - phi*)^2: FP64 partial losses, one slot per warp, and the seed
 // adjoint of the state (dL/dg~_i = 2 (phi - phi*), dL/df~_i = 0).
 template <typename T>
 __global__ void __launch_bounds__(TX *TY) ka_seed(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
@@ -986,7 +986,23 @@ __global__ void __launch_bounds__(TX *TY) ka_seed(const InstDev *__restrict__ in
         }
     }
     for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss + t.x, l);
+    if (threadIdx.x == 0) loss[blockIdx.x * TY + threadIdx.y] = l;
+}
+
+// The loss of each instance from its tiles' slots, in a fixed order.
+__global__ void __launch_bounds__(256) ka_loss(const InstDev *__restrict__ insts, const double *__restrict__ part, double *loss)
+{
+    __shared__ double s[256];
+    const InstDev &I = insts[blockIdx.x];
+    double l = 0.0;
+    for (int w = threadIdx.x; w < I.ntiles * TY; w += 256) l += part[(long long)I.tile0 * TY + w];
+    s[threadIdx.x] = l;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) loss[blockIdx.x] = s[0];
 }
 
 }  // namespace dugks

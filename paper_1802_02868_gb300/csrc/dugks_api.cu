@@ -78,7 +78,7 @@ struct dugks_sim {
     int n_uni_s[kNumKernelShapes] = {};
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph2 = nullptr;   // k_step(A -> B), k_step(B -> A)
-    int *d_status = nullptr;      // per instance, then the error word of the many-step launches
+    int *d_status = nullptr;      // per instance, then the error word of the many-step launches and the refused word
     // many-step launches: progress counters, ring neighbours (FLOW_NB per tile) and the value
     // that every counter holds; built by the first call that uses it
     unsigned *d_flow = nullptr;
@@ -779,25 +779,27 @@ int launch_step(dugks_sim *s)
     const dim3 blk(TX, TY);
     const unsigned g = (unsigned)s->n_tiles;
     { Timed t(s, K_MU); k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P); }
-    { Timed t(s, K_MACRO); k_macro<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P, 0); }
+    { Timed t(s, K_MACRO); k_macro<T, false><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P, DenseOut{}); }
     { Timed t(s, K_CELL); k_cell<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P); }
     { Timed t(s, K_FACE); k_face<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P); }
     return cuda_status(cudaGetLastError());
 }
 
+// flag word: set on the device when a call's input is refused
+int *refused(const dugks_sim *s) { return s->d_status + s->n_inst + 1; }
+
+// in: dense phi, ux, uy, p on the device (NULL but for phi: zero); keep: where the
+// adjoint's copy of them goes, NULL for none
 template <typename T>
-int do_init(dugks_sim *s)
+int do_init(dugks_sim *s, const double *const in[4], double *keep)
 {
     Planes<T> &P = planes<T>(s);
     const dim3 blk(TX, TY);
     const unsigned g = (unsigned)s->n_tiles;
-    const long long D = s->n_dense;
-    { Timed t(s, -1); k_unpack_phi<phi_t<T>><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_stage + 0 * D, P.phi, s->d_dense0); }
-    { Timed t(s, -1); k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_stage + 1 * D, P.ux, s->d_dense0); }
-    { Timed t(s, -1); k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_stage + 2 * D, P.uy, s->d_dense0); }
-    { Timed t(s, -1); k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_stage + 3 * D, P.p, s->d_dense0); }
-    { Timed t(s, K_MU); k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P); }
-    { Timed t(s, K_INIT); k_init<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_geo, P); }
+    const AxisRecT<T> *geo = (const AxisRecT<T> *)s->d_geoT;
+    { Timed t(s, -1); k_unpack_init<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, in[0], in[1], in[2], in[3], P, keep, s->n_dense, s->d_dense0, refused(s)); }
+    { Timed t(s, K_MU); k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P); }
+    { Timed t(s, K_INIT); k_init<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P, refused(s)); }
     // FP64: phi = sum g of the new state, as the next step recomputes it; FP32:
     // the given phi stays the authoritative FP64 order parameter
     if (sizeof(T) == sizeof(double)) { Timed t(s, -1); k_phi<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, P); }
@@ -812,44 +814,29 @@ int do_moments(dugks_sim *s, double *const dst[5])
     Planes<T> &P = planes<T>(s);
     const dim3 blk(TX, TY);
     const unsigned g = (unsigned)s->n_tiles;
-    { Timed t(s, K_MU); k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P); }
-    { Timed t(s, K_MACRO); k_macro<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, (const AxisRecT<T> *)s->d_geoT, P, 1); }
-    if (dst[0]) { Timed t(s, -1); k_pack_phi<phi_t<T>><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, P.phi, dst[0], s->d_dense0); }
-    T *src[4] = {P.rho, P.ux, P.uy, P.p};
-    for (int k = 0; k < 4; k++) {
-        if (!dst[k + 1]) continue;
-        Timed t(s, -1);
-        k_pack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, src[k], dst[k + 1], s->d_dense0);
-    }
+    const AxisRecT<T> *geo = (const AxisRecT<T> *)s->d_geoT;
+    DenseOut D;
+    for (int k = 0; k < 5; k++) D.out[k] = dst[k];
+    D.dense0 = s->d_dense0;
+    { Timed t(s, K_MU); k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P); }
+    { Timed t(s, K_MACRO); k_macro<T, true><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P, D); }
     return cuda_status(cudaGetLastError());
 }
 
 template <typename T>
 int do_pack_state(dugks_sim *s, double *dst_dev)
 {
-    Planes<T> &P = planes<T>(s);
-    const dim3 blk(TX, TY);
-    const unsigned g = (unsigned)s->n_tiles;
-    for (int q = 0; q < 2 * Q; q++) {
-        const T *src = (q < Q ? P.f : P.g) + (long long)(q % Q) * P.N;
-        Timed t(s, -1);
-        k_pack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, src, dst_dev + (long long)q * s->n_dense, s->d_dense0);
-    }
+    Timed t(s, -1);
+    k_pack_state<T><<<(unsigned)s->n_tiles, dim3(TX, TY), 0, s->stream>>>(s->d_inst, s->d_tiles, planes<T>(s), dst_dev, s->n_dense, s->d_dense0);
     return cuda_status(cudaGetLastError());
 }
 
 template <typename T>
 int do_unpack_state(dugks_sim *s, const double *src_dev)
 {
-    Planes<T> &P = planes<T>(s);
-    const dim3 blk(TX, TY);
-    const unsigned g = (unsigned)s->n_tiles;
-    for (int q = 0; q < 2 * Q; q++) {
-        T *dst = (q < Q ? P.f : P.g) + (long long)(q % Q) * P.N;
-        Timed t(s, -1);
-        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, src_dev + (long long)q * s->n_dense, dst, s->d_dense0);
-    }
-    { Timed t(s, -1); k_phi<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, P); }
+    Timed t(s, -1);
+    k_unpack_state<T><<<(unsigned)s->n_tiles, dim3(TX, TY), 0, s->stream>>>(s->d_inst, s->d_tiles, planes<T>(s), src_dev, s->n_dense, s->d_dense0,
+                                                                           refused(s));
     return cuda_status(cudaGetLastError());
 }
 
@@ -944,14 +931,14 @@ void assign_planes(dugks_sim *s, Planes<T> &P, T *base)
         P.fbp = p; p += Q * N;
         P.gbp = p; p += Q * N;
     }
-    T **one[] = {&P.mu, &P.lapmu, &P.gmux, &P.gmuy, &P.gphix, &P.gphiy, &P.p, &P.ux, &P.uy, &P.gpx, &P.gpy, &P.rho};
+    T **one[] = {&P.mu, &P.lapmu, &P.gmux, &P.gmuy, &P.gphix, &P.gphiy, &P.p, &P.ux, &P.uy, &P.gpx, &P.gpy};
     for (T **q : one) { *q = p; p += N; }
     P.phi = (phi_t<T> *)s->d_phi;
     P.N = N;
     P.status = s->d_status;
 }
 
-constexpr int kNumScalarPlanes = 12;
+constexpr int kNumScalarPlanes = 11;
 
 void free_sim(dugks_sim *s)
 {
@@ -994,33 +981,49 @@ void free_sim(dugks_sim *s)
     delete s;
 }
 
-// A new state: every instance finite and running, the counters of the many-step launches (which a
-// wait that ran out leaves uneven) and error word at zero.
-cudaError_t reset_status(dugks_sim *s)
+// The counters of the many-step launches (which a wait that ran out leaves uneven)
+// and their error word to zero.
+cudaError_t reset_flow(dugks_sim *s)
 {
-    cudaError_t e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * (s->n_inst + 1), s->stream);
-    if (e == cudaSuccess && s->d_flow) {
-        e = cudaMemsetAsync(s->d_flow, 0, sizeof(unsigned) * s->n_tiles_s[s->tile0], s->stream);
-        s->flow_base = 0;
-    }
+    if (!s->d_flow) return cudaSuccess;
+    s->flow_base = 0;
+    cudaError_t e = cudaMemsetAsync(s->d_status + s->n_inst, 0, sizeof(int), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->d_flow, 0, sizeof(unsigned) * s->n_tiles_s[s->tile0], s->stream);
     return e;
 }
 
-// After a synchronisation: a single simulation reports a non-finite state as
-// DUGKS_ERR_NONFINITE; a batch masks the affected instances and reports them
-// through dugks_batch_status only.
+// A new state: every instance finite and running, nothing refused.
+cudaError_t reset_status(dugks_sim *s)
+{
+    const cudaError_t e = cudaMemsetAsync(s->d_status, 0, sizeof(int) * (s->n_inst + 2), s->stream);
+    return e == cudaSuccess ? reset_flow(s) : e;
+}
+
+// Synchronise, and report a wait that ran out, and for a single simulation a
+// non-finite state; a batch masks the affected instances and reports them through
+// dugks_batch_status only.
 int sync_status(dugks_sim *s)
 {
-    cudaError_t e = cudaStreamSynchronize(s->stream);
+    int st[2] = {0, 0};   // the status of a single sim, the error word
+    cudaError_t e = cudaSuccess;
+    if (s->n_inst == 1) e = cudaMemcpyAsync(st, s->d_status, sizeof(int) * 2, cudaMemcpyDeviceToHost, s->stream);
+    else if (s->d_flow) e = cudaMemcpyAsync(st + 1, s->d_status + s->n_inst, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
-    if (s->n_inst > 1 && !s->d_flow) return DUGKS_OK;
-    // the status of the instance (of a single sim) and the error word
-    const int first = s->n_inst > 1 ? s->n_inst : 0, n = s->n_inst + 1 - first;
-    int st[2] = {0, 0};
-    e = cudaMemcpy(st, s->d_status + first, sizeof(int) * n, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_status(e);
-    if (st[n - 1]) return DUGKS_ERR_TIMEOUT;
-    return n == 2 && (st[0] & ST_NONFINITE) ? DUGKS_ERR_NONFINITE : DUGKS_OK;
+    if (st[1]) return DUGKS_ERR_TIMEOUT;
+    return st[0] & ST_NONFINITE ? DUGKS_ERR_NONFINITE : DUGKS_OK;
+}
+
+// Start the check of n dense values on the device for a non-finite one, which sets
+// the refused word.
+cudaError_t check_input(dugks_sim *s, const double *v, long long n)
+{
+    cudaError_t e = cudaMemsetAsync(refused(s), 0, sizeof(int), s->stream);
+    if (e != cudaSuccess) return e;
+    const unsigned g = (unsigned)std::min<long long>(s->n_sm * 8, (n + 255) / 256);
+    Timed t(s, -1);
+    k_any_nonfinite<<<g, 256, 0, s->stream>>>(v, n, refused(s));
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -1153,8 +1156,8 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     // takes (the four-kernel step recomputes in place, and needs it all)
     const size_t keep_bytes = s->fused ? phi_bytes : state_bytes;
     constexpr int NC = 13;                             // cell planes of the adjoint
-    const size_t n_slot = (size_t)s->n_fseg + 2 * (size_t)s->n_cseg + 2 * n_tslot;
-    const size_t bytes = state_bytes * (size_t)(nck + nseg) + keep_bytes + sizeof(double) * (n_slot + (size_t)(4 * n + 2 * D))
+    const size_t n_slot = (size_t)s->n_fseg + 2 * (size_t)s->n_cseg + 2 * n_tslot, n_lslot = (size_t)s->n_tiles * TY;
+    const size_t bytes = state_bytes * (size_t)(nck + nseg) + keep_bytes + sizeof(double) * (n_slot + n_lslot + (size_t)(4 * n + 2 * D))
                        + sizeof(T) * ((size_t)N * (3 * 2 * Q + NC) + (size_t)NF * 2 * NFP) + 16 * 32;
     void *mem = nullptr;
     cudaError_t e = dmalloc(s, &mem, bytes);
@@ -1164,6 +1167,7 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     unsigned char *ckpt = take(state_bytes * (size_t)nck), *seg = take(state_bytes * (size_t)nseg);
     unsigned char *keep = take(keep_bytes);
     double *slots = (double *)take(sizeof(double) * n_slot), *pk = (double *)take(sizeof(double) * 2 * n);
+    double *loss_part = (double *)take(sizeof(double) * n_lslot);
     double *loss_d = (double *)take(sizeof(double) * n), *target = (double *)take(sizeof(double) * D);
     double *phi0b = (double *)take(sizeof(double) * D);
     int2 *trng_d = (int2 *)take(sizeof(int2) * n);
@@ -1193,14 +1197,13 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     const bool split = s->n_cseg <= 4 * s->n_sm;
     const unsigned fg = (unsigned)((s->n_fseg + fw - 1) / fw), cg = (unsigned)((s->n_cseg + cw - 1) / cw);
     // forward from the saved init inputs, with checkpoints
-    e = cudaMemcpyAsync(s->d_stage, s->d_init_in, sizeof(double) * 4 * D, cudaMemcpyDeviceToDevice, s->stream);
-    if (e == cudaSuccess) e = reset_status(s);
+    e = reset_status(s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(target, target_h, sizeof(double) * D, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(trng_d, trng.data(), sizeof(int2) * n, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(slots, 0, sizeof(double) * n_slot, s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss_d, 0, sizeof(double) * n, s->stream);
     if (e != cudaSuccess) rc = cuda_status(e);
-    if (!rc) rc = do_init<T>(s);
+    const double *const in[4] = {s->d_init_in, s->d_init_in + D, s->d_init_in + 2 * D, s->d_init_in + 3 * D};
+    if (!rc) rc = do_init<T>(s, in, nullptr);
     for (long c = 0; c < nck && !rc; c++) {
         copy(state(ckpt + state_bytes * (size_t)c), State<T>{P.f, P.phi});
         rc = dugks_step(s, std::min<long>(K, nsteps - c * K));
@@ -1210,8 +1213,9 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
         else copy(state(keep), State<T>{P.f, P.phi});
         // loss and the seed adjoint
         ka_seed<T><<<(unsigned)s->n_tiles, dim3(TX, TY), 0, s->stream>>>(s->d_inst, s->d_tiles, P, xb, xb + (size_t)Q * N, target,
-                                                                        s->d_dense0, loss_d);
-        s->launches++;
+                                                                        s->d_dense0, loss_part);
+        ka_loss<<<(unsigned)n, 256, 0, s->stream>>>(s->d_inst, loss_part, loss_d);
+        s->launches += 2;
     }
     // reverse sweep, one checkpoint segment at a time
     for (long c = nck - 1; c >= 0 && !rc; c--) {
@@ -1258,17 +1262,14 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     if (!rc) {
         const dim3 blk(TX, TY);
         const unsigned g = (unsigned)s->n_tiles;
-        k_unpack_phi<phi_t<T>><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in, P.phi, s->d_dense0);
-        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + D, P.ux, s->d_dense0);
-        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 2 * D, P.uy, s->d_dense0);
-        k_unpack<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, s->d_init_in + 3 * D, P.p, s->d_dense0);
+        k_unpack_init<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, in[0], in[1], in[2], in[3], P, nullptr, D, s->d_dense0, nullptr);
         k_mu<T><<<g, blk, 0, s->stream>>>(s->d_inst, s->d_tiles, geo, P);
         A.xf = xb; A.xg = xb + (size_t)Q * N;
         ka_init<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, P, A);
         ka_mu<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, P, A);
         ka_phi0<T><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, A, phi0b, s->d_dense0);
         ka_params<<<(unsigned)n, 256, 0, s->stream>>>(s->d_segrng, trng_d, A.lam_face, A.lam_cell, A.kap0, A.lam_macro, A.kap, pk);
-        s->launches += 9;
+        s->launches += 6;
         // leave the simulation at the final state of the forward run
         if (s->fused) cudaMemcpyAsync(P.phi, keep, phi_bytes, cudaMemcpyDeviceToDevice, s->stream);
         else copy(State<T>{P.f, P.phi}, state(keep));
@@ -1309,6 +1310,24 @@ double *host_alias(double *p)
     return a.type == cudaMemoryTypeHost ? static_cast<double *>(a.devicePointer) : nullptr;
 }
 
+}  // namespace
+
+namespace {
+// The end of a call that brought a new state (init: by dugks_init): unless it was
+// refused, what the many-step launches kept of the old one goes.
+int new_state(dugks_sim *s, bool init)
+{
+    int st[3] = {0, 0, 0};
+    const int first = s->n_inst == 1 ? 0 : 1;   // a single sim's status, then the error and the refused word
+    cudaError_t e = cudaMemcpyAsync(st + first, s->d_status + s->n_inst - 1 + first, sizeof(int) * (3 - first), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_status(e);
+    if (st[2]) return DUGKS_ERR_NONFINITE;
+    if (init) s->has_init = true;
+    e = reset_flow(s);
+    if (e != cudaSuccess) return cuda_status(e);
+    return st[0] & ST_NONFINITE ? DUGKS_ERR_NONFINITE : DUGKS_OK;
+}
 }  // namespace
 
 extern "C" {
@@ -1490,7 +1509,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
     chk(dmalloc(s, (void **)&s->d_phi_alt_alloc, sizeof(double) * (size_t)s->N));
     s->d_alt = s->d_alt_alloc;
     s->d_phi_alt = s->d_phi_alt_alloc;
-    chk(dmalloc(s, (void **)&s->d_status, sizeof(int) * (n + 1)));
+    chk(dmalloc(s, (void **)&s->d_status, sizeof(int) * (n + 2)));
     chk(dmalloc(s, (void **)&s->d_partials, sizeof(double2) * tiles.size()));
     // FP32 sims: the conservation sums' tile records and compact widths
     std::vector<RedTile> red;
@@ -1534,7 +1553,7 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
     chk(cudaMemset(s->d_phi, 0, sizeof(double) * (size_t)s->N));
     chk(cudaMemset(s->d_alt_alloc, 0, esz * 2 * Q * (size_t)s->N));
     chk(cudaMemset(s->d_phi_alt_alloc, 0, sizeof(double) * (size_t)s->N));
-    chk(cudaMemset(s->d_status, 0, sizeof(int) * (n + 1)));
+    chk(cudaMemset(s->d_status, 0, sizeof(int) * (n + 2)));
     if (e != cudaSuccess) {
         int rc = cuda_status(e);
         free_sim(s);
@@ -1562,32 +1581,19 @@ int dugks_init(dugks_sim *s, const double *phi, const double *ux, const double *
 {
     if (!s || !phi) return DUGKS_ERR_ARG;
     const long long D = s->n_dense;
-    const double *src[4] = {phi, ux, uy, p};
+    const double *src[4] = {phi, ux, uy, p}, *in[4];
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 4 && e == cudaSuccess; k++) {
+        in[k] = src[k] ? s->d_stage + k * D : nullptr;
         if (src[k]) e = cudaMemcpyAsync(s->d_stage + k * D, src[k], sizeof(double) * D, cudaMemcpyHostToDevice, s->stream);
-        else e = cudaMemsetAsync(s->d_stage + k * D, 0, sizeof(double) * D, s->stream);
     }
-    // a non-finite phi is refused before any state changes: checked on the
-    // uploaded copy (the staging buffer is scratch), the flag in the reduction
-    // scratch, which no call holds across this one
-    int *flag = reinterpret_cast<int *>(s->d_partials), bad = 0;
-    if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), s->stream);
-    if (e == cudaSuccess) {
-        { Timed t(s, -1); k_any_nonfinite<<<(unsigned)(s->n_sm * 8), 256, 0, s->stream>>>(s->d_stage, D, flag); }
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    // a non-finite phi is refused before any state changes: the uploaded copy is
+    // checked, and the kernels that would change the state ask the answer
+    if (e == cudaSuccess) e = check_input(s, s->d_stage, D);
     if (e != cudaSuccess) return cuda_status(e);
-    if (bad) return DUGKS_ERR_NONFINITE;
-    e = reset_status(s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->d_init_in, s->d_stage, sizeof(double) * 4 * D, cudaMemcpyDeviceToDevice, s->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-    int rc = s->prec == DUGKS_FP64 ? do_init<double>(s) : do_init<float>(s);
+    int rc = s->prec == DUGKS_FP64 ? do_init<double>(s, in, s->d_init_in) : do_init<float>(s, in, s->d_init_in);
     if (rc) return rc;
-    s->has_init = true;
-    return sync_status(s);
+    return new_state(s, true);
 }
 
 int dugks_step(dugks_sim *s, long nsteps)
@@ -1811,14 +1817,13 @@ int dugks_load(dugks_sim *s, const void *buf, size_t bytes)
     if (!s || !buf) return DUGKS_ERR_ARG;
     const size_t need = sizeof(double) * 2 * Q * (size_t)s->n_dense;
     if (bytes != need) return DUGKS_ERR_ARG;
-    const double *h = (const double *)buf;
-    for (size_t k = 0; k < need / sizeof(double); k++) if (!std::isfinite(h[k])) return DUGKS_ERR_NONFINITE;
+    // a non-finite value is refused before any state changes, as in dugks_init
     cudaError_t e = cudaMemcpyAsync(s->d_stage, buf, need, cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) e = reset_status(s);
+    if (e == cudaSuccess) e = check_input(s, s->d_stage, 2 * Q * s->n_dense);
     if (e != cudaSuccess) return cuda_status(e);
     int rc = s->prec == DUGKS_FP64 ? do_unpack_state<double>(s, s->d_stage) : do_unpack_state<float>(s, s->d_stage);
     if (rc) return rc;
-    return sync_status(s);
+    return new_state(s, false);
 }
 
 int dugks_launch_count(const dugks_sim *s, long *count)

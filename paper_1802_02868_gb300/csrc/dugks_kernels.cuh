@@ -231,16 +231,24 @@ __device__ __forceinline__ void grad_phi(const InstDev &I, const phi_t<T> *__res
 
 // ---------------------------------------------------------------------------
 // k_macro: grad mu, lap mu, grad phi, total force F = -phi grad mu + F_b, and
-// Eqs. (u), (P) from the tracked f.
+// Eqs. (u), (P) from the tracked f, into the planes; or (MOMENTS) phi, rho, ux, uy, p
+// as dense FP64 fields at out[0..4] (NULL to skip one), without the planes between: a
+// moments call was two kernels and one gather per field.
 // ---------------------------------------------------------------------------
-template <typename T>
+struct DenseOut {
+    double *out[5];
+    const long long *dense0;
+};
+
+template <typename T, bool MOMENTS>
 __global__ void __launch_bounds__(TX *TY) k_macro(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                  const AxisRecT<T> *__restrict__ geo, Planes<T> P, int write_rho)
+                                                  const AxisRecT<T> *__restrict__ geo, Planes<T> P, DenseOut D)
 {
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
-    if (P.status[t.x] & ST_NONFINITE) return;   // masked: non-finite instance of a batch (a paused one still gets its macros)
+    const bool masked = P.status[t.x] & ST_NONFINITE;   // non-finite instance of a batch (a paused one still gets its macros)
+    if (!MOMENTS && masked) return;
     const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
     if (i >= I.nx || j >= I.ny) return;
     const auto &ax = geo[I.gx_off + i];
@@ -270,15 +278,24 @@ __global__ void __launch_bounds__(TX *TY) k_macro(const InstDev *__restrict__ in
     T uy = (my + hdt * cs2 * Fy) / (cs2 * rho);
     T grx = Pr.drho * gfx, gry = Pr.drho * gfy;
     T p = sf + hdt * cs2 * (ux * grx + uy * gry - Pr.gamma * rho * Pr.lambda * lmu);
-    P.gmux[c] = gmx;
-    P.gmuy[c] = gmy;
-    P.lapmu[c] = lmu;
-    P.gphix[c] = gfx;
-    P.gphiy[c] = gfy;
-    P.ux[c] = ux;
-    P.uy[c] = uy;
-    P.p[c] = p;
-    if (write_rho) P.rho[c] = rho;
+    if constexpr (MOMENTS) {
+        const long long d = D.dense0[t.x] + (long long)j * I.nx + i;
+        if (masked) { ux = P.ux[c]; uy = P.uy[c]; p = P.p[c]; }   // what a kernel last left there
+        if (D.out[0]) D.out[0][d] = phi_to_double(P.phi[c]);
+        if (D.out[1]) D.out[1][d] = (double)rho;
+        if (D.out[2]) D.out[2][d] = (double)ux;
+        if (D.out[3]) D.out[3][d] = (double)uy;
+        if (D.out[4]) D.out[4][d] = (double)p;
+    } else {
+        P.gmux[c] = gmx;
+        P.gmuy[c] = gmy;
+        P.lapmu[c] = lmu;
+        P.gphix[c] = gfx;
+        P.gphiy[c] = gfy;
+        P.ux[c] = ux;
+        P.uy[c] = uy;
+        P.p[c] = p;
+    }
 }
 
 template <typename T>
@@ -596,15 +613,16 @@ __global__ void __launch_bounds__(TX *TY) k_face(const InstDev *__restrict__ ins
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(TX *TY) k_init(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                                                 const AxisRec *__restrict__ geo, Planes<T> P)
+                                                 const AxisRecT<T> *__restrict__ geo, Planes<T> P, const int *refused)
 {
+    if (*refused) return;
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
     const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
     if (i >= I.nx || j >= I.ny) return;
-    const AxisRec &ax = geo[I.gx_off + i];
-    const AxisRec &ay = geo[I.gy_off + j];
+    const AxisRecT<T> &ax = geo[I.gx_off + i];
+    const AxisRecT<T> &ay = geo[I.gy_off + j];
     const long long c = cell_of(I, i, j);
     const long long N = P.N;
     Pt<T> s;
@@ -805,27 +823,74 @@ __global__ void k_reduce_inst(const InstDev *__restrict__ insts, int n_inst, con
     out[k] = s;
 }
 
-// Gather the stored phi plane into a dense double array and back.
-template <typename S>
-__global__ void k_pack_phi(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, const S *__restrict__ src,
-                           double *__restrict__ dst, const long long *__restrict__ dense0)
+// Dense phi, ux, uy, p (NULL: zero) of the init inputs into the planes, into the
+// copy that the adjoint starts from (if any), and every instance's status to zero;
+// nothing of it when *refused is set (NULL: not asked).
+template <typename T>
+__global__ void __launch_bounds__(TX *TY) k_unpack_init(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
+                                                        const double *phi, const double *ux, const double *uy, const double *p,
+                                                        Planes<T> P, double *keep, long long n_dense,
+                                                        const long long *__restrict__ dense0, const int *refused)
 {
+    if (refused && *refused) return;
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
     if (i >= I.nx || j >= I.ny) return;
-    dst[dense0[t.x] + (long long)j * I.nx + i] = phi_to_double(src[cell_of(I, i, j)]);
+    const long long d = dense0[t.x] + (long long)j * I.nx + i, c = cell_of(I, i, j);
+    const double v0 = phi[d], v1 = ux ? ux[d] : 0.0, v2 = uy ? uy[d] : 0.0, v3 = p ? p[d] : 0.0;
+    phi_from_double(v0, P.phi[c]);
+    P.ux[c] = (T)v1;
+    P.uy[c] = (T)v2;
+    P.p[c] = (T)v3;
+    if (keep) {
+        keep[d] = v0;
+        keep[n_dense + d] = v1;
+        keep[2 * n_dense + d] = v2;
+        keep[3 * n_dense + d] = v3;
+        if (i == 0 && j == 0) P.status[t.x] = 0;
+    }
 }
 
-template <typename S>
-__global__ void k_unpack_phi(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
-                             const double *__restrict__ src, S *__restrict__ dst, const long long *__restrict__ dense0)
+// The tracked state as dense FP64 [2][9][n_dense], f first, and back, with phi = sum
+// g; one launch each for the 18 planes.  Not done when *refused is set.
+template <typename T>
+__global__ void __launch_bounds__(TX *TY) k_pack_state(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, Planes<T> P,
+                                                       double *__restrict__ dst, long long n_dense, const long long *__restrict__ dense0)
 {
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
     if (i >= I.nx || j >= I.ny) return;
-    phi_from_double(src[dense0[t.x] + (long long)j * I.nx + i], dst[cell_of(I, i, j)]);
+    const long long d = dense0[t.x] + (long long)j * I.nx + i, c = cell_of(I, i, j), N = P.N;
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        dst[q * n_dense + d] = (double)P.f[q * N + c];
+        dst[(Q + q) * n_dense + d] = (double)P.g[q * N + c];
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(TX *TY) k_unpack_state(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, Planes<T> P,
+                                                         const double *__restrict__ src, long long n_dense,
+                                                         const long long *__restrict__ dense0, const int *refused)
+{
+    if (*refused) return;
+    const int4 t = tiles[blockIdx.x];
+    const InstDev &I = insts[t.x];
+    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
+    if (i >= I.nx || j >= I.ny) return;
+    const long long d = dense0[t.x] + (long long)j * I.nx + i, c = cell_of(I, i, j), N = P.N;
+    double phi = 0;
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        P.f[q * N + c] = (T)src[q * n_dense + d];
+        const T g = (T)src[(Q + q) * n_dense + d];
+        P.g[q * N + c] = g;
+        phi += (double)g;
+    }
+    phi_from_double(phi, P.phi[c]);
+    if (i == 0 && j == 0) P.status[t.x] = 0;
 }
 
 // Set *flag (zeroed by the caller) when a[0..n) holds a non-finite value: the
@@ -837,31 +902,6 @@ __global__ void k_any_nonfinite(const double *__restrict__ a, long long n, int *
     for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
         bad |= !isfinite(a[c]);
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
-}
-
-// Gather a padded plane (type T) into a dense double array and back.
-template <typename T>
-__global__ void k_pack(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, const T *__restrict__ src,
-                       double *__restrict__ dst, const long long *__restrict__ dense0)
-{
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
-    const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
-    if (i >= I.nx || j >= I.ny) return;
-    dst[dense0[t.x] + (long long)j * I.nx + i] = (double)src[cell_of(I, i, j)];
-}
-
-template <typename T>
-__global__ void k_unpack(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles, const double *__restrict__ src,
-                         T *__restrict__ dst, const long long *__restrict__ dense0)
-{
-    const int4 t = tiles[blockIdx.x];
-    const InstDev &I = insts[t.x];
-    const ParT<T> &Pr = par<T>(I);
-    const int i = t.y + threadIdx.x, j = t.z + threadIdx.y;
-    if (i >= I.nx || j >= I.ny) return;
-    dst[cell_of(I, i, j)] = (T)src[dense0[t.x] + (long long)j * I.nx + i];
 }
 
 }  // namespace dugks
