@@ -2,6 +2,7 @@
 // validation, derived parameters, mesh geometry tables, the tile table of a
 // batch, device memory, and the launch sequence of one step.
 #include <cuda_runtime.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <climits>
@@ -1026,6 +1027,23 @@ cudaError_t check_input(dugks_sim *s, const double *v, long long n)
     return cudaGetLastError();
 }
 
+// Touch the pages of a host array that a copy from the device is about to fill, while
+// the device still works on what was enqueued before.  A pageable array of a few MB
+// fresh from the allocator has no pages yet, and where the device writes through the
+// host's page tables its copy then faults them in one by one: 5 fields of 2.1 MB took
+// 9.4 ms on GB300, 3.6 ms with the pages touched first on an idle device, 0.6 ms when
+// they are there.  Contents are kept (the atomic or of 0 is a write for the page
+// tables).  Above 4 MB, where numpy asks for huge pages, the copy's own faults are the
+// cheaper ones (33 MB: 2.5 ms, touched first 12.7 ms).
+void touch_pages(void *p, size_t bytes)
+{
+    static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    if (!p || bytes < 16 * page || bytes > (size_t(4) << 20)) return;
+    unsigned char *c = (unsigned char *)p;
+    for (size_t k = 0; k < bytes; k += page) __atomic_fetch_or(c + k, 0, __ATOMIC_RELAXED);
+    __atomic_fetch_or(c + bytes - 1, 0, __ATOMIC_RELAXED);
+}
+
 // ---------------------------------------------------------------------------
 // Adjoint: checkpointed forward, then the reverse sweep of dugks_adjoint.cuh
 // ---------------------------------------------------------------------------
@@ -1277,6 +1295,7 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     }
     std::vector<double> pkh(2 * n), loss(n);
     if (!rc) {
+        touch_pages(phi0b_h, sizeof(double) * D);
         e = cudaMemcpyAsync(pkh.data(), pk, sizeof(double) * 2 * n, cudaMemcpyDeviceToHost, s->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(loss.data(), loss_d, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream);
         if (e == cudaSuccess && phi0b_h) e = cudaMemcpyAsync(phi0b_h, phi0b, sizeof(double) * D, cudaMemcpyDeviceToHost, s->stream);
@@ -1621,6 +1640,8 @@ int dugks_moments(dugks_sim *s, double *phi, double *rho, double *ux, double *uy
     }
     int rc = s->prec == DUGKS_FP64 ? do_moments<double>(s, dst) : do_moments<float>(s, dst);
     if (rc) return rc;
+    for (int k = 0; k < 5; k++)
+        if (!alias[k]) touch_pages(out[k], sizeof(double) * D);
     for (int k = 0; k < 5; k++) {
         if (!out[k] || alias[k]) continue;
         cudaError_t e = cudaMemcpyAsync(out[k], dst[k], sizeof(double) * D, cudaMemcpyDeviceToHost, s->stream);
@@ -1658,6 +1679,7 @@ int dugks_laplace_pressure(dugks_sim *s, double *P)
     if (!s || !P) return DUGKS_ERR_ARG;
     int rc = s->prec == DUGKS_FP64 ? do_diag<double>(s, s->d_stage) : do_diag<float>(s, s->d_stage);
     if (rc) return rc;
+    if (!host_alias(P)) touch_pages(P, sizeof(double) * s->n_dense);
     cudaError_t e = cudaMemcpyAsync(P, s->d_stage, sizeof(double) * s->n_dense, cudaMemcpyDeviceToHost, s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     return sync_status(s);
@@ -1805,6 +1827,7 @@ int dugks_save(dugks_sim *s, void *buf, size_t *bytes)
     if (*bytes < need) return DUGKS_ERR_ARG;
     int rc = s->prec == DUGKS_FP64 ? do_pack_state<double>(s, s->d_stage) : do_pack_state<float>(s, s->d_stage);
     if (rc) return rc;
+    if (!host_alias((double *)buf)) touch_pages(buf, need);
     cudaError_t e = cudaMemcpyAsync(buf, s->d_stage, need, cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
