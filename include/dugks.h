@@ -111,7 +111,11 @@ int dugks_init(dugks_sim *sim, const double *phi, const double *ux, const double
 
 /* Steps 2-7 repeated nsteps times (Sec. 2.2; Eqs. relations1/2, fbar_h,
    original-function, microfluxf, updatef).  Asynchronous on the sim's stream;
-   a non-finite state is reported by the next synchronising call. */
+   a non-finite state is reported by the next synchronising call.  A call of 16
+   steps or more may run as one cooperative launch per 512 steps, whose tiles wait
+   for each other; a wait that runs out (seconds) is reported by the next
+   synchronising call as DUGKS_ERR_TIMEOUT, and the state is then undefined until
+   the next dugks_init or dugks_load. */
 int dugks_step(dugks_sim *sim, long nsteps);
 
 /* Macroscopic fields at the cell centres from the current state (Eqs. phi,
@@ -179,7 +183,8 @@ int dugks_load(dugks_sim *sim, const void *buf, size_t bytes);
    gradient is its exact transpose).
    The forward run is replayed from the saved init inputs with a checkpoint of
    the state every ckpt_every steps; each segment is recomputed and swept
-   backwards.  Outputs (host, each may be NULL): loss[n_instances],
+   backwards.  The recomputation keeps what the reverse steps read of every step of
+   a segment while that takes at most 4 GB and can be allocated.  Outputs (host, each may be NULL): loss[n_instances],
    dL_dphi0[cells] (the gradient with respect to the initial phi field, u0 and
    p0 held fixed), dL_dkappa[n_instances], dL_dlambda[n_instances] (lambda =
    the mobility).  phi_target: host array of all cells.  Allocates its
@@ -189,7 +194,8 @@ int dugks_load(dugks_sim *sim, const void *buf, size_t bytes);
 int dugks_adjoint(dugks_sim *sim, long nsteps, int ckpt_every, const double *phi_target, double *loss,
                   double *dL_dphi0, double *dL_dkappa, double *dL_dlambda);
 
-/* Counts kernel launches issued by this sim (for the caller's accounting). */
+/* Counts kernel launches issued by this sim (for the caller's accounting); a
+   launch of many steps counts once. */
 int dugks_launch_count(const dugks_sim *sim, long *count);
 
 /* Per-kernel timing with CUDA events on the sim's stream: enable (1) or

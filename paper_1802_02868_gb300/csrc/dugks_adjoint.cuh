@@ -682,37 +682,34 @@ __device__ __forceinline__ T stencil_t(const InstDev &I, const AxisRecT<T> *__re
     return s;
 }
 
-// Stencil transpose (see stencil_t) on a shared plane S of pitch W at entry e; st: the
-// step to the next position of the axis, r, rm, rp: the records of the position and of
-// its neighbours.
-template <typename T, int KIND>
-__device__ __forceinline__ T stencil_s(const T *S, int e, int st, const AxisRecT<T> &r, const AxisRecT<T> &rm, const AxisRecT<T> &rp,
-                                       bool hm, bool hp)
-{
-    T s = coef<T, KIND>(r, 0) * S[e];
-    s += hm ? coef<T, KIND>(rm, +1) * S[e - st] : coef<T, KIND>(r, -1) * S[e];
-    s += hp ? coef<T, KIND>(rp, -1) * S[e + st] : coef<T, KIND>(r, +1) * S[e];
-    return s;
-}
+// Coefficients of the stencil transposes (see stencil_t) at one position of an axis:
+// of the adjoint at the position before, after, and at the position itself, for the
+// first and the second derivative; z*: the position itself, the difference forms.
+template <typename T>
+struct TCoef {
+    T m1, p1, c1, z1, m2, p2, c2, z2;
+};
 
 // The rest of the step's transpose for a BX x BY tile per thread block, each on the
 // ring that the next one reads: grad p, then p, u, F (Eqs. u, P) on a 2-cell ring;
 // grad mu and lap mu, then mu = psi'(phi) - kappa lap(phi) (Eq. chemicalpotential) on
-// a 1-cell ring; grad phi and lap phi, then phi = sum g~ on the tile.  As three
-// kernels these took 14 + 7 + 11 us of a 256x512 FP32 step, most of it to add to planes
-// in memory one after the other.
+// a 1-cell ring; grad phi and lap phi, then phi = sum g~ on the tile.  The stencils'
+// coefficients and the adjoint of grad p are staged first, so that a phase has one
+// load latency and not a chain through the geometry records.
 template <typename T, int BX, int BY, int NT>
 __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
                                               const AxisRecT<T> *__restrict__ geo, Planes<T> P, AdjPlanes<T> Ad)
 {
-    constexpr int W2 = BX + 4, A2 = W2 * (BY + 4), W1 = BX + 2, A1 = W1 * (BY + 2);
-    __shared__ T gmx[A2], gmy[A2], lmu[A2], gfx[A2], gfy[A2], lph[A1], phb[BX * BY];
+    constexpr int W2 = BX + 4, H2 = BY + 4, A2 = W2 * H2, W1 = BX + 2, A1 = W1 * (BY + 2);
+    constexpr int WX = BX + 6, AX_ = WX * H2, AY_ = W2 * (BY + 6);
+    __shared__ T gmx[A2], gmy[A2], lmu[A2], gfx[A2], gfy[A2], lph[A1], phb[BX * BY], sgx[AX_], sgy[AY_];
+    __shared__ TCoef<T> tc[W2 + H2];
+    __shared__ int gi[W2 + H2];   // global index of positions -2 .. (-1 outside), columns then rows
     const int4 t = tiles[blockIdx.x];
     const InstDev &I = insts[t.x];
     const ParT<T> &Pr = par<T>(I);
     const int i0 = t.y, j0 = t.z, tid = threadIdx.x;
     const long long N = P.N;
-    // global index of a position (-1 outside)
     auto wrap = [](int g, int n, int bc) -> int {
         if (bc == 0) {
             while (g < 0) g += n;
@@ -721,15 +718,47 @@ __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts,
         }
         return g < 0 || g >= n ? -1 : g;
     };
+    for (int r = tid; r < AX_ + AY_; r += NT) {
+        const bool isx = r < AX_;
+        const int k = isx ? r : r - AX_, w = isx ? WX : W2;
+        const int i = wrap(i0 + k % w - (isx ? 3 : 2), I.nx, I.bcx), j = wrap(j0 + k / w - (isx ? 2 : 3), I.ny, I.bcy);
+        const T v = i >= 0 && j >= 0 ? (isx ? Ad.gpx : Ad.gpy)[cell_of(I, i, j)] : T(0);
+        (isx ? sgx : sgy)[k] = v;
+    }
+    for (int r = tid; r < W2 + H2; r += NT) {
+        const bool isx = r < W2;
+        const int g = isx ? wrap(i0 + r - 2, I.nx, I.bcx) : wrap(j0 + r - W2 - 2, I.ny, I.bcy);
+        gi[r] = g;
+        if (g < 0) continue;
+        const AxisRecT<T> &c = rec<T>(I, geo, isx ? 0 : 1, g), &m = rec<T>(I, geo, isx ? 0 : 1, c.km), &p = rec<T>(I, geo, isx ? 0 : 1, c.kp);
+        const bool hm = !c.lo_wall, hp = !c.hi_wall;   // a wall's ghost is the cell itself
+        TCoef<T> k;
+        const T s1 = (hm ? T(0) : c.c1m) + (hp ? T(0) : c.c1p), s2 = (hm ? T(0) : c.c2m) + (hp ? T(0) : c.c2p);
+        k.m1 = hm ? m.c1p : T(0);
+        k.p1 = hp ? p.c1m : T(0);
+        k.c1 = c.c10 + s1;
+        k.z1 = s1 - (c.c1m + c.c1p);
+        k.m2 = hm ? m.c2p : T(0);
+        k.p2 = hp ? p.c2m : T(0);
+        k.c2 = c.c20 + s2;
+        k.z2 = s2 - (c.c2m + c.c2p);
+        tc[r] = k;
+    }
+    __syncthreads();
     const T cs2 = Cst<T>::cs2, hdt = T(0.5) * Pr.dt;
     T lamb = 0, kapb = 0;
     for (int r = tid; r < A2; r += NT) {
         const int x = r % W2 - 2, y = r / W2 - 2;
-        const int i = wrap(i0 + x, I.nx, I.bcx), j = wrap(j0 + y, I.ny, I.bcy);
-        if (i < 0 || j < 0) continue;
+        const int i = gi[x + 2], j = gi[W2 + y + 2];
+        if (i < 0 || j < 0) {   // its neighbours read it with a zero coefficient
+            gmx[r] = gmy[r] = lmu[r] = gfx[r] = gfy[r] = T(0);
+            continue;
+        }
         const bool own = x >= 0 && x < BX && y >= 0 && y < BY && i0 + x < I.nx && j0 + y < I.ny;
         const long long c = cell_of(I, i, j);
-        const T pb = Ad.p[c] + stencil_t<T, 0>(I, geo, Ad.gpx, 0, i, j) + stencil_t<T, 0>(I, geo, Ad.gpy, 1, i, j);
+        const TCoef<T> &kx = tc[x + 2], &ky = tc[W2 + y + 2];
+        const T *sx = sgx + (y + 2) * WX + x + 3, *sy = sgy + (y + 3) * W2 + x + 2;
+        const T pb = Ad.p[c] + (kx.c1 * sx[0] + kx.m1 * sx[-1] + kx.p1 * sx[1]) + (ky.c1 * sy[0] + ky.m1 * sy[-W2] + ky.p1 * sy[W2]);
         T uxb = Ad.ux[c], uyb = Ad.uy[c];
         const T phi = T(phi_val(P.phi[c]));
         const T rho = Pr.rhoB + Pr.drho * (phi - Pr.phiB);
@@ -767,25 +796,30 @@ __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts,
     __syncthreads();
     for (int r = tid; r < A1; r += NT) {
         const int x = r % W1 - 1, y = r / W1 - 1;
-        const int i = wrap(i0 + x, I.nx, I.bcx), j = wrap(j0 + y, I.ny, I.bcy);
-        if (i < 0 || j < 0) continue;
+        const int i = gi[x + 2], j = gi[W2 + y + 2];
+        if (i < 0 || j < 0) {
+            lph[r] = T(0);
+            continue;
+        }
         const bool own = x >= 0 && x < BX && y >= 0 && y < BY && i0 + x < I.nx && j0 + y < I.ny;
         const long long c = cell_of(I, i, j);
-        const AxisRecT<T> &ax = rec<T>(I, geo, 0, i), &ay = rec<T>(I, geo, 1, j);
-        const AxisRecT<T> &axm = rec<T>(I, geo, 0, ax.km), &axp = rec<T>(I, geo, 0, ax.kp);
-        const AxisRecT<T> &aym = rec<T>(I, geo, 1, ay.km), &ayp = rec<T>(I, geo, 1, ay.kp);
-        const bool xm = !ax.lo_wall, xp = !ax.hi_wall, ym = !ay.lo_wall, yp = !ay.hi_wall;
+        const TCoef<T> &kx = tc[x + 2], &ky = tc[W2 + y + 2];
         const int e = (y + 2) * W2 + x + 2;
-        const T mub = Ad.mu[c] + stencil_s<T, 0>(gmx, e, 1, ax, axm, axp, xm, xp) + stencil_s<T, 0>(gmy, e, W2, ay, aym, ayp, ym, yp)
-                    + stencil_s<T, 2>(lmu, e, 1, ax, axm, axp, xm, xp) + stencil_s<T, 2>(lmu, e, W2, ay, aym, ayp, ym, yp);
+        const T mub = Ad.mu[c] + (kx.c1 * gmx[e] + kx.m1 * gmx[e - 1] + kx.p1 * gmx[e + 1])
+                    + (ky.c1 * gmy[e] + ky.m1 * gmy[e - W2] + ky.p1 * gmy[e + W2])
+                    + (kx.c2 * lmu[e] + kx.m2 * lmu[e - 1] + kx.p2 * lmu[e + 1])
+                    + (ky.c2 * lmu[e] + ky.m2 * lmu[e - W2] + ky.p2 * lmu[e + W2]);
         lph[r] = -Pr.kappa * mub;
         if (own) {
+            const AxisRecT<T> &ax = rec<T>(I, geo, 0, i), &ay = rec<T>(I, geo, 1, j);
             const phi_t<T> p0 = P.phi[c];
             const T phi = T(phi_val(p0));
             const T a = phi - Pr.phiA, b = phi - Pr.phiB, m = phi - T(0.5) * (Pr.phiA + Pr.phiB);
             const T d2psi = T(4) * Pr.beta * (b * m + a * m + a * b);
-            const T lap = (ax.c2m * phi_sub(P.phi[cell_of(I, ax.km, j)], p0) + ax.c2p * phi_sub(P.phi[cell_of(I, ax.kp, j)], p0))
-                        + (ay.c2m * phi_sub(P.phi[cell_of(I, i, ay.km)], p0) + ay.c2p * phi_sub(P.phi[cell_of(I, i, ay.kp)], p0));
+            const int im = ax.lo_wall ? i : gi[x + 1], ip = ax.hi_wall ? i : gi[x + 3];
+            const int jm = ay.lo_wall ? j : gi[W2 + y + 1], jp = ay.hi_wall ? j : gi[W2 + y + 3];
+            const T lap = (ax.c2m * phi_sub(P.phi[cell_of(I, im, j)], p0) + ax.c2p * phi_sub(P.phi[cell_of(I, ip, j)], p0))
+                        + (ay.c2m * phi_sub(P.phi[cell_of(I, i, jm)], p0) + ay.c2p * phi_sub(P.phi[cell_of(I, i, jp)], p0));
             phb[y * BX + x] += d2psi * mub;
             kapb -= lap * mub;
         }
@@ -795,13 +829,12 @@ __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts,
         const int x = r % BX, y = r / BX, i = i0 + x, j = j0 + y;
         if (i >= I.nx || j >= I.ny) continue;
         const long long c = cell_of(I, i, j);
-        const AxisRecT<T> &ax = rec<T>(I, geo, 0, i), &ay = rec<T>(I, geo, 1, j);
-        const AxisRecT<T> &axm = rec<T>(I, geo, 0, ax.km), &axp = rec<T>(I, geo, 0, ax.kp);
-        const AxisRecT<T> &aym = rec<T>(I, geo, 1, ay.km), &ayp = rec<T>(I, geo, 1, ay.kp);
-        const bool xm = !ax.lo_wall, xp = !ax.hi_wall, ym = !ay.lo_wall, yp = !ay.hi_wall;
+        const TCoef<T> &kx = tc[x + 2], &ky = tc[W2 + y + 2];
         const int e2 = (y + 2) * W2 + x + 2, e1 = (y + 1) * W1 + x + 1;
-        const T phib = phb[r] + stencil_s<T, 1>(gfx, e2, 1, ax, axm, axp, xm, xp) + stencil_s<T, 1>(gfy, e2, W2, ay, aym, ayp, ym, yp)
-                     + stencil_s<T, 3>(lph, e1, 1, ax, axm, axp, xm, xp) + stencil_s<T, 3>(lph, e1, W1, ay, aym, ayp, ym, yp);
+        const T phib = phb[r] + (kx.z1 * gfx[e2] + kx.m1 * gfx[e2 - 1] + kx.p1 * gfx[e2 + 1])
+                     + (ky.z1 * gfy[e2] + ky.m1 * gfy[e2 - W2] + ky.p1 * gfy[e2 + W2])
+                     + (kx.z2 * lph[e1] + kx.m2 * lph[e1 - 1] + kx.p2 * lph[e1 + 1])
+                     + (ky.z2 * lph[e1] + ky.m2 * lph[e1 - W1] + ky.p2 * lph[e1 + W1]);
 #pragma unroll
         for (int q = 0; q < Q; q++) Ad.ag[q * N + c] += phib;
     }

@@ -1084,12 +1084,12 @@ int ensure_segs(dugks_sim *s)
     return DUGKS_OK;
 }
 
-template <typename T, int BX, int BY, int NT>
+template <typename T, int BX, int BY, int NT, int MODE>
 int launch_planes_shape(dugks_sim *s, int k, const ToPlanes<T> &a)
 {
     using L = FusedLayout<T, BX, BY, false>;
     constexpr int MB = fused_minb<T, NT, false>();
-    auto f = k_step<T, BX, BY, NT, MB, false, false, MODE_PLANES>;
+    auto f = k_step<T, BX, BY, NT, MB, false, false, MODE>;
     static bool attr_set = false;
     if (!attr_set) {
         const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
@@ -1107,15 +1107,16 @@ int launch_planes_shape(dugks_sim *s, int k, const ToPlanes<T> &a)
 template <typename T>
 int adj_shape(const dugks_sim *s) { return sizeof(T) == 8 ? (s->tile0 >= 9 ? 9 : 7) : (s->tile0 == 8 ? 8 : 0); }
 
-// bar-plus and the cell fields of a state into the planes of P
-template <typename T>
+// bar-plus and the cell fields of a state into the planes of P; MODE_BOTH: and the
+// step after it
+template <typename T, int MODE>
 int launch_planes(dugks_sim *s, const ToPlanes<T> &a)
 {
     const int k = adj_shape<T>(s);
     if constexpr (sizeof(T) == 8)
-        return k == 9 ? launch_planes_shape<T, 8, 4, 128>(s, k, a) : launch_planes_shape<T, 16, 8, 128>(s, k, a);
+        return k == 9 ? launch_planes_shape<T, 8, 4, 128, MODE>(s, k, a) : launch_planes_shape<T, 16, 8, 128, MODE>(s, k, a);
     else
-        return k == 8 ? launch_planes_shape<T, 8, 8, 256>(s, k, a) : launch_planes_shape<T, 32, 8, 256>(s, k, a);
+        return k == 8 ? launch_planes_shape<T, 8, 8, 256, MODE>(s, k, a) : launch_planes_shape<T, 32, 8, 256, MODE>(s, k, a);
 }
 
 template <typename T>
@@ -1177,8 +1178,24 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     const size_t n_slot = (size_t)s->n_fseg + 2 * (size_t)s->n_cseg + 2 * n_tslot, n_lslot = (size_t)s->n_tiles * TY;
     const size_t bytes = state_bytes * (size_t)(nck + nseg) + keep_bytes + sizeof(double) * (n_slot + n_lslot + (size_t)(4 * n + 2 * D))
                        + sizeof(T) * ((size_t)N * (3 * 2 * Q + NC) + (size_t)NF * 2 * NFP) + 16 * 32;
+    // The recomputation of a segment forms what the reverse steps read (bar-plus and
+    // NR cell planes); it is kept for every step of the segment where that takes at
+    // most STORE_MAX and can be had, else formed again.
+    // FP32 256x512: the step that also writes them takes 33.4 us against 31.9, and saves
+    // the 20.6 us of MODE_PLANES (cold caches); 146 -> 134 us per step of a gradient,
+    // FP64 48x96 141 -> 130.
+    constexpr int NR = 11;
+    constexpr size_t STORE_MAX = size_t(4) << 30;
+    const size_t rec_bytes = sizeof(T) * (size_t)N * (2 * Q + NR);
+    const long nrec = std::min<long>(K, nsteps);
+    bool stored = s->fused && rec_bytes * (size_t)nrec <= STORE_MAX;
     void *mem = nullptr;
-    cudaError_t e = dmalloc(s, &mem, bytes);
+    cudaError_t e = dmalloc(s, &mem, bytes + (stored ? rec_bytes * (size_t)nrec : 0));
+    if (e != cudaSuccess && stored) {
+        cudaGetLastError();
+        stored = false;
+        e = dmalloc(s, &mem, bytes);
+    }
     if (e != cudaSuccess) return cuda_status(e);
     unsigned char *m = (unsigned char *)mem;
     auto take = [&](size_t b) { unsigned char *r = m; m += (b + 15) / 16 * 16; return r; };
@@ -1195,6 +1212,7 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     A.N = N;
     A.NF = NF;
     for (T *&f : A.face) f = (T *)take(sizeof(T) * (size_t)NF * NFP);
+    T *const recs = (T *)m;
     T **one[NC] = {&A.phi, &A.mu, &A.lapmu, &A.gmx, &A.gmy, &A.gfx, &A.gfy, &A.gpx, &A.gpy, &A.p, &A.ux, &A.uy, &A.lapphi};
     for (T **q : one) { *q = sc; sc += N; }
     A.lam_face = slots;
@@ -1238,11 +1256,34 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
     // reverse sweep, one checkpoint segment at a time
     for (long c = nck - 1; c >= 0 && !rc; c--) {
         const long len = std::min<long>(K, nsteps - c * K);
+        auto planes_of = [&](long k) {   // of step k of the segment: the state and where its fields go
+            const State<T> a = state(k == 0 ? ckpt + state_bytes * (size_t)c : seg + state_bytes * (size_t)(k - 1));
+            ToPlanes<T> tp;
+            tp.io = step_io<T>(s);
+            tp.io.f_in = a.f; tp.io.g_in = a.f + (size_t)Q * N; tp.io.phi_in = a.phi;
+            tp.P = P;
+            tp.P.f = a.f; tp.P.g = a.f + (size_t)Q * N; tp.P.phi = a.phi;
+            tp.P.fbp = fbp; tp.P.gbp = fbp + (size_t)Q * N;
+            if (stored) {
+                T *r = recs + rec_bytes / sizeof(T) * (size_t)k;
+                tp.P.fbp = r; tp.P.gbp = r + (size_t)Q * N;
+                r += (size_t)2 * Q * N;
+                T **f[NR] = {&tp.P.mu, &tp.P.lapmu, &tp.P.gmux, &tp.P.gmuy, &tp.P.gphix, &tp.P.gphiy, &tp.P.p, &tp.P.ux, &tp.P.uy,
+                             &tp.P.gpx, &tp.P.gpy};
+                for (T **q : f) { *q = r; r += N; }
+            }
+            return tp;
+        };
         auto at = [&](long k) { return state(k == 0 ? ckpt + state_bytes * (size_t)c : seg + state_bytes * (size_t)(k - 1)); };
         if (!s->fused && len > 1) copy(State<T>{P.f, P.phi}, at(0));
         for (long k = 0; k + 1 < len && !rc; k++) {
             const State<T> a = at(k), b = at(k + 1);
-            if (s->fused) {
+            if (stored) {
+                ToPlanes<T> tp = planes_of(k);
+                tp.io.f_out = b.f; tp.io.g_out = b.f + (size_t)Q * N; tp.io.phi_out = b.phi;
+                rc = launch_planes<T, MODE_BOTH>(s, tp);
+                s->launches++;
+            } else if (s->fused) {
                 StepIO<T> io = step_io<T>(s);
                 io.f_in = a.f; io.g_in = a.f + (size_t)Q * N; io.phi_in = a.phi;
                 io.f_out = b.f; io.g_out = b.f + (size_t)Q * N; io.phi_out = b.phi;
@@ -1255,23 +1296,20 @@ int adjoint_impl(dugks_sim *s, long nsteps, int K, const double *target_h, doubl
             }
         }
         for (long k = len - 1; k >= 0 && !rc; k--) {
-            const State<T> a = at(k);
-            ToPlanes<T> tp;
-            tp.io = step_io<T>(s);
-            tp.io.f_in = a.f; tp.io.g_in = a.f + (size_t)Q * N; tp.io.phi_in = a.phi;
-            tp.P = P;
-            tp.P.f = a.f; tp.P.g = a.f + (size_t)Q * N; tp.P.phi = a.phi;
-            tp.P.fbp = fbp; tp.P.gbp = fbp + (size_t)Q * N;
+            const ToPlanes<T> tp = planes_of(k);
             const Planes<T> &R = tp.P;
-            rc = launch_planes<T>(s, tp);
-            if (rc) break;
+            if (!stored || k == len - 1) {
+                rc = launch_planes<T, MODE_PLANES>(s, tp);
+                s->launches++;
+                if (rc) break;
+            }
             A.xf = xb; A.xg = xb + (size_t)Q * N;
             A.af = xn; A.ag = xn + (size_t)Q * N;
             ka_face<T><<<fg, 32 * fw, 0, s->stream>>>(s->d_inst, s->d_fseg, s->n_fseg, geo, R, A);
             if (split) ka_cell<T, true><<<(unsigned)s->n_cseg, 128, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, R, A);
             else ka_cell<T, false><<<cg, 32 * cw, 0, s->stream>>>(s->d_inst, s->d_cseg, s->n_cseg, geo, R, A);
             launch_tail<T>(s, R, A);
-            s->launches += 4;
+            s->launches += 3;
             std::swap(xb, xn);
             rc = cuda_status(cudaGetLastError());
         }

@@ -374,16 +374,17 @@ struct Flow {
     int *err;                  // set when a wait ran out
     unsigned limit;            // polls before a wait gives up
 };
-// What k_step does: one step; many steps; or the step up to bar-plus, whose cell
-// fields and bar-plus go to the planes P (for the adjoint's reverse step).
-constexpr int MODE_STEP = 0, MODE_FLOW = 1, MODE_PLANES = 2;
+// What k_step does: one step; many steps; the step up to bar-plus, whose cell
+// fields and bar-plus go to the planes P (for the adjoint's reverse step); or that and
+// the step.
+constexpr int MODE_STEP = 0, MODE_FLOW = 1, MODE_PLANES = 2, MODE_BOTH = 3;
 template <typename T>
 struct ToPlanes {
     StepIO<T> io;
     Planes<T> P;
 };
 template <typename T, int MODE>
-using step_arg = std::conditional_t<MODE == MODE_FLOW, Flow<T>, std::conditional_t<MODE == MODE_PLANES, ToPlanes<T>, StepIO<T>>>;
+using step_arg = std::conditional_t<MODE == MODE_FLOW, Flow<T>, std::conditional_t<MODE >= MODE_PLANES, ToPlanes<T>, StepIO<T>>>;
 template <typename T>
 __device__ __forceinline__ const StepIO<T> &step_io_of(const StepIO<T> &io, int) { return io; }
 template <typename T>
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
                                                    const AxisRecT<T> *__restrict__ geo,
                                                    const __grid_constant__ step_arg<T, MODE> arg)
 {
-    constexpr bool FLOW = MODE == MODE_FLOW, PLANES = MODE == MODE_PLANES;
+    constexpr bool FLOW = MODE == MODE_FLOW, PLANES = MODE == MODE_PLANES || MODE == MODE_BOTH;
     static_assert(NT % 32 == 0 && NT >= BX * BY, "thread count");
     using TL = Tile<T, BX, BY, UNI, SEP>;
     using L = typename TL::L;
@@ -770,7 +771,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
             }
         }
     }
-    if (PLANES) break;
+    if (MODE == MODE_PLANES) break;
 
     // ---- phase 5: every face of the tile once (x faces first in the item space)
     for (int k = tid; k < L::NFT; k += NT) {

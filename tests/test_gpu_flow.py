@@ -82,3 +82,24 @@ def test_batches_with_paused_and_nonfinite_instances():
     fa, fb = a.state(), b.state()
     keep = np.r_[0:o, o + k:a.ncells]
     assert all(np.array_equal(x[:, keep], y[:, keep]) for x, y in zip(fa, fb))
+
+
+def test_two_sims_on_two_streams_and_threads():
+    """Many-step launches of two sims in flight at once, from two host threads."""
+    import threading
+
+    import torch
+    cs = [I.stationary_drop(n=96, radius=24.0), I.rayleigh_taylor(nx=128, ny=256)]
+    streams = [torch.cuda.Stream() for _ in cs]
+    sims = [dugks.Sim(c.mesh, c.params, dugks.FP32, stream=st.cuda_stream).init(c.phi0) for c, st in zip(cs, streams)]
+    ts = [threading.Thread(target=lambda s=s: [s.step(40) for _ in range(10)]) for s in sims]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    for c, s in zip(cs, sims):
+        ref = dugks.Sim(c.mesh, c.params, dugks.FP32).init(c.phi0)
+        for _ in range(40):
+            ref.step(10)
+        for x, y in zip(s.state(), ref.state()):
+            assert np.array_equal(x, y)
