@@ -465,6 +465,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         }
         if (st & ST_NONFINITE) break;   // masked: non-finite instance of a batch
         if (!PLANES && (st & ST_PAUSED)) {   // paused: the state passes to the other buffer unchanged
+            if (FLOW && step > 0) break;      // and is in both after the first step
             const int x = tid % BX, y = tid / BX;
             if (tid < BX * BY && i0 + x < I.nx && j0 + y < I.ny) {
                 const long long c = I.cell0 + (long long)(j0 + y) * I.nxp + (i0 + x);
