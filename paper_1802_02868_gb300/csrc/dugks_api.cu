@@ -650,17 +650,19 @@ int ensure_flow(dugks_sim *s, int k)
     }
     cudaError_t e = dmalloc(s, (void **)&F.nbr, sizeof(int) * nbr.size());
     if (e == cudaSuccess) e = dmalloc(s, (void **)&F.done, sizeof(unsigned) * first);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(F.nbr, nbr.data(), sizeof(int) * nbr.size(), cudaMemcpyHostToDevice, s->stream);
+    // (a plain copy: the list goes out of scope with this call)
+    if (e == cudaSuccess) e = cudaMemcpy(F.nbr, nbr.data(), sizeof(int) * nbr.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemsetAsync(F.done, 0, sizeof(unsigned) * first, s->stream);
     if (e != cudaSuccess) {
         dfree(s, F.nbr);
         dfree(s, F.done);
         F.nbr = nullptr;
         F.done = nullptr;
+        return cuda_status(e);
     }
     F.base = 0;
     s->any_flow = true;
-    return cuda_status(e);
+    return DUGKS_OK;
 }
 
 template <typename T, int BX, int BY, int NT>
