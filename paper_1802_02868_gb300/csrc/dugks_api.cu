@@ -170,6 +170,34 @@ void dfree(dugks_sim *s, void *p)
     else cudaFree(p);
 }
 
+// The stream on which a sim's tables and first values are written: its own, so that
+// the writes come after whatever used the memory before (an allocator may hand out
+// blocks in stream order) and before the kernels that read them.  The legacy stream of
+// a plain cudaMemcpy has neither order with a non-blocking stream.  While the caller
+// captures the sim's stream, a private one: a table is not part of the captured work.
+cudaError_t table_stream(dugks_sim *s, cudaStream_t *st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    *st = s->stream;
+    if (cudaStreamIsCapturing(s->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return cudaSuccess;
+    cudaGetLastError();
+    if (!s->cap_stream) {
+        const cudaError_t e = cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+    }
+    *st = s->cap_stream;
+    return cudaSuccess;
+}
+
+// Copy a host table, which may go out of scope with the call, to the device.
+cudaError_t upload(dugks_sim *s, void *dst, const void *src, size_t bytes)
+{
+    cudaStream_t st;
+    cudaError_t e = table_stream(s, &st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
 
 int validate(const dugks_mesh &m, const dugks_params &p)
@@ -437,7 +465,7 @@ int ensure_tiles(dugks_sim *s, int k)
         if (pass == 0) s->n_uni_s[k] = (int)tiles.size();
     }
     cudaError_t e = dmalloc(s, (void **)&s->d_tiles_s[k], sizeof(int4) * tiles.size());
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_tiles_s[k], tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(s, s->d_tiles_s[k], tiles.data(), sizeof(int4) * tiles.size());
     if (e != cudaSuccess) {
         dfree(s, s->d_tiles_s[k]);
         s->d_tiles_s[k] = nullptr;
@@ -650,8 +678,7 @@ int ensure_flow(dugks_sim *s, int k)
     }
     cudaError_t e = dmalloc(s, (void **)&F.nbr, sizeof(int) * nbr.size());
     if (e == cudaSuccess) e = dmalloc(s, (void **)&F.done, sizeof(unsigned) * first);
-    // (a plain copy: the list goes out of scope with this call)
-    if (e == cudaSuccess) e = cudaMemcpy(F.nbr, nbr.data(), sizeof(int) * nbr.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(s, F.nbr, nbr.data(), sizeof(int) * nbr.size());
     if (e == cudaSuccess) e = cudaMemsetAsync(F.done, 0, sizeof(unsigned) * first, s->stream);
     if (e != cudaSuccess) {
         dfree(s, F.nbr);
@@ -866,8 +893,8 @@ int ensure_strips8(dugks_sim *s)
     }
     cudaError_t e = dmalloc(s, (void **)&s->d_strips8, sizeof(int4) * st.size());
     if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_strip_rng, sizeof(int2) * rng.size());
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_strips8, st.data(), sizeof(int4) * st.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_strip_rng, rng.data(), sizeof(int2) * rng.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(s, s->d_strips8, st.data(), sizeof(int4) * st.size());
+    if (e == cudaSuccess) e = upload(s, s->d_strip_rng, rng.data(), sizeof(int2) * rng.size());
     if (e != cudaSuccess) {
         dfree(s, s->d_strips8);
         dfree(s, s->d_strip_rng);
@@ -1082,9 +1109,9 @@ int ensure_segs(dugks_sim *s)
     cudaError_t e = dmalloc(s, (void **)&s->d_fseg, sizeof(AdjSeg) * fs.size());
     if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_segrng, sizeof(int4) * rng.size());
     if (e == cudaSuccess) e = dmalloc(s, (void **)&s->d_cseg, sizeof(AdjSeg) * cs.size());
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_fseg, fs.data(), sizeof(AdjSeg) * fs.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_segrng, rng.data(), sizeof(int4) * rng.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->d_cseg, cs.data(), sizeof(AdjSeg) * cs.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(s, s->d_fseg, fs.data(), sizeof(AdjSeg) * fs.size());
+    if (e == cudaSuccess) e = upload(s, s->d_segrng, rng.data(), sizeof(int4) * rng.size());
+    if (e == cudaSuccess) e = upload(s, s->d_cseg, cs.data(), sizeof(AdjSeg) * cs.size());
     if (e != cudaSuccess) {
         dfree(s, s->d_cseg);
         dfree(s, s->d_fseg);
@@ -1611,20 +1638,23 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         free_sim(s);
         return rc;
     }
-    chk(cudaMemcpy(s->d_inst, s->h_inst.data(), sizeof(InstDev) * n, cudaMemcpyHostToDevice));
-    chk(cudaMemcpy(s->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice));
-    chk(cudaMemcpy(s->d_geo, geo.data(), sizeof(AxisRec) * geo.size(), cudaMemcpyHostToDevice));
-    chk(cudaMemcpy(s->d_geoT, is64 ? (const void *)g64.data() : (const void *)g32.data(), geoT_bytes, cudaMemcpyHostToDevice));
-    chk(cudaMemcpy(s->d_dense0, s->h_dense0.data(), sizeof(long long) * n, cudaMemcpyHostToDevice));
+    chk(upload(s, s->d_inst, s->h_inst.data(), sizeof(InstDev) * n));
+    chk(upload(s, s->d_tiles, tiles.data(), sizeof(int4) * tiles.size()));
+    chk(upload(s, s->d_geo, geo.data(), sizeof(AxisRec) * geo.size()));
+    chk(upload(s, s->d_geoT, is64 ? (const void *)g64.data() : (const void *)g32.data(), geoT_bytes));
+    chk(upload(s, s->d_dense0, s->h_dense0.data(), sizeof(long long) * n));
     if (!is64) {
-        chk(cudaMemcpy(s->d_red, red.data(), sizeof(RedTile) * red.size(), cudaMemcpyHostToDevice));
-        chk(cudaMemcpy(s->d_redgeo, redgeo.data(), sizeof(float2) * redgeo.size(), cudaMemcpyHostToDevice));
+        chk(upload(s, s->d_red, red.data(), sizeof(RedTile) * red.size()));
+        chk(upload(s, s->d_redgeo, redgeo.data(), sizeof(float2) * redgeo.size()));
     }
-    chk(cudaMemset(s->d_planes, 0, esz * plane_elems));
-    chk(cudaMemset(s->d_phi, 0, sizeof(double) * (size_t)s->N));
-    chk(cudaMemset(s->d_alt_alloc, 0, esz * 2 * Q * (size_t)s->N));
-    chk(cudaMemset(s->d_phi_alt_alloc, 0, sizeof(double) * (size_t)s->N));
-    chk(cudaMemset(s->d_status, 0, sizeof(int) * (n + 2)));
+    cudaStream_t st = nullptr;
+    chk(table_stream(s, &st));
+    chk(cudaMemsetAsync(s->d_planes, 0, esz * plane_elems, st));
+    chk(cudaMemsetAsync(s->d_phi, 0, sizeof(double) * (size_t)s->N, st));
+    chk(cudaMemsetAsync(s->d_alt_alloc, 0, esz * 2 * Q * (size_t)s->N, st));
+    chk(cudaMemsetAsync(s->d_phi_alt_alloc, 0, sizeof(double) * (size_t)s->N, st));
+    chk(cudaMemsetAsync(s->d_status, 0, sizeof(int) * (n + 2), st));
+    if (st != s->stream) chk(cudaStreamSynchronize(st));
     if (e != cudaSuccess) {
         int rc = cuda_status(e);
         free_sim(s);
@@ -1805,8 +1835,7 @@ int rewrite_paused(dugks_sim *s, const std::vector<char> &paused)
     if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     for (int k = 0; k < s->n_inst; k++) st[k] = (st[k] & ~ST_PAUSED) | (paused[k] ? ST_PAUSED : 0);
-    e = cudaMemcpy(s->d_status, st.data(), sizeof(int) * s->n_inst, cudaMemcpyHostToDevice);
-    return cuda_status(e);
+    return cuda_status(upload(s, s->d_status, st.data(), sizeof(int) * s->n_inst));
 }
 
 // the tile of shape 0 for the instances that are not paused

@@ -1,0 +1,109 @@
+"""The library's host code on a stand-in for the CUDA runtime that keeps "device"
+memory on the host, runs no kernel and records what is ordered on which stream
+(host_calls/recording_cudart.cpp): which stream every table goes to, and what the
+calls report.  No GPU is needed."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1802_02868_gb300 import build, dugks
+from paper_1802_02868_gb300 import inputs as I
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+STREAM = 0x5550   # what the calls get as the caller's stream: never dereferenced
+
+
+class Recorder:
+    def __init__(self, lib):
+        self.lib = lib
+        lib.rec_op.restype = ctypes.c_char_p
+        for n in ("rec_count", "rec_coop_launches"):
+            getattr(lib, n).restype = ctypes.c_long
+        for n in ("rec_dst", "rec_bytes", "rec_stream", "rec_unreachable"):
+            getattr(lib, n).restype = ctypes.c_ulonglong
+        lib.rec_unreachable.argtypes = [ctypes.c_size_t]
+        lib.rec_set_late.argtypes = [ctypes.c_ulonglong]
+
+    def calls(self, fn):
+        """What fn() put on the streams: (operation, destination, bytes, stream)."""
+        L = self.lib
+        L.rec_clear()
+        fn()
+        return [(L.rec_op(k).decode(), L.rec_dst(k), L.rec_bytes(k), L.rec_stream(k)) for k in map(ctypes.c_long, range(L.rec_count()))]
+
+
+@pytest.fixture(scope="module")
+def recording_library(tmp_path_factory):
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")))
+    if not shutil.which("g++") or not os.path.isdir(os.path.join(cuda, "include")):
+        pytest.skip("no host compiler or CUDA headers")
+    build.build()
+    objs = sorted(glob.glob(os.path.join(build.BUILD_DIR, "dugks_*.o")))
+    out = str(tmp_path_factory.mktemp("rec") / "libdugks_recording.so")
+    r = subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-I", os.path.join(cuda, "include"), "-Wl,-Bsymbolic",
+                        "-Wl,--no-undefined", os.path.join(HERE, "host_calls", "recording_cudart.cpp")] + objs + ["-o", out],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return out
+
+
+@pytest.fixture
+def rec(recording_library, monkeypatch):
+    monkeypatch.setattr(build, "LIB", recording_library)
+    monkeypatch.setattr(dugks, "_lib", None)
+    r = Recorder(dugks.load())
+    yield r
+    r.lib.rec_set_capturing(0)
+    r.lib.rec_set_late(0)
+
+
+def _drops(sizes, prec, stream=STREAM):
+    cs = [I.stationary_drop(n=n, radius=0.25 * n) for n in sizes]
+    s = dugks.Sim([c.mesh for c in cs], [c.params for c in cs], prec, stream=stream)
+    return s, [c.phi0 for c in cs]
+
+
+@pytest.mark.parametrize("prec", [dugks.FP64, dugks.FP32])
+@pytest.mark.parametrize("sizes", [(64,), (24, 41, 64)])
+def test_tables_and_status_are_written_on_the_sims_stream(rec, sizes, prec):
+    """A non-blocking stream has no order with the legacy stream of a plain copy:
+    every write goes to the sim's stream, and the host waits on that stream for a
+    copy out of its own memory before the call returns."""
+    made = []
+    log = [rec.calls(lambda: made.append(_drops(sizes, prec)))]
+    s, phi = made[0]
+    with s:
+        log.append(rec.calls(lambda: s.init(phi)))
+        log.append(rec.calls(lambda: s.step(64)))          # the many-step launch's tables
+        assert any(op.startswith("cooperative") for op, *_ in log[-1])
+        log.append(rec.calls(lambda: s.step(3)))
+        log.append(rec.calls(lambda: s.set_tile_shape(5)))
+        log.append(rec.calls(s.diagnostics_array))
+        log.append(rec.calls(lambda: s.set_paused([k == 0 for k in range(len(sizes))])))
+        log.append(rec.calls(lambda: s.set_paused([False] * len(sizes))))
+        log.append(rec.calls(lambda: s.step_each([20 + k for k in range(len(sizes))])))
+        log.append(rec.calls(lambda: s.adjoint(3, phi)))
+    for calls in log:
+        writes = [k for k, c in enumerate(calls) if c[0] == "copy h2d" or c[0] == "memset"]
+        assert all(calls[k][3] == STREAM for k in writes), [calls[k] for k in writes]
+        up = [k for k in writes if calls[k][0] == "copy h2d"]
+        if up:
+            assert any(c[0] == "sync" and c[3] == STREAM for c in calls[up[-1] + 1:])
+    assert sum(c[0] == "copy h2d" for c in sum(log, [])) >= 15
+
+
+def test_a_table_made_while_the_caller_captures_stays_out_of_the_capture(rec):
+    s, phi = _drops((64,), dugks.FP32)
+    with s:
+        s.init(phi)
+        rec.lib.rec_set_capturing(1)
+        calls = rec.calls(lambda: s.step(1))               # the first step makes the tile table
+        up = [c for c in calls if c[0] == "copy h2d"]
+        assert len(up) == 1 and up[0][3] not in (0, STREAM)
+        assert ("sync", 0, 0, up[0][3]) in calls
+        assert not any(c[0] == "sync" and c[3] == STREAM for c in calls)
