@@ -456,28 +456,28 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
     const StepIO<T> &io = step_io_of<T>(arg, step);
     const int i0 = t.y, j0 = t.z;
     do {   // left by the threads that have nothing more to do for the tile
-    {
-        int st;
-        if constexpr (FLOW) {
-            st = s_status;
-        } else {
-            st = io.status[t.x];
-        }
-        if (st & ST_NONFINITE) break;   // masked: non-finite instance of a batch
-        if (!PLANES && (st & ST_PAUSED)) {   // paused: the state passes to the other buffer unchanged
-            if (FLOW && step > 0) break;      // and is in both after the first step
-            const int x = tid % BX, y = tid / BX;
-            if (tid < BX * BY && i0 + x < I.nx && j0 + y < I.ny) {
-                const long long c = I.cell0 + (long long)(j0 + y) * I.nxp + (i0 + x);
+    int st;
+    if constexpr (FLOW) {
+        st = s_status;
+    } else {
+        st = io.status[t.x];
+    }
+    // paused: the state passes to the other buffer unchanged (a paused instance does
+    // not step, so all its threads read the same word)
+    if (!PLANES && (st & ST_PAUSED)) {
+        if (st & ST_NONFINITE) break;
+        if (FLOW && step > 0) break;      // it is in both after the first step
+        const int x = tid % BX, y = tid / BX;
+        if (tid < BX * BY && i0 + x < I.nx && j0 + y < I.ny) {
+            const long long c = I.cell0 + (long long)(j0 + y) * I.nxp + (i0 + x);
 #pragma unroll
-                for (int q = 0; q < Q; q++) {
-                    io.f_out[q * io.N + c] = io.f_in[q * io.N + c];
-                    io.g_out[q * io.N + c] = io.g_in[q * io.N + c];
-                }
-                io.phi_out[c] = io.phi_in[c];
+            for (int q = 0; q < Q; q++) {
+                io.f_out[q * io.N + c] = io.f_in[q * io.N + c];
+                io.g_out[q * io.N + c] = io.g_in[q * io.N + c];
             }
-            break;
+            io.phi_out[c] = io.phi_in[c];
         }
+        break;
     }
     const long long N = io.N;
 
@@ -496,7 +496,15 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ i
         }
         S.gg[r] = g;
     }
-    if (fresh) __syncthreads();
+    // masked: non-finite instance of a batch.  Another block of the instance may set
+    // the bit while this one starts, so its threads agree on one answer: some leaving
+    // and some not would leave holes in what the phases share (the indices above).
+    if constexpr (FLOW) {
+        if (fresh) __syncthreads();
+        if (st & ST_NONFINITE) break;
+    } else {
+        if (__syncthreads_or(st & ST_NONFINITE)) break;
+    }
     auto gpos = [&](bool isx, int pos) -> int { return S.gg[isx ? pos + 4 : L::W4 + pos + 4]; };
     auto cell = [&](int gi, int gj) -> long long { return I.cell0 + (long long)gj * I.nxp + gi; };
 

@@ -80,7 +80,9 @@ __global__ void __launch_bounds__(NT, MINB) k_strip(const InstDev *__restrict__ 
     auto cell = [&](int gi, int gj) -> long long { return I.cell0 + (long long)gj * I.nxp + gi; };
     {
         const int st = io.status[t.x];
-        if (st & ST_NONFINITE) return;   // masked: non-finite instance of a batch
+        // masked: non-finite instance of a batch; one answer for the whole block, for
+        // another block of the instance may set the bit meanwhile
+        if (__syncthreads_or(st & ST_NONFINITE)) return;
         if (st & ST_PAUSED) {            // paused: the state passes to the other buffer unchanged
             for (int r = tid; r < BX * BY * nblk; r += NT) {
                 const int gi = i0 + r % BX, gj = j0 + r / BX;
