@@ -16,6 +16,9 @@
 //   rho)) for f, both xi.(c fg (F - grad p)) for g (Eqs. feq, geq, F, G with
 //   (xi - u).X = xi.X - u.X); the weight of the diagonals is part of b and c;
 // - one reciprocal of rho (6K + X) serves 1/rho and the f weights;
+// - sums start from their small terms (flux sums, sources, tangential derivatives)
+//   and end with the one product as large as the result, so that a value is rounded
+//   at its own size once or twice and not after each term;
 // - face values are stored without the face area, which the update cancels
 //   against the cell volume;
 // - grad mu, grad phi, lap mu and u of the p phase are kept for the bar-plus
@@ -164,11 +167,11 @@ __device__ __forceinline__ void pair_of(double a, double A, double D, double Bx,
     const double X = q == 1 ? Ex : q == 2 ? Ey : q == 5 ? ad(Ex, Ey) : sb(Ey, Ex);
     const double ev = fm(t, X, fm(s, D, A)), od = fm(t, D, fm(s, X, B));
     if (q < 5) {   // the axis weight is four times the diagonals'
-        o0 = fm(4.0, ad(ev, od), mu(a, v0));
-        o1 = fm(4.0, sb(ev, od), mu(a, v1));
+        o0 = fm(a, v0, mu(4.0, ad(ev, od)));
+        o1 = fm(a, v1, mu(4.0, sb(ev, od)));
     } else {
-        o0 = ad(fm(a, v0, ev), od);
-        o1 = sb(fm(a, v1, ev), od);
+        o0 = fm(a, v0, ad(ev, od));
+        o1 = fm(a, v1, sb(ev, od));
     }
 }
 template <int q>
@@ -185,7 +188,7 @@ __device__ __forceinline__ void pair_g(const PtC<double> &C, const Eq &E, double
 // bar-plus of f or g at a cell (Eq. relations1), in place of the nine values
 __device__ __forceinline__ void bar_plus_f(const Eq &E, double (&v)[Q])
 {
-    v[0] = fm(16.0, fm(E.s0, E.K1, E.K0), mu(E.a, v[0]));
+    v[0] = fm(E.a, v[0], mu(16.0, fm(E.s0, E.K1, E.K0)));
     pair_f<1>(E, v[1], v[3], v[1], v[3]);
     pair_f<2>(E, v[2], v[4], v[2], v[4]);
     pair_f<5>(E, v[5], v[7], v[5], v[7]);
@@ -194,8 +197,8 @@ __device__ __forceinline__ void bar_plus_f(const Eq &E, double (&v)[Q])
 __device__ __forceinline__ void bar_plus_g(const PtC<double> &C, const Eq &E, double phi, double m, double (&v)[Q])
 {
     // the rest direction's H is phi - (1 - w_0) eta mu
-    const double rest = fm(C.gb36, phi, fm(-C.gbe36, m, mu(C.ga, v[0])));
-    v[0] = fm(16.0, fm(E.s0, E.D2, E.A2), rest);
+    const double rest = fm(-C.gbe36, m, mu(16.0, fm(E.s0, E.D2, E.A2)));
+    v[0] = fm(C.ga, v[0], fm(C.gb36, phi, rest));
     pair_g<1>(C, E, v[1], v[3], v[1], v[3]);
     pair_g<2>(C, E, v[2], v[4], v[2], v[4]);
     pair_g<5>(C, E, v[5], v[7], v[5], v[7]);
@@ -374,15 +377,17 @@ __device__ __forceinline__ void face(const InstDev &I, const TL &S, int xa, int 
                 cL = t > 0 ? sb(cL, L0) : ad(cL, L0);
                 cR = t > 0 ? sb(cR, R0) : ad(cR, R0);
             }
-            double vf = fm(cL, bL.x, mu(cR, bR.x)), vg = fm(cL, bL.y, mu(cR, bR.y));
             if (t) {
                 const double2 a0 = B[ia + tm], a1 = B[ia + tp], b0 = B[ib + tm], b1 = B[ib + tp];
                 const double l0 = t > 0 ? -Lmt : Lmt, l1 = t > 0 ? -Lpt : Lpt, r0 = t > 0 ? -Rmt : Rmt, r1 = t > 0 ? -Rpt : Rpt;
-                vf = fm(l0, a0.x, fm(l1, a1.x, fm(r0, b0.x, fm(r1, b1.x, vf))));
-                vg = fm(l0, a0.y, fm(l1, a1.y, fm(r0, b0.y, fm(r1, b1.y, vg))));
+                const double df = fm(l0, a0.x, fm(l1, a1.x, fm(r0, b0.x, mu(r1, b1.x))));
+                const double dg = fm(l0, a0.y, fm(l1, a1.y, fm(r0, b0.y, mu(r1, b1.y))));
+                fb[q] = fm(cL, bL.x, fm(cR, bR.x, df));
+                gb[q] = fm(cL, bL.y, fm(cR, bR.y, dg));
+            } else {
+                fb[q] = fm(cL, bL.x, mu(cR, bR.x));
+                gb[q] = fm(cL, bL.y, mu(cR, bR.y));
             }
-            fb[q] = vf;
-            gb[q] = vg;
         }
         const int ma = S.i3(xa, ya), mb = S.i3(xb, yb);
         x.mu = fm(wL, S.mu[ma], mu(wR, S.mu[mb]));
@@ -409,8 +414,14 @@ __device__ __forceinline__ void face(const InstDev &I, const TL &S, int xa, int 
             const double s = -(double)ca(q, 1 - A);
             const double2 *B = S.bp + q * A1;
             const double2 b = B[ic], b0 = B[ic + nm], b1 = B[ic + np], t0 = B[ic + tm], t1 = B[ic + tp];
-            fb[q] = fm(off, fm(fm_, b0.x, fm(f0, b.x, mu(fp, b1.x))), fm(s, fm(em, t0.x, fm(e0, b.x, mu(ep, t1.x))), b.x));
-            gb[q] = fm(off, fm(fm_, b0.y, fm(f0, b.y, mu(fp, b1.y))), fm(s, fm(em, t0.y, fm(e0, b.y, mu(ep, t1.y))), b.y));
+            const double nf = fm(fm_, b0.x, fm(f0, b.x, mu(fp, b1.x))), ng = fm(fm_, b0.y, fm(f0, b.y, mu(fp, b1.y)));
+            if (ca(q, 1 - A)) {
+                fb[q] = ad(b.x, fm(off, nf, mu(s, fm(em, t0.x, fm(e0, b.x, mu(ep, t1.x))))));
+                gb[q] = ad(b.y, fm(off, ng, mu(s, fm(em, t0.y, fm(e0, b.y, mu(ep, t1.y))))));
+            } else {
+                fb[q] = fm(off, nf, b.x);
+                gb[q] = fm(off, ng, b.y);
+            }
         }
 #pragma unroll
         for (int q = 0; q < Q; q++) {
@@ -437,18 +448,18 @@ __device__ __forceinline__ void face(const InstDev &I, const TL &S, int xa, int 
 template <typename FE, typename FW, typename FN, typename FS, typename FO, typename FB>
 __device__ __forceinline__ void update(double kx, double ky, FE e, FW w, FN n, FS s, FO old, FB bp, double (&nw)[Q])
 {
+    double J[Q];   // -dt / |V| times the flux sum
+    J[0] = 0.0;
 #pragma unroll
-    for (int q = 0; q < Q; q++) nw[q] = fm(4.0 / 3.0, bp(q), mu(-1.0 / 3.0, old(q)));
-#pragma unroll
-    for (int m = 0; m < 6; m++) {
-        const int qx = xset(m);
-        nw[qx] = fm(cx(qx) > 0 ? -kx : kx, sb(e(m), w(m)), nw[qx]);
-    }
+    for (int m = 0; m < 6; m++) J[xset(m)] = mu(cx(xset(m)) > 0 ? -kx : kx, sb(e(m), w(m)));
 #pragma unroll
     for (int m = 0; m < 6; m++) {
-        const int qy = yset(m);
-        nw[qy] = fm(cy(qy) > 0 ? -ky : ky, sb(n(m), s(m)), nw[qy]);
+        const int q = yset(m);
+        const double k = cy(q) > 0 ? -ky : ky, d = sb(n(m), s(m));
+        J[q] = cx(q) ? fm(k, d, J[q]) : mu(k, d);
     }
+#pragma unroll
+    for (int q = 0; q < Q; q++) nw[q] = fm(4.0 / 3.0, bp(q), fm(-1.0 / 3.0, old(q), J[q]));
 }
 
 // The update's KIND (1 f, 2 g, 3 both) at cell c: writes the new state; false if
