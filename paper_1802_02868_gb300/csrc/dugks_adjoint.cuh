@@ -77,6 +77,9 @@ struct APt {
 // (a cell: b = 1 - a); fsum is sum f ob, the adjoint of a.  B: the adjoint of the
 // point, with that of rho and of the weights in phi's; of a cell's u and p, and at a
 // face, whose p and u are formed from its bars, of sum f (in p) and sum xi f (in u).
+// A cell's u lacks the share b rho sum w xi ob of the equilibrium's term linear in u,
+// which the relaxation cancels in the adjoint of tilde (ka_cell): its effect on F and
+// rho is in B already.
 template <typename T, int A>
 __device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const T (&ob)[Q], const T (&yb)[Q], T fsum, bool wall,
                                        APt<T> &B, T &lam)
@@ -94,7 +97,7 @@ __device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const 
     const T uF = s.ux * Fx + s.uy * Fy, uE = s.ux * ECx + s.uy * ECy;
     const T rl = rho * s.lmu, src = C.cgl * rl + uF;
     const T rho3 = rho * T(1.0 / 3.0);
-    const T K1 = b * rho3 - c * uE;
+    const T KL = CELL ? b * rho3 : T(0), K1 = (CELL ? T(0) : b * rho3) - c * uE;   // KL: the share left out
     const T fx = c * Fx, fy = c * Fy, ex = c * ECx, ey = c * ECy;
     const T Gx = Fx - s.gpx, Gy = Fy - s.gpy, Pg = C.gc * s.phi * irho, gx = Pg * Gx, gy = Pg * Gy;
     const T ug = s.ux * gx + s.uy * gy, D2 = C.gb * s.phi - ug;
@@ -117,11 +120,11 @@ __device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const 
             if (cx(q)) { fxb += T(cx(q)) * z; exb += T(cx(q)) * zs; gxb += T(cx(q)) * (y + ys); }
             if (cy(q)) { fyb += T(cy(q)) * z; eyb += T(cy(q)) * zs; gyb += T(cy(q)) * (y + ys); }
             sb += z * xi_dot<T>(q, ex, ey) + y * xi_dot<T>(q, gx, gy);
-            const T xub = sb * (T(9) * xu + T(3));
+            const T xub = CELL ? T(9) * xu * (sb + z * KL) + T(3) * sb : sb * (T(9) * xu + T(3));
             if (cx(q)) uxb += T(cx(q)) * xub;
             if (cy(q)) uyb += T(cy(q)) * xub;
         }
-        s0b += sb;
+        s0b += CELL ? sb + z * KL : sb;
     }
     uxb -= T(3) * s.ux * s0b;
     uyb -= T(3) * s.uy * s0b;
@@ -162,6 +165,12 @@ __device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const 
     Fyb += c * fyb + tb * s.uy + EyB;
     uxb += tb * Fx + uEb * ECx;
     uyb += tb * Fy + uEb * ECy;
+    if (CELL) {   // the share of u's adjoint that is left out, b rho sum xi z, through u = (3 m + dt/2 F) / rho
+        const T lx = b * fxb, ly = b * fyb, hdt = T(0.5) * Pr.dt;
+        Fxb += hdt * lx;
+        Fyb += hdt * ly;
+        rhob -= s.ux * lx + s.uy * ly;
+    }
     T gfxb = C.cd * ExB, gfyb = C.cd * EyB;
     // weights: a, b, c over 6K + k X; b-bar and a-bar nearly cancel (f is near
     // equilibrium), so their difference is formed first
@@ -198,6 +207,28 @@ __device__ __forceinline__ T point_adj(const InstDev &I, const APt<T> &s, const 
     B.uy = uyb;
     B.p = pb;
     return CELL ? T(36) * b : a;
+}
+
+// v minus its part in the sums of f and of xi f: v_q - sum w v - 3 xi_q . sum w xi v,
+// from differences of v alone, so that a v which is such a part gives zero.
+template <typename T>
+__device__ __forceinline__ void nonconserved(const T (&v)[Q], T (&r)[Q])
+{
+    const T d1 = v[1] - v[3], d2 = v[2] - v[4], d5 = v[5] - v[7], d6 = v[6] - v[8];
+    const T e1 = (v[1] - v[0]) + (v[3] - v[0]), e2 = (v[2] - v[0]) + (v[4] - v[0]);
+    const T e5 = (v[5] - v[0]) + (v[7] - v[0]), e6 = (v[6] - v[0]) + (v[8] - v[0]);
+    const T m = (T(4) * (e1 + e2) + (e5 + e6)) * T(1.0 / 36.0);   // sum w v - v_0
+    const T o1 = (T(2) * d1 - (d5 - d6)) * T(1.0 / 12.0), o2 = (T(2) * d2 - (d5 + d6)) * T(1.0 / 12.0);
+    const T o5 = (d5 - (d1 + d2)) * T(1.0 / 3.0), o6 = (d6 - (d2 - d1)) * T(1.0 / 3.0);
+    r[0] = -m;
+    r[1] = (T(0.5) * e1 - m) + o1;
+    r[3] = (T(0.5) * e1 - m) - o1;
+    r[2] = (T(0.5) * e2 - m) + o2;
+    r[4] = (T(0.5) * e2 - m) - o2;
+    r[5] = (T(0.5) * e5 - m) + o5;
+    r[7] = (T(0.5) * e5 - m) - o5;
+    r[6] = (T(0.5) * e6 - m) + o6;
+    r[8] = (T(0.5) * e6 - m) - o6;
 }
 
 template <typename T>
@@ -517,11 +548,19 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 && !SPLIT ? 4 : 2) ka_cell
         const T b = point_adj<T, -1>(I, s, pf, pg, fsum, false, B, lam);
         // a p - x / 3 with p = 4/3 x + G and a = 1 - b: as an increment of x, so that
         // a uniform adjoint passes the step unchanged (4/3, 1/3 and a rounded one by
-        // one would leave a bias that grows with the steps)
+        // one would leave a bias that grows with the steps).  Of f, the
+        // relaxation -b p and what the equilibrium's p and u give back of it, b times
+        // p's part in the sums of f and of xi f, are formed as one here (the latter is
+        // not added in ka_tail): they cancel on an adjoint that is such a part, and
+        // rounded one by one they left an eigenvalue of 1 + 1e-8, an error of 2.5e-5 in
+        // dL/dkappa after 2000 FP32 steps of Rayleigh-Taylor 256x512 (5e-7 as one; 133
+        // us per step of a gradient either way, FP64 256x512 1.25 and 1.27 ms).
         const T bg = cellc<T>(I).gb36;
+        T r[Q];
+        nonconserved(pf, r);
 #pragma unroll
         for (int q = 0; q < Q; q++) {
-            Ad.af[q * N + c] = xf[q] + (Gf[q] - b * pf[q]);
+            Ad.af[q * N + c] = xf[q] + (Gf[q] - b * r[q]);
             Ad.ag[q * N + c] = xg[q] + (Gg[q] - bg * pg[q]);
         }
         T *const out[8] = {Ad.mu, Ad.lapmu, Ad.gmx, Ad.gmy, Ad.gfx, Ad.gfy, Ad.gpx, Ad.gpy};
@@ -758,7 +797,9 @@ __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts,
         const long long c = cell_of(I, i, j);
         const TCoef<T> &kx = tc[x + 2], &ky = tc[W2 + y + 2];
         const T *sx = sgx + (y + 2) * WX + x + 3, *sy = sgy + (y + 3) * W2 + x + 2;
-        const T pb = Ad.p[c] + (kx.c1 * sx[0] + kx.m1 * sx[-1] + kx.p1 * sx[1]) + (ky.c1 * sy[0] + ky.m1 * sy[-W2] + ky.p1 * sy[W2]);
+        // of sum f: the share that comes from bar-plus is in ka_cell's af already
+        const T pg = (kx.c1 * sx[0] + kx.m1 * sx[-1] + kx.p1 * sx[1]) + (ky.c1 * sy[0] + ky.m1 * sy[-W2] + ky.p1 * sy[W2]);
+        const T pb = Ad.p[c] + pg;
         T uxb = Ad.ux[c], uyb = Ad.uy[c];
         const T phi = T(phi_val(P.phi[c]));
         const T rho = Pr.rhoB + Pr.drho * (phi - Pr.phiB);
@@ -790,7 +831,7 @@ __global__ void __launch_bounds__(NT) ka_tail(const InstDev *__restrict__ insts,
             lamb -= pk * Pr.gamma * rho * lm;
             phb[y * BX + x] = Ad.phi[c] + (sb.phi + Pr.drho * sb.rho);
 #pragma unroll
-            for (int q = 0; q < Q; q++) Ad.af[q * N + c] += pb + T(cx(q)) * mxb + T(cy(q)) * myb;
+            for (int q = 0; q < Q; q++) Ad.af[q * N + c] += pg + T(cx(q)) * mxb + T(cy(q)) * myb;
         }
     }
     __syncthreads();
