@@ -113,9 +113,10 @@ int dugks_init(dugks_sim *sim, const double *phi, const double *ux, const double
    original-function, microfluxf, updatef).  Asynchronous on the sim's stream;
    a non-finite state is reported by the next synchronising call.  A call of 16
    steps or more may run as one cooperative launch per 512 steps, whose tiles wait
-   for each other; a wait that runs out (seconds) is reported by the next
-   synchronising call as DUGKS_ERR_TIMEOUT, and the state is then undefined until
-   the next dugks_init or dugks_load. */
+   for each other; a wait that runs out (seconds; DUGKS_WAIT_POLLS in the environment
+   of dugks_create sets it in polls) is reported by every synchronising call from then
+   on as DUGKS_ERR_TIMEOUT, and the state is undefined until the next dugks_init,
+   dugks_load or dugks_adjoint. */
 int dugks_step(dugks_sim *sim, long nsteps);
 
 /* Macroscopic fields at the cell centres from the current state (Eqs. phi,

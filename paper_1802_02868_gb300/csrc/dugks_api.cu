@@ -90,6 +90,7 @@ struct dugks_sim {
     } flow[kNumKernelShapes];
     bool any_flow = false;
     bool flow_off = false;        // the cooperative launch was refused
+    unsigned wait_polls = 1u << 22;   // polls before a wait of a many-step launch gives up: a few seconds
     // adjoint: runs of cells and of faces, and each instance's ranges of them;
     // built by the first dugks_adjoint
     AdjSeg *d_cseg = nullptr, *d_fseg = nullptr;
@@ -721,7 +722,7 @@ int launch_flow(dugks_sim *s, int k, int n)
     fl.done = s->flow[k].done;
     fl.nbr = s->flow[k].nbr;
     fl.err = s->d_status + s->n_inst;
-    fl.limit = 1u << 22;   // a few seconds of polls
+    fl.limit = s->wait_polls;
     const int grid = std::min(fl.n_tiles, resident[uni] * s->n_sm);
     const int4 *tiles = s->d_tiles_s[k];
     const InstDev *insts = s->d_inst;
@@ -1054,6 +1055,17 @@ int sync_status(dugks_sim *s)
     if (e != cudaSuccess) return cuda_status(e);
     if (st[1]) return DUGKS_ERR_TIMEOUT;
     return st[0] & ST_NONFINITE ? DUGKS_ERR_NONFINITE : DUGKS_OK;
+}
+
+// After a synchronisation, for the calls that do not report a non-finite state: a
+// wait of a many-step launch that ran out.
+int wait_error(dugks_sim *s)
+{
+    if (!s->any_flow) return DUGKS_OK;
+    int late = 0;
+    cudaError_t e = cudaMemcpyAsync(&late, s->d_status + s->n_inst, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    return e != cudaSuccess ? cuda_status(e) : late ? DUGKS_ERR_TIMEOUT : DUGKS_OK;
 }
 
 // Start the check of n dense values on the device for a non-finite one, which sets
@@ -1470,6 +1482,8 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         s->use_graph = !(g && g[0] == '1');
         const char *u = std::getenv("DUGKS_GENERAL_ONLY");
         s->use_uni = !(u && u[0] == '1');
+        const char *w = std::getenv("DUGKS_WAIT_POLLS");
+        if (w && w[0]) s->wait_polls = (unsigned)std::strtoul(w, nullptr, 10);
     }
     s->stream = (cudaStream_t)cuda_stream;
     s->alloc_fn = g_alloc_fn;
@@ -1823,7 +1837,7 @@ int dugks_batch_status(dugks_sim *s, int *per_instance_status)
     e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     for (int k = 0; k < s->n_inst; k++) per_instance_status[k] = (st[k] & ST_NONFINITE) ? DUGKS_ERR_NONFINITE : DUGKS_OK;
-    return DUGKS_OK;
+    return wait_error(s);
 }
 
 namespace {
@@ -1835,7 +1849,8 @@ int rewrite_paused(dugks_sim *s, const std::vector<char> &paused)
     if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     for (int k = 0; k < s->n_inst; k++) st[k] = (st[k] & ~ST_PAUSED) | (paused[k] ? ST_PAUSED : 0);
-    return cuda_status(upload(s, s->d_status, st.data(), sizeof(int) * s->n_inst));
+    e = upload(s, s->d_status, st.data(), sizeof(int) * s->n_inst);
+    return e != cudaSuccess ? cuda_status(e) : wait_error(s);
 }
 
 // the tile of shape 0 for the instances that are not paused
@@ -1869,7 +1884,7 @@ int read_paused(dugks_sim *s, std::vector<char> &paused)
     if (e != cudaSuccess) return cuda_status(e);
     paused.resize(s->n_inst);
     for (int k = 0; k < s->n_inst; k++) paused[k] = (st[k] & ST_PAUSED) ? 1 : 0;
-    return DUGKS_OK;
+    return wait_error(s);
 }
 }  // namespace
 
@@ -1941,7 +1956,7 @@ int dugks_save(dugks_sim *s, void *buf, size_t *bytes)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     *bytes = need;
-    return DUGKS_OK;
+    return wait_error(s);
 }
 
 int dugks_load(dugks_sim *s, const void *buf, size_t bytes)
@@ -1984,7 +1999,7 @@ int dugks_kernel_times(dugks_sim *s, double *ms, long *launches)
         s->k_ms[k] = 0.0;
         s->k_n[k] = 0;
     }
-    return DUGKS_OK;
+    return wait_error(s);
 }
 
 const char *dugks_kernel_name(int k)
@@ -2028,6 +2043,8 @@ int dugks_set_tile_shape(dugks_sim *s, int shape)
             s->graph2 = nullptr;
         }
         s->shape = shape;
+        const int rc = wait_error(s);
+        if (rc) return rc;
     }
     return s->prec == DUGKS_FP64 ? prepare_fused<double>(s) : prepare_fused<float>(s);
 }
@@ -2105,6 +2122,7 @@ int dugks_autotune(dugks_sim *s, int steps, int *chosen, double *ms_per_step)
     s->launches = launches;
     if (rc == DUGKS_OK && e != cudaSuccess) rc = cuda_status(e);
     if (rc == DUGKS_OK) rc = dugks_set_tile_shape(s, best);
+    if (rc == DUGKS_OK) rc = wait_error(s);
     if (rc == DUGKS_OK) {
         if (chosen) *chosen = best;
         if (ms_per_step) *ms_per_step = best_ms / steps;

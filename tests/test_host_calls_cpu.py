@@ -4,11 +4,12 @@ memory on the host, runs no kernel and records what is ordered on which stream
 calls report.  No GPU is needed."""
 import ctypes
 import glob
+import importlib.util
 import os
 import shutil
 import subprocess
+import types
 
-import numpy as np
 import pytest
 
 from paper_1802_02868_gb300 import build, dugks
@@ -53,18 +54,23 @@ def recording_library(tmp_path_factory):
 
 
 @pytest.fixture
-def rec(recording_library, monkeypatch):
-    monkeypatch.setattr(build, "LIB", recording_library)
-    monkeypatch.setattr(dugks, "_lib", None)
-    r = Recorder(dugks.load())
+def rec(recording_library):
+    # a second copy of the binding, so that simulations of the real library, which may
+    # be collected at any time, never meet this one
+    spec = importlib.util.spec_from_file_location("paper_1802_02868_gb300.dugks_recording", dugks.__file__)
+    binding = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(binding)
+    binding._build = types.SimpleNamespace(LIB=recording_library)
+    r = Recorder(binding.load())
+    r.dugks = binding
     yield r
     r.lib.rec_set_capturing(0)
     r.lib.rec_set_late(0)
 
 
-def _drops(sizes, prec, stream=STREAM):
+def _drops(rec, sizes, prec, stream=STREAM):
     cs = [I.stationary_drop(n=n, radius=0.25 * n) for n in sizes]
-    s = dugks.Sim([c.mesh for c in cs], [c.params for c in cs], prec, stream=stream)
+    s = rec.dugks.Sim([c.mesh for c in cs], [c.params for c in cs], prec, stream=stream)
     return s, [c.phi0 for c in cs]
 
 
@@ -75,7 +81,7 @@ def test_tables_and_status_are_written_on_the_sims_stream(rec, sizes, prec):
     every write goes to the sim's stream, and the host waits on that stream for a
     copy out of its own memory before the call returns."""
     made = []
-    log = [rec.calls(lambda: made.append(_drops(sizes, prec)))]
+    log = [rec.calls(lambda: made.append(_drops(rec, sizes, prec)))]
     s, phi = made[0]
     with s:
         log.append(rec.calls(lambda: s.init(phi)))
@@ -98,7 +104,7 @@ def test_tables_and_status_are_written_on_the_sims_stream(rec, sizes, prec):
 
 
 def test_a_table_made_while_the_caller_captures_stays_out_of_the_capture(rec):
-    s, phi = _drops((64,), dugks.FP32)
+    s, phi = _drops(rec, (64,), dugks.FP32)
     with s:
         s.init(phi)
         rec.lib.rec_set_capturing(1)
@@ -107,3 +113,35 @@ def test_a_table_made_while_the_caller_captures_stays_out_of_the_capture(rec):
         assert len(up) == 1 and up[0][3] not in (0, STREAM)
         assert ("sync", 0, 0, up[0][3]) in calls
         assert not any(c[0] == "sync" and c[3] == STREAM for c in calls)
+
+
+@pytest.mark.parametrize("sizes", [(64,), (24, 41, 64)])
+def test_every_synchronising_call_reports_a_wait_that_ran_out(rec, sizes):
+    made = []
+    n = len(sizes)
+    calls = rec.calls(lambda: made.append(_drops(rec, sizes, dugks.FP32)))
+    s, phi = made[0]
+    with s:
+        # the per-instance status, the error word, the refused word
+        (at,) = {c[1] for c in calls if c[0] == "memset" and c[2] == 4 * (n + 2)}
+        s.init(phi)
+        start = s.state()
+        rec.lib.rec_set_late(at + 4 * n)
+        s.step(64)
+        assert rec.lib.rec_coop_launches() > 0
+        rec.lib.rec_set_late(0)
+        for name, fn in (("save", s.state), ("status", s.status), ("set_paused", lambda: s.set_paused([False] * n)),
+                         ("step_each", lambda: s.step_each([1] * n)), ("moments", s.moments), ("conservation", s.conservation),
+                         ("diagnostics", s.diagnostics_array), ("laplace_pressure", s.laplace_pressure),
+                         ("kernel_times", s.kernel_times), ("set_tile_shape", lambda: s.set_tile_shape(1)), ("autotune", s.autotune)):
+            with pytest.raises(rec.dugks.DugksError) as e:
+                fn()
+            assert e.value.rc == -5, name
+        s.init(phi)                                     # a new state: nothing to report
+        s.step(64)
+        assert s.status() == [0] * n
+        rec.lib.rec_set_late(at + 4 * n)
+        s.step(64)
+        rec.lib.rec_set_late(0)
+        s.set_state(*start)
+        s.state()
