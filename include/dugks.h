@@ -120,7 +120,10 @@ int dugks_init(dugks_sim *sim, const double *phi, const double *ux, const double
 int dugks_step(dugks_sim *sim, long nsteps);
 
 /* Macroscopic fields at the cell centres from the current state (Eqs. phi,
-   oderrho, u, P).  Host outputs of all cells, each may be NULL.  Synchronises. */
+   oderrho, u, P).  Host outputs of all cells, each may be NULL.  Synchronises.
+   An instance that became non-finite reports phi of its present state beside rho, u
+   and p as the last dugks_moments found them while it was finite (before any: rho
+   zero, u and p of dugks_init). */
 int dugks_moments(dugks_sim *sim, double *phi, double *rho, double *ux, double *uy, double *p);
 
 /* FP64 volume-weighted sums of phi and rho per instance (Eq. locallyconserved);

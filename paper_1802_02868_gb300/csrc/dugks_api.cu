@@ -968,14 +968,14 @@ void assign_planes(dugks_sim *s, Planes<T> &P, T *base)
         P.fbp = p; p += Q * N;
         P.gbp = p; p += Q * N;
     }
-    T **one[] = {&P.mu, &P.lapmu, &P.gmux, &P.gmuy, &P.gphix, &P.gphiy, &P.p, &P.ux, &P.uy, &P.gpx, &P.gpy};
+    T **one[] = {&P.mu, &P.lapmu, &P.gmux, &P.gmuy, &P.gphix, &P.gphiy, &P.p, &P.ux, &P.uy, &P.gpx, &P.gpy, &P.rho};
     for (T **q : one) { *q = p; p += N; }
     P.phi = (phi_t<T> *)s->d_phi;
     P.N = N;
     P.status = s->d_status;
 }
 
-constexpr int kNumScalarPlanes = 11;
+constexpr int kNumScalarPlanes = 12;
 
 void free_sim(dugks_sim *s)
 {

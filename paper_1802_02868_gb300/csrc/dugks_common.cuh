@@ -215,7 +215,7 @@ struct Planes {
     // phi is FP64 in both precisions: in FP32 mode it is the authoritative
     // order parameter, advanced by the conservative flux form of the update
     phi_t<T> *phi;
-    T *mu, *lapmu, *gmux, *gmuy, *gphix, *gphiy, *p, *ux, *uy, *gpx, *gpy;
+    T *mu, *lapmu, *gmux, *gmuy, *gphix, *gphiy, *p, *ux, *uy, *gpx, *gpy, *rho;
     long long N;
     int *status;   // per instance, bit 0 = non-finite seen
 };

@@ -232,8 +232,9 @@ __device__ __forceinline__ void grad_phi(const InstDev &I, const phi_t<T> *__res
 // ---------------------------------------------------------------------------
 // k_macro: grad mu, lap mu, grad phi, total force F = -phi grad mu + F_b, and
 // Eqs. (u), (P) from the tracked f, into the planes; or (MOMENTS) phi, rho, ux, uy, p
-// as dense FP64 fields at out[0..4] (NULL to skip one), without the planes between: a
-// moments call was two kernels and one gather per field.
+// as dense FP64 fields at out[0..4] (NULL to skip one) beside the planes: a moments
+// call was two kernels and one gather per field.  The planes of rho, u and p are what
+// a masked instance reports: its last values while it was finite.
 // ---------------------------------------------------------------------------
 struct DenseOut {
     double *out[5];
@@ -280,7 +281,17 @@ __global__ void __launch_bounds__(TX *TY) k_macro(const InstDev *__restrict__ in
     T p = sf + hdt * cs2 * (ux * grx + uy * gry - Pr.gamma * rho * Pr.lambda * lmu);
     if constexpr (MOMENTS) {
         const long long d = D.dense0[t.x] + (long long)j * I.nx + i;
-        if (masked) { ux = P.ux[c]; uy = P.uy[c]; p = P.p[c]; }   // what a kernel last left there
+        if (masked) {
+            rho = P.rho[c];
+            ux = P.ux[c];
+            uy = P.uy[c];
+            p = P.p[c];
+        } else {
+            P.rho[c] = rho;
+            P.ux[c] = ux;
+            P.uy[c] = uy;
+            P.p[c] = p;
+        }
         if (D.out[0]) D.out[0][d] = phi_to_double(P.phi[c]);
         if (D.out[1]) D.out[1][d] = (double)rho;
         if (D.out[2]) D.out[2][d] = (double)ux;
