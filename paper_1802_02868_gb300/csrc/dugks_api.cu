@@ -1087,11 +1087,19 @@ cudaError_t check_input(dugks_sim *s, const double *v, long long n)
 // 9.4 ms on GB300, 3.6 ms with the pages touched first on an idle device, 0.6 ms when
 // they are there.  Contents are kept (the atomic or of 0 is a write for the page
 // tables).  Above 4 MB, where numpy asks for huge pages, the copy's own faults are the
-// cheaper ones (33 MB: 2.5 ms, touched first 12.7 ms).
+// cheaper ones (33 MB: 2.5 ms, touched first 12.7 ms).  Only ordinary host memory:
+// page-locked arrays have their pages, and memory that the host cannot write (a device
+// pointer) is for the copy to judge.
 void touch_pages(void *p, size_t bytes)
 {
     static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
     if (!p || bytes < 16 * page || bytes > (size_t(4) << 20)) return;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (a.type != cudaMemoryTypeUnregistered) return;
     unsigned char *c = (unsigned char *)p;
     for (size_t k = 0; k < bytes; k += page) __atomic_fetch_or(c + k, 0, __ATOMIC_RELAXED);
     __atomic_fetch_or(c + bytes - 1, 0, __ATOMIC_RELAXED);
@@ -1736,8 +1744,7 @@ int dugks_moments(dugks_sim *s, double *phi, double *rho, double *ux, double *uy
     }
     int rc = s->prec == DUGKS_FP64 ? do_moments<double>(s, dst) : do_moments<float>(s, dst);
     if (rc) return rc;
-    for (int k = 0; k < 5; k++)
-        if (!alias[k]) touch_pages(out[k], sizeof(double) * D);
+    for (double *o : out) touch_pages(o, sizeof(double) * D);
     for (int k = 0; k < 5; k++) {
         if (!out[k] || alias[k]) continue;
         cudaError_t e = cudaMemcpyAsync(out[k], dst[k], sizeof(double) * D, cudaMemcpyDeviceToHost, s->stream);
@@ -1775,7 +1782,7 @@ int dugks_laplace_pressure(dugks_sim *s, double *P)
     if (!s || !P) return DUGKS_ERR_ARG;
     int rc = s->prec == DUGKS_FP64 ? do_diag<double>(s, s->d_stage) : do_diag<float>(s, s->d_stage);
     if (rc) return rc;
-    if (!host_alias(P)) touch_pages(P, sizeof(double) * s->n_dense);
+    touch_pages(P, sizeof(double) * s->n_dense);
     cudaError_t e = cudaMemcpyAsync(P, s->d_stage, sizeof(double) * s->n_dense, cudaMemcpyDeviceToHost, s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     return sync_status(s);
@@ -1951,7 +1958,7 @@ int dugks_save(dugks_sim *s, void *buf, size_t *bytes)
     if (*bytes < need) return DUGKS_ERR_ARG;
     int rc = s->prec == DUGKS_FP64 ? do_pack_state<double>(s, s->d_stage) : do_pack_state<float>(s, s->d_stage);
     if (rc) return rc;
-    if (!host_alias((double *)buf)) touch_pages(buf, need);
+    touch_pages(buf, need);
     cudaError_t e = cudaMemcpyAsync(buf, s->d_stage, need, cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);

@@ -10,6 +10,7 @@ import shutil
 import subprocess
 import types
 
+import numpy as np
 import pytest
 
 from paper_1802_02868_gb300 import build, dugks
@@ -145,3 +146,28 @@ def test_every_synchronising_call_reports_a_wait_that_ran_out(rec, sizes):
         rec.lib.rec_set_late(0)
         s.set_state(*start)
         s.state()
+
+
+def test_outputs_that_the_host_cannot_write_are_left_to_the_copy(rec):
+    """Device memory as an output of a size whose pages are touched ahead of the copy:
+    the runtime refuses the copy, and the process lives to see it."""
+    s, phi = _drops(rec, (128,), dugks.FP64)              # 128 KB a field
+    n = 8 * s.ncells
+    with s:
+        s.init(phi)
+
+        def refused(name, *args):
+            return getattr(rec.lib, name)(s.h, *args) == -2   # the runtime's error
+        tgt = np.zeros(s.ncells)
+        at = [ctypes.c_void_p(rec.lib.rec_unreachable(n)) for _ in range(5)]
+        big = ctypes.c_void_p(rec.lib.rec_unreachable(18 * n))
+        checks = [lambda: refused("dugks_moments", *[ctypes.cast(a, ctypes.POINTER(ctypes.c_double)) for a in at]),
+                  lambda: refused("dugks_laplace_pressure", ctypes.cast(at[0], ctypes.POINTER(ctypes.c_double))),
+                  lambda: refused("dugks_save", big, ctypes.byref(ctypes.c_size_t(18 * n))),
+                  lambda: refused("dugks_adjoint", 2, 1, tgt.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), None,
+                                  ctypes.cast(at[0], ctypes.POINTER(ctypes.c_double)), None, None)]
+        for k, ok in enumerate(checks):
+            pid = os.fork()                                # a child: the fault would be a signal
+            if pid == 0:
+                os._exit(0 if ok() else 1)
+            assert os.waitpid(pid, 0)[1] == 0, k
