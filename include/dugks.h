@@ -112,8 +112,9 @@ int dugks_init(dugks_sim *sim, const double *phi, const double *ux, const double
 /* Steps 2-7 repeated nsteps times (Sec. 2.2; Eqs. relations1/2, fbar_h,
    original-function, microfluxf, updatef).  Asynchronous on the sim's stream;
    a non-finite state is reported by the next synchronising call.  A call of 16
-   steps or more may run as one cooperative launch per 512 steps, whose tiles wait
-   for each other; a wait that runs out (seconds; DUGKS_WAIT_POLLS in the environment
+   steps or more may run as cooperative launches of many steps each (at most 512, and
+   about 20 ms or four steps, during which work of other streams may have to wait for
+   the device), whose tiles wait for each other; a wait that runs out (seconds; DUGKS_WAIT_POLLS in the environment
    of dugks_create sets it in polls) is reported by every synchronising call from then
    on as DUGKS_ERR_TIMEOUT, and the state is undefined until the next dugks_init,
    dugks_load or dugks_adjoint. */

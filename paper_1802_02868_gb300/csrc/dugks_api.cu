@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -411,23 +412,32 @@ int shape_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm
 // 670, 851, FP32 32.8, 41, 62; 4x256 channel FP64 85, 57, 36, 25 (4x8: its four
 // columns fill a tile, where 32 columns hold each cell eight times), FP32 9.1,
 // 6.4, 5.1; four 100x100 drops FP64 111, 99, 111, 136, FP32 11.3, 10.1, 10.9.
+struct TileCost {
+    int k;             // index into kShapes
+    double lat, sat;
+};
+const TileCost kCost64[] = {{0, 80, 82.5}, {7, 51, 41}, {8, 33.7, 25}, {9, 20.6, 15.8}, {10, 20.6, 15.8}};
+const TileCost kCost32[] = {{0, 9.1, 4.2}, {7, 7.0, 2.6}, {8, 5.4, 2.4}};
+
+// estimated us of a step of that many tiles
+double tile_step_us(const TileCost &c, long long tiles, int precision, int n_sm)
+{
+    double per = (double)tiles / n_sm;
+    if (precision == DUGKS_FP64 && per <= 2) per = std::ceil(per);
+    return c.lat + std::max(0.0, per - 1) * c.sat;
+}
+
 int tile_for_sizes(const int *nx, const int *ny, int n, int precision, int n_sm)
 {
-    struct Cost { int k; double lat, sat; };
-    static const Cost f64[] = {{0, 80, 82.5}, {7, 51, 41}, {8, 33.7, 25}, {9, 20.6, 15.8}, {10, 20.6, 15.8}};
-    static const Cost f32[] = {{0, 9.1, 4.2}, {7, 7.0, 2.6}, {8, 5.4, 2.4}};
     const bool d = precision == DUGKS_FP64;
-    const Cost *c = d ? f64 : f32;
     int best = 0;
     double best_t = 0;
-    for (int i = 0; i < (d ? 5 : 3); i++) {
-        const ShapeDesc &S = kShapes[c[i].k];
+    for (const TileCost *c = d ? kCost64 : kCost32, *end = d ? std::end(kCost64) : std::end(kCost32); c != end; c++) {
+        const ShapeDesc &S = kShapes[c->k];
         long long tiles = 0;
         for (int k = 0; k < n; k++) tiles += (long long)((nx[k] + S.bx - 1) / S.bx) * ((ny[k] + S.by - 1) / S.by);
-        double per = (double)tiles / n_sm;
-        if (d && per <= 2) per = std::ceil(per);
-        const double t = c[i].lat + std::max(0.0, per - 1) * c[i].sat;
-        if (i == 0 || t < best_t) { best = c[i].k; best_t = t; }
+        const double t = tile_step_us(*c, tiles, precision, n_sm);
+        if (c->k == 0 || t < best_t) { best = c->k; best_t = t; }
     }
     return best;
 }
@@ -637,6 +647,24 @@ int build_graph2(dugks_sim *s)
 // tiles per SM: 130 and 147).
 constexpr long FLOW_MIN = 16, FLOW_MAX = 512;
 constexpr int FLOW_TILES = 7;
+// A many-step launch holds its SMs until its last step, and a kernel of another stream
+// that needs a whole SM waits for it, where it used to start within 0.2 ms, between two
+// steps.  So it takes at most about FLOW_US of estimated time, or FLOW_LEAST steps: beside
+// 300 FP64 steps of 256x1024 such a kernel waited 152 ms for a launch without this bound,
+// 18 ms with it.  Each further launch of a call costs the end of one more wave, about 0.09
+// ms there, half a percent of 20 ms (576 us per step in one launch of 20 steps, 585 in
+// three; 577 with this bound in calls of 20 and 60).
+constexpr double FLOW_US = 20000;
+constexpr long FLOW_LEAST = 4;
+
+// steps per many-step launch of kernel shape k
+long flow_steps(const dugks_sim *s, int k)
+{
+    double us = 0;
+    for (const TileCost &c : kCost64) if (s->prec == DUGKS_FP64 && c.k == k) us = tile_step_us(c, s->n_tiles_s[k], s->prec, s->n_sm);
+    for (const TileCost &c : kCost32) if (s->prec == DUGKS_FP32 && c.k == k) us = tile_step_us(c, s->n_tiles_s[k], s->prec, s->n_sm);
+    return std::min(FLOW_MAX, std::max(FLOW_LEAST, (long)(FLOW_US / us)));
+}
 
 // The tiles that each tile's 4-cell ring reads, itself among them, by the tile
 // columns and rows that hold the ring's cells (a narrow last column or row lets
@@ -756,9 +784,11 @@ long step_flow(dugks_sim *s, long n)
         cudaGetLastError();
         return 0;
     }
+    // launches of about equal length, none of them shorter than it must be
+    const long most = flow_steps(s, k), launches = (n + most - 1) / most;
     long done = 0;
-    while (n - done >= FLOW_MIN) {
-        const int m = (int)std::min(n - done, FLOW_MAX);
+    for (long l = 0; l < launches; l++) {
+        const int m = (int)((n - done) / (launches - l));
         int rc;
         if constexpr (sizeof(T) == 8) {
             rc = k == 7 ? launch_flow<T, 16, 8, 128>(s, k, m) : k == 8 ? launch_flow<T, 8, 8, 128>(s, k, m)

@@ -171,3 +171,17 @@ def test_outputs_that_the_host_cannot_write_are_left_to_the_copy(rec):
             if pid == 0:
                 os._exit(0 if ok() else 1)
             assert os.waitpid(pid, 0)[1] == 0, k
+
+
+@pytest.mark.parametrize("nx,ny,prec,n,least,most", [(256, 1024, dugks.FP64, 512, 12, 20), (512, 1024, dugks.FP64, 512, 24, 40),
+                                                     (64, 64, dugks.FP32, 512, 1, 1), (64, 64, dugks.FP64, 512, 1, 1),
+                                                     (64, 64, dugks.FP32, 1050, 3, 3)])
+def test_a_many_step_launch_holds_the_device_for_milliseconds(rec, nx, ny, prec, n, least, most):
+    """512 steps of a small mesh, but about 20 ms of a large one: a step of
+    256x1024 in FP64 takes 0.6 ms, one of 512x1024 twice that, one of 64x64 0.02 ms."""
+    m = I.uniform_mesh(nx, ny)
+    with rec.dugks.Sim(m, I.stationary_drop().params, prec, stream=STREAM) as s:
+        s.init(I.drop_field(m, 0.3 * nx, (0.5 * nx, 0.5 * ny), 4.0))
+        calls = rec.calls(lambda: s.step(n))
+        assert least <= rec.lib.rec_coop_launches() <= most
+        assert not any(c[0].startswith(("kernel", "graph")) for c in calls)   # they take every step of the call
