@@ -233,7 +233,9 @@ int dugks_kernel_bytes_per_cell(const dugks_sim *sim, int k, double *bytes);
    reports shape 0.  dugks_autotune times every shape on the sim's current state for
    `steps` steps each (CUDA events on the sim's stream), restores the state and
    the per-instance status after each trial, keeps the fastest shape and
-   returns its index and time per step.  It allocates a temporary snapshot of
+   returns its index and time per step.  A trial is one call of `steps` steps, after
+   an untimed call that sets up what it needs: below 16 steps it times single-step
+   launches, which is what calls of that length get (see dugks_step).  It allocates a temporary snapshot of
    the state (cudaMalloc) for the duration of the call and synchronises. */
 #define DUGKS_NUM_TILE_SHAPES 7
 int dugks_autotune(dugks_sim *sim, int steps, int *chosen, double *ms_per_step);

@@ -2130,10 +2130,11 @@ int dugks_autotune(dugks_sim *s, int steps, int *chosen, double *ms_per_step)
     for (int k = 0; k < DUGKS_NUM_TILE_SHAPES && e == cudaSuccess && rc == DUGKS_OK; k++) {
         rc = dugks_set_tile_shape(s, k);
         if (rc) break;
-        // warm-up: the first launch of the instantiation, and the capture of
-        // the two-step graph that multi-step calls replay (set_tile_shape
-        // drops it), so that neither falls in the timed steps
-        rc = dugks_step(s, 2);
+        // warm-up: the first launch of the instantiation, and what a call of that
+        // many steps sets up (the two-step graph, which set_tile_shape drops, or the
+        // tables and the kernel of the many-step launch), so that neither falls in
+        // the timed steps
+        rc = dugks_step(s, std::max<long>(2, std::min<long>(steps, FLOW_MIN)));
         if (rc) break;
         e = cudaEventRecord(a, s->stream);
         if (e != cudaSuccess) break;

@@ -185,3 +185,20 @@ def test_a_many_step_launch_holds_the_device_for_milliseconds(rec, nx, ny, prec,
         calls = rec.calls(lambda: s.step(n))
         assert least <= rec.lib.rec_coop_launches() <= most
         assert not any(c[0].startswith(("kernel", "graph")) for c in calls)   # they take every step of the call
+
+
+@pytest.mark.parametrize("steps", [5, 20])
+def test_autotune_sets_up_before_it_times(rec, steps):
+    """Between the two events of a trial there are only launches, of kernels that ran
+    before: no allocation, upload, capture or wait for one."""
+    s, phi = _drops(rec, (64,), dugks.FP32)
+    with s:
+        s.init(phi)
+        calls = rec.calls(lambda: s.autotune(steps))
+        marks = [k for k, c in enumerate(calls) if c[0] == "event"]
+        assert len(marks) == 2 * dugks.NUM_TILE_SHAPES
+        for a, b in zip(marks[::2], marks[1::2]):
+            timed = [c[0] for c in calls[a + 1:b]]
+            assert timed and all(op.startswith(("kernel", "cooperative", "graph")) for op in timed), timed
+            assert {op for op in timed if op != "graph"} <= {c[0] for c in calls[:a]}
+        assert any(c[0].startswith("cooperative") for c in calls) == (steps >= 16)
