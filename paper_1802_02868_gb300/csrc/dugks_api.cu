@@ -634,17 +634,21 @@ int build_graph2(dugks_sim *s)
     return cuda_status(e);
 }
 
-// Steps of one call from which a many-step launch takes them, and the most per
-// launch.  A call of fewer steps keeps its launch per step (or per two): the
-// cooperative launch costs about two of a small mesh's steps.  us per step in
-// calls of 60, launches and many-step: FP32 64x64 drop 6.2 and 4.5, four 4x256
-// channels 7.2 and 5.8, Rayleigh-Taylor 256x512 24.7 and 19.4 and 256x1024 39.0
-// and 38.3; FP64 64x64 drop 22.5 and 20.6, 4x256 channel 26.7 and 24.7, four
-// 100x100 drops 132 and 98.6, Rayleigh-Taylor 256x1024 594 and 576.  FP32
-// meshes of more tiles than FLOW_TILES per SM keep the launches: their last wave
-// is a small part of a step, and a tile that comes by the hardware's scheduler
-// needs no wait (512x512 drop, 6.7 tiles per SM: 32.8 and 32.8; 1024x1024, 27
-// tiles per SM: 130 and 147).
+// Steps of one call from which many-step launches take them, and the most per
+// launch.  us per step in calls of 60, launches and many-step: FP32 64x64 drop 6.2
+// and 4.5, four 4x256 channels 7.2 and 5.8, Rayleigh-Taylor 256x512 24.6 and 19.3 and
+// 256x1024 39.0 and 38.3; FP64 64x64 drop 22.3 and 20.5, 4x256 channel 26.7 and 24.3,
+// four 100x100 drops 132 and 99, Rayleigh-Taylor 256x1024 591 and 577.  Calls of
+// fewer steps keep their launch per step (or per two), though the line could lie
+// lower: in calls of 4 and 8 steps the many-step launch measured 5.2 and 4.8 (FP32
+// 64x64 drop), 6.7 and 6.4 (channels), 20.7 and 19.8 (256x512), 21.4 and 21.2 (FP64
+// drop), 105 and 103 (four drops), 577 and 577 (FP64 256x1024); of 2 steps no less
+// than launches, but for the FP64 drops.
+// FP32 meshes of more tiles than FLOW_TILES per SM keep the launches: their last wave
+// is a small part of a step, and a tile that comes by the hardware's scheduler needs
+// no wait.  Launches and many-step by tiles per SM: 6.7 (512x512 drop) 33.1 and 33.0;
+// 8.4 41.0 and 42.4; 10.1 48.1 and 50.2; 13.5 63.2 and 67.4; 20 102 and 108; 27
+// (1024x1024) 131 and 149.
 constexpr long FLOW_MIN = 16, FLOW_MAX = 512;
 constexpr int FLOW_TILES = 7;
 // A many-step launch holds its SMs until its last step, and a kernel of another stream

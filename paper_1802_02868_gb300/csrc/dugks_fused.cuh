@@ -394,18 +394,21 @@ __device__ __forceinline__ const StepIO<T> &step_io_of(const Flow<T> &fl, int st
 
 // NT threads (a multiple of 32, at least BX * BY) share the phases of a
 // BX x BY tile; the first BX * BY of them own one cell each in the update.
-// One step: a thread block per tile.  FLOW: many steps in one cooperative launch,
-// without a barrier of the device between them: block b takes the items b, b + gridDim.x, ... of the sequence (step 0:
-// all tiles, step 1: all tiles, ...), and waits for an item only until the tiles
-// that its ring reads have finished the step before.  All blocks are resident
-// (cooperative launch) and an item waits only for earlier items, so every wait
-// ends.  The two state buffers alternate: a tile overwrites a buffer only after
-// its neighbours, which are the tiles that read it (the ring relation is
-// symmetric), have finished the step that read it.
+//
+// One step (MODE_STEP): a thread block per tile.
+//
+// Many steps (MODE_FLOW): one cooperative launch without a barrier of the device.
+// - Items are (step, tile) pairs, step by step; block b takes items b, b + gridDim.x,
+//   and so on.
+// - An item waits until the tiles that its ring reads have finished the step before.
+//   It waits only for earlier items, and all blocks are resident, so every wait ends.
+// - The two state buffers alternate.  A tile overwrites a buffer only after its
+//   neighbours have finished the step that read it; they are all its readers, for the
+//   ring relation is symmetric.
 // What bounded the launches it replaces: a small mesh paid the gap between two
-// dependent kernels (about 2 us) and the geometry set-up every step, and a step of
-// a few waves waited for its last, partly filled one (four 100x100 drops in FP64:
-// 364 tiles of 16x8 on 304 resident blocks, 132 -> 98.6 us per step).
+// dependent kernels (about 2 us) and the geometry set-up every step, and a step of a
+// few waves waited for its last, partly filled one (four 100x100 drops in FP64, 364
+// tiles of 16x8 on 304 resident blocks: 132 -> 99 us per step).
 template <typename T, int BX, int BY, int NT, int MINB, bool UNI, bool SEP, int MODE = MODE_STEP>
 __global__ void __launch_bounds__(NT, MINB) k_step(const InstDev *__restrict__ insts, const int4 *__restrict__ tiles,
                                                    const AxisRecT<T> *__restrict__ geo,
