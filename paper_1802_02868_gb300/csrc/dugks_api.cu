@@ -79,7 +79,7 @@ struct dugks_sim {
     int n_tiles_s[kNumKernelShapes] = {};
     int n_uni_s[kNumKernelShapes] = {};
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t graph2 = nullptr;   // k_step(A -> B), k_step(B -> A)
+    cudaGraphExec_t graph2[kNumKernelShapes] = {};   // k_step(A -> B), k_step(B -> A), per kernel shape
     int *d_status = nullptr;      // per instance, then the error word of the many-step launches and the refused word
     // many-step launches, per kernel shape: progress counters, ring neighbours
     // (FLOW_NB per tile) and the value that every counter holds; built by the first
@@ -629,7 +629,7 @@ int build_graph2(dugks_sim *s)
     enqueue_fused<T>(s, b, s->cap_stream);
     e = cudaStreamEndCapture(s->cap_stream, &g);
     if (e != cudaSuccess) return cuda_status(e);
-    e = cudaGraphInstantiate(&s->graph2, g, 0);
+    e = cudaGraphInstantiate(&s->graph2[kernel_shape(s)], g, 0);
     cudaGraphDestroy(g);
     return cuda_status(e);
 }
@@ -825,13 +825,14 @@ int step_fused(dugks_sim *s, long n)
             if (rc) return rc;
             k++;
         }
-        if (!s->graph2) {
+        const cudaGraphExec_t &graph = s->graph2[kernel_shape(s)];
+        if (!graph) {
             int rc = build_graph2<T>(s);
             if (rc) return rc;
         }
         for (; k + 2 <= n; k += 2) {
             Timed t(s, K_STEP, 2, 2 * fused_launches(s));
-            cudaError_t e = cudaGraphLaunch(s->graph2, s->stream);
+            cudaError_t e = cudaGraphLaunch(graph, s->stream);
             if (e != cudaSuccess) return cuda_status(e);
         }
     }
@@ -1011,6 +1012,14 @@ void assign_planes(dugks_sim *s, Planes<T> &P, T *base)
 
 constexpr int kNumScalarPlanes = 12;
 
+void drop_graphs(dugks_sim *s)
+{
+    for (cudaGraphExec_t &g : s->graph2) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 void free_sim(dugks_sim *s)
 {
     if (!s) return;
@@ -1042,7 +1051,7 @@ void free_sim(dugks_sim *s)
     dfree(s, s->d_init_in);
     dfree(s, s->d_diag_parts);
     dfree(s, s->d_diag_out);
-    if (s->graph2) cudaGraphExecDestroy(s->graph2);
+    drop_graphs(s);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     for (auto &e : s->ev_used) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
     for (auto e : s->ev_pool) cudaEventDestroy(e);
@@ -1906,17 +1915,6 @@ int tile_for_running(const dugks_sim *s, const std::vector<char> &paused)
     return !s->fused || nx.empty() ? s->tile0 : tile_for_sizes(nx.data(), ny.data(), (int)nx.size(), s->prec, s->n_sm);
 }
 
-// change the tile of shape 0 (with no step in flight: the two-step graph holds it)
-void set_tile0(dugks_sim *s, int k)
-{
-    if (k == s->tile0) return;
-    if (s->graph2 && s->shape == 0) {
-        cudaGraphExecDestroy(s->graph2);
-        s->graph2 = nullptr;
-    }
-    s->tile0 = k;
-}
-
 int read_paused(dugks_sim *s, std::vector<char> &paused)
 {
     cudaError_t e = cudaStreamSynchronize(s->stream);
@@ -1958,13 +1956,13 @@ int dugks_batch_step_each(dugks_sim *s, const long *nsteps)
         rc = rewrite_paused(s, p);
         // shape 0 runs on the tile for the instances that still move: four 100x100
         // drops in FP64 take 16x8 tiles, the last of them alone 8x4 (51 and 41 us per step)
-        if (rc == DUGKS_OK && T - done >= FLOW_MIN) set_tile0(s, tile_for_running(s, p));
+        if (rc == DUGKS_OK && T - done >= FLOW_MIN) s->tile0 = tile_for_running(s, p);
         if (rc == DUGKS_OK) rc = dugks_step(s, T - done);
         if (rc) break;
         done = T;
     }
     const int rc2 = rewrite_paused(s, orig);   // synchronises
-    set_tile0(s, tile0);
+    s->tile0 = tile0;
     return rc ? rc : rc2;
 }
 
@@ -2079,10 +2077,7 @@ int dugks_set_tile_shape(dugks_sim *s, int shape)
     if (shape != s->shape) {
         cudaError_t e = cudaStreamSynchronize(s->stream);
         if (e != cudaSuccess) return cuda_status(e);
-        if (s->graph2) {
-            cudaGraphExecDestroy(s->graph2);
-            s->graph2 = nullptr;
-        }
+        drop_graphs(s);
         s->shape = shape;
         const int rc = wait_error(s);
         if (rc) return rc;

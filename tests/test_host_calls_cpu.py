@@ -202,3 +202,17 @@ def test_autotune_sets_up_before_it_times(rec, steps):
             assert timed and all(op.startswith(("kernel", "cooperative", "graph")) for op in timed), timed
             assert {op for op in timed if op != "graph"} <= {c[0] for c in calls[:a]}
         assert any(c[0].startswith("cooperative") for c in calls) == (steps >= 16)
+
+
+def test_segments_on_another_tile_keep_the_usual_tiles_graph(rec):
+    """Per-instance step counts may run a segment on another tile; the two-step graph of
+    short calls is not captured again after each."""
+    s, phi = _drops(rec, (100, 100, 100, 100), dugks.FP64)
+    with s:
+        s.init(phi)
+        s.step(4)
+        for _ in range(2):
+            s.step_each([20, 20, 20, 60])               # the last segment: one instance, smaller tiles
+            calls = rec.calls(lambda: s.step(4))
+            assert any(c[0] == "graph" for c in calls)
+            assert not any(c[0] == "begin capture" for c in calls)
