@@ -1883,11 +1883,11 @@ int dugks_batch_status(dugks_sim *s, int *per_instance_status)
     if (!s || !per_instance_status) return DUGKS_ERR_ARG;
     cudaError_t e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
-    std::vector<int> st(s->n_inst);
-    e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
+    std::vector<int> st(s->n_inst + 1);   // and the error word
+    e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * st.size(), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     for (int k = 0; k < s->n_inst; k++) per_instance_status[k] = (st[k] & ST_NONFINITE) ? DUGKS_ERR_NONFINITE : DUGKS_OK;
-    return wait_error(s);
+    return st.back() ? DUGKS_ERR_TIMEOUT : DUGKS_OK;
 }
 
 namespace {
@@ -1895,12 +1895,12 @@ namespace {
 int rewrite_paused(dugks_sim *s, const std::vector<char> &paused)
 {
     cudaError_t e = cudaStreamSynchronize(s->stream);
-    std::vector<int> st(s->n_inst);
-    if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
+    std::vector<int> st(s->n_inst + 1);   // and the error word
+    if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * st.size(), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     for (int k = 0; k < s->n_inst; k++) st[k] = (st[k] & ~ST_PAUSED) | (paused[k] ? ST_PAUSED : 0);
     e = upload(s, s->d_status, st.data(), sizeof(int) * s->n_inst);
-    return e != cudaSuccess ? cuda_status(e) : wait_error(s);
+    return e != cudaSuccess ? cuda_status(e) : st.back() ? DUGKS_ERR_TIMEOUT : DUGKS_OK;
 }
 
 // the tile of shape 0 for the instances that are not paused
@@ -1918,12 +1918,12 @@ int tile_for_running(const dugks_sim *s, const std::vector<char> &paused)
 int read_paused(dugks_sim *s, std::vector<char> &paused)
 {
     cudaError_t e = cudaStreamSynchronize(s->stream);
-    std::vector<int> st(s->n_inst);
-    if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * s->n_inst, cudaMemcpyDeviceToHost);
+    std::vector<int> st(s->n_inst + 1);   // and the error word
+    if (e == cudaSuccess) e = cudaMemcpy(st.data(), s->d_status, sizeof(int) * st.size(), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_status(e);
     paused.resize(s->n_inst);
     for (int k = 0; k < s->n_inst; k++) paused[k] = (st[k] & ST_PAUSED) ? 1 : 0;
-    return wait_error(s);
+    return st.back() ? DUGKS_ERR_TIMEOUT : DUGKS_OK;
 }
 }  // namespace
 
