@@ -1534,7 +1534,9 @@ int dugks_batch_create(int n, const dugks_mesh *meshes, const dugks_params *para
         const char *u = std::getenv("DUGKS_GENERAL_ONLY");
         s->use_uni = !(u && u[0] == '1');
         const char *w = std::getenv("DUGKS_WAIT_POLLS");
-        if (w && w[0]) s->wait_polls = (unsigned)std::strtoul(w, nullptr, 10);
+        char *end = nullptr;
+        const unsigned long polls = w ? std::strtoul(w, &end, 10) : 0;
+        if (w && end != w && !*end && polls < 1ul << 31) s->wait_polls = (unsigned)polls;
     }
     s->stream = (cudaStream_t)cuda_stream;
     s->alloc_fn = g_alloc_fn;
